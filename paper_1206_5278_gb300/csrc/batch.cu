@@ -25,7 +25,7 @@
 
 #include "cde_internal.h"
 #include "loo_common.cuh"
-#include "loo_mma.cuh"
+#include "loo_pack.cuh"
 
 namespace cde {
 
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256, 2) k_loo_batch(const LooArgs* __restrict_
             __syncthreads();
         }
         const CoefSmem cf{A.a1, A.a2};
-        loo_tile_mma<G1, G2, KERN>(A, cf, work[w].y, reinterpret_cast<float*>(sm4));
+        LooBody<G1, G2>::template tile<KERN>(A, cf, work[w].y, reinterpret_cast<float*>(sm4));
     }
 }
 
@@ -91,7 +91,7 @@ __global__ void k_loo_final_batch(const LooArgs* __restrict__ items, const int* 
 template <int G1, int G2, int KERN>
 static int launch_batch_shape_k(const LooArgs* d_items, const int2* d_work, int n_work, int* counter,
                                 int grid, cudaStream_t st, int dmax) {
-    using C = MmaCfg<G1, G2>;
+    using C = typename LooBody<G1, G2>::Cfg;
     static std::atomic<uint64_t> attr{0};
     CDE_CUDA(smem_attr_once(attr, k_loo_batch<G1, G2, KERN>, (int)C::smem_bytes(kMaxD)));
     k_loo_batch<G1, G2, KERN><<<grid, C::kThreads, C::smem_bytes(dmax), st>>>(d_items, d_work, n_work, counter);
@@ -116,6 +116,7 @@ static int launch_batch(int T1, int T2, int kern, const LooArgs* d_items, const 
                         int* counter, int grid, cudaStream_t st, int dmax) {
 #define CDE_BSHAPE(A, B) \
     if (T1 == A && T2 == B) return launch_batch_shape<A, B>(kern, d_items, d_work, n_work, counter, grid, st, dmax);
+    CDE_BSHAPE(4, 4) CDE_BSHAPE(4, 8) CDE_BSHAPE(8, 4) CDE_BSHAPE(8, 8)
     CDE_BSHAPE(16, 8) CDE_BSHAPE(16, 16) CDE_BSHAPE(16, 32)
     CDE_BSHAPE(32, 8) CDE_BSHAPE(32, 16) CDE_BSHAPE(32, 32)
 #undef CDE_BSHAPE
@@ -167,12 +168,13 @@ static int build_plan(cde_ctx* ctx, const std::vector<BatchItem>& items, BatchPl
     int dmax = 1;
     for (int b = 0; b < n; ++b) {
         const BatchItem& it = items[b];
-        const int T1 = loo_pad1(it.G1), T2 = loo_pad2(it.G2);
+        int T1, T2;
+        loo_shape(*it.D, it.G1, it.G2, true, T1, T2);   // no member takes the d >= 16 kernel here
         shape[b] = it.D->kernel * 4096 + T1 * 64 + T2;
         LooArgs& a = args[b];
         memset(&a, 0, sizeof(a));
         fill_loo_args(a, *it.D, it.h1, it.G1, it.h2, it.G2, T1, T2);
-        const int JW = 1024 / (T1 * T2);
+        const int JW = loo_unit_rows(T1, T2);
         a.rows = nullptr;
         a.n_rows = it.D->N;
         a.n_units = (int)((it.D->N + JW - 1) / JW);

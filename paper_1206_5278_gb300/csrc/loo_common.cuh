@@ -201,7 +201,7 @@ constexpr float kFbEx2Fix = 7.39e-8f;
 template <class C, class Coef>
 __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, float* sm, int nfl) {
     constexpr int GG = C::GG, G2 = C::G2v, JW = C::JW, NT = C::kThreads, NW = C::kWarps;
-    constexpr int LG2 = G2 == 8 ? 3 : (G2 == 16 ? 4 : 5);
+    constexpr int LG2 = G2 == 4 ? 2 : G2 == 8 ? 3 : (G2 == 16 ? 4 : 5);
     constexpr int JG = JW * GG;
     static_assert(8 * JG <= C::COMB, "fallback scratch must fit in the combine buffer");
     static_assert(JW <= 8, "per-row fallback parameters hold 8 rows");
@@ -435,8 +435,9 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
 // cells, rows in order; `first`: the tile's first unit, which stores instead).
 template <class C, int KERN, class Coef>
 __device__ __forceinline__ void loo_unit_epilogue(const LooArgs& a, const Coef& cf, float* sm, int u,
-                                                  bool first, int tile, const float (&At)[4]) {
-    constexpr int JW = C::JW, GG = C::GG, G1 = C::G1v, G2 = C::G2v;
+                                                  bool first, int tile,
+                                                  const float (&At)[(C::JW * C::GG + 255) / 256]) {
+    constexpr int JW = C::JW, GG = C::GG, G1 = C::G1v, G2 = C::G2v, CELLS = JW * GG;
     constexpr double LN2 = 0.69314718055994530942;
     const int tid = threadIdx.x;
     const int d = a.d;
@@ -450,8 +451,9 @@ __device__ __forceinline__ void loo_unit_epilogue(const LooArgs& a, const Coef& 
         // ---- shifted log numerators; flag cells that lost range ----
         double* la2 = reinterpret_cast<double*>(big);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
+        for (int m = 0; m < (CELLS + 255) / 256; ++m) {
             const int c = tid + 256 * m;
+            if (CELLS % 256 != 0 && c >= CELLS) continue;
             const int jl = c / GG;
             if (!vr_s[jl]) continue;
             const float v = At[m];
@@ -474,50 +476,86 @@ __device__ __forceinline__ void loo_unit_epilogue(const LooArgs& a, const Coef& 
         }
         __syncthreads();
 
-        // ---- FP64 log-ratio; each thread owns whole grid cells (all rows of
-        //      the unit, in row order) and adds them to the tile partial ----
-        {
-            double* part = a.part + CDE_CK(tile, a.n_tiles, 106) * 2 * GG;
-            constexpr int NOWN = GG >= 256 ? GG / 256 : 1;
+        // ---- FP64 log-ratio: a row's terms of cell (k, l) ----
+        const auto terms = [&](int jl, int k, int l, double a1k, double a2l, double lam, double kap, double& ell,
+                               double& lnA) {
+            const double shy = a2l * (double)my_s[jl];
+            const double lA = la2[jl * GG + k * G2 + l];
+            // a zero numerator (Epanechnikov: empty support, also when
+            // the denominator is zero) is ell = -inf, never NaN
+            ell = lA == -INFINITY ? -INFINITY : LN2 * (lA - btl_s[jl * G1 + k] - shy) - kap;
+            lnA = LN2 * (lA - a1k * (double)mx_s[jl] - shy) - lam - kap;
+            if (a.ell_rows && k < a.G1r && l < a.G2r) {
+                const int64_t r = CDE_CK((int64_t)u * JW + jl, a.n_rows, 107);
+                a.ell_rows[r * a.ell_ld_row + (int64_t)k * a.ell_ld_k + l] = ell;
+            }
+        };
+        // each thread adds whole grid cells (the unit's rows in row order) to the tile partial
+        double* part = a.part + CDE_CK(tile, a.n_tiles, 106) * 2 * GG;
+        const auto add_cell = [&](int kl, double sc, double se) {
+            if (first) {
+                part[kl] = sc;
+                part[GG + kl] = se;
+            } else {
+                part[kl] += sc;
+                part[GG + kl] += se;
+            }
+        };
+        if constexpr (GG < 256) {
+            // fewer cells than threads: every thread forms terms (else GG of the 256 threads
+            // would form all JW rows' in turn), then the cells' owners add them in row order
+            double* ells = la2 + CELLS;
+            double* lnAs = ells + CELLS;
 #pragma unroll
-            for (int s = 0; s < NOWN; ++s) {
+            for (int m = 0; m < (CELLS + 255) / 256; ++m) {
+                const int c = tid + 256 * m;
+                if (CELLS % 256 != 0 && c >= CELLS) continue;
+                const int jl = c / GG, kl = c - jl * GG, k = kl / G2, l = kl - k * G2;
+                double ell = 0.0, lnA = 0.0;
+                if (vr_s[jl]) terms(jl, k, l, (double)cf.a1(k), (double)cf.a2(l), a.lam1[k], a.kap2[l], ell, lnA);
+                ells[c] = ell;
+                lnAs[c] = lnA;
+            }
+            __syncthreads();
+            if (tid < GG) {
+                double sc = 0.0, se = 0.0;
+#pragma unroll
+                for (int jl = 0; jl < JW; ++jl) {   // rows past the last add an exact 0
+                    sc += ells[jl * GG + tid];
+                    se += lnAs[jl * GG + tid];
+                }
+                add_cell(tid, sc, se);
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < GG / 256; ++s) {
                 const int kl = tid + 256 * s;
-                if (kl >= GG) continue;
                 const int k = kl / G2, l = kl - k * G2;
                 const double a1k = (double)cf.a1(k), a2l = (double)cf.a2(l);
                 const double lam = a.lam1[k], kap = a.kap2[l];
                 double sc = 0.0, se = 0.0;
                 for (int jl = 0; jl < JW; ++jl) {
                     if (!vr_s[jl]) continue;
-                    const int c = jl * GG + kl;
-                    const double shy = a2l * (double)my_s[jl];
-                    const double lA = la2[c];
-                    // a zero numerator (Epanechnikov: empty support, also when
-                    // the denominator is zero) is ell = -inf, never NaN
-                    const double ell = lA == -INFINITY ? -INFINITY : LN2 * (lA - btl_s[jl * G1 + k] - shy) - kap;
-                    const double lnA = LN2 * (lA - a1k * (double)mx_s[jl] - shy) - lam - kap;
+                    double ell, lnA;
+                    terms(jl, k, l, a1k, a2l, lam, kap, ell, lnA);
                     sc += ell;
                     se += lnA;
-                    if (a.ell_rows && k < a.G1r && l < a.G2r) {
-                        const int64_t r = CDE_CK((int64_t)u * JW + jl, a.n_rows, 107);
-                        a.ell_rows[r * a.ell_ld_row + (int64_t)k * a.ell_ld_k + l] = ell;
-                    }
                 }
-                if (first) {
-                    part[kl] = sc;
-                    part[GG + kl] = se;
-                } else {
-                    part[kl] += sc;
-                    part[GG + kl] += se;
-                }
+                add_cell(kl, sc, se);
             }
         }
 }
 
 // Grid shapes of the tile kernels: k (h1) padded to an M-tile multiple of 16,
-// l (h2) to 8, 16 or 32.
+// l (h2) to 8, 16 or 32.  The autotuner's classes are these shapes.
 inline int loo_pad1(int g) { return g <= 16 ? 16 : 32; }
 inline int loo_pad2(int g) { return g <= 8 ? 8 : (g <= 16 ? 16 : 32); }
+// Grids of at most 8 x 8 on the direct kernel (d_x < 16, or `direct`) take the packed
+// body (loo_pack.cuh) with 4 or 8 bandwidths per axis, in the 16 x 8 body's place (and
+// in its tuning class: the units have the same 8 rows).
+void loo_shape(const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2);
+// rows per unit of a (direct) shape
+inline int loo_unit_rows(int T1, int T2) { return T1 < 16 ? 8 : 1024 / (T1 * T2); }
 
 int launch_loo_tile_kernel(int T1, int T2, const LooArgs& a, int grid, cudaStream_t st);
 // d_x >= 16: the kernel with the x cross-term on the tensor cores (loo_gram.cu)

@@ -36,7 +36,7 @@
 
 #include "cde_internal.h"
 #include "loo_common.cuh"
-#include "loo_mma.cuh"
+#include "loo_pack.cuh"
 
 namespace cde {
 
@@ -340,7 +340,7 @@ __global__ void k_loo_final(const double* __restrict__ part, int n_tiles, int GG
 // --------------------------------------------------------------------------
 template <int G1, int G2, int KERN>
 static int launch_shape_k(const LooArgs& a, int grid, cudaStream_t st) {
-    using C = MmaCfg<G1, G2>;
+    using C = typename LooBody<G1, G2>::Cfg;
     const size_t smem = C::smem_bytes(a.d);
     static std::atomic<uint64_t> attr{0};   // per instantiation
     CDE_CUDA(smem_attr_once(attr, k_loo_mma<G1, G2, KERN>, (int)C::smem_bytes(kMaxD)));
@@ -356,9 +356,19 @@ static int launch_shape(const LooArgs& a, int grid, cudaStream_t st) {
 }
 
 
+void loo_shape(const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2) {
+    T1 = loo_pad1(g1);
+    T2 = loo_pad2(g2);
+    if (g1 <= 8 && g2 <= 8 && (direct || !loo_use_gram(D, T1, T2))) {
+        T1 = g1 <= 4 ? 4 : 8;
+        T2 = g2 <= 4 ? 4 : 8;
+    }
+}
+
 int launch_loo_tile_kernel(int T1, int T2, const LooArgs& a, int grid, cudaStream_t st) {
 #define CDE_SHAPE(A, B) \
     if (T1 == A && T2 == B) return launch_shape<A, B>(a, grid, st);
+    CDE_SHAPE(4, 4) CDE_SHAPE(4, 8) CDE_SHAPE(8, 4) CDE_SHAPE(8, 8)
     CDE_SHAPE(16, 8) CDE_SHAPE(16, 16) CDE_SHAPE(16, 32)
     CDE_SHAPE(32, 8) CDE_SHAPE(32, 16) CDE_SHAPE(32, 32)
 #undef CDE_SHAPE
@@ -419,7 +429,9 @@ void fill_loo_args(LooArgs& a, const Dataset& D, const double* h1, int g1, const
     (void)T1; (void)T2;
 }
 
-static int shape_index(int T) { return T <= 8 ? 0 : T <= 16 ? 1 : 2; }
+// tuning class of a shape (the packed shapes are in the 16 x 8 class)
+static int class1(int T1) { return T1 <= 16 ? 1 : 2; }
+static int class2(int T2) { return T2 <= 8 ? 0 : T2 <= 16 ? 1 : 2; }
 
 // Units per tile: the autotuned value for this grid shape when the context has
 // one, else enough units for 8 rows per tile.  Both the single-dataset and the
@@ -430,8 +442,8 @@ static int shape_index(int T) { return T <= 8 ? 0 : T <= 16 ? 1 : 2; }
 static thread_local int t_cand_a = -1, t_cand_b = -1, t_cand_upt = 0, t_cand_ctas = 0;
 
 void tuning_candidate(int T1, int T2, int units_per_tile, int ctas_per_sm) {
-    t_cand_a = shape_index(T1);
-    t_cand_b = shape_index(T2);
+    t_cand_a = class1(T1);
+    t_cand_b = class2(T2);
     t_cand_upt = units_per_tile;
     t_cand_ctas = ctas_per_sm;
 }
@@ -439,13 +451,13 @@ void tuning_candidate(int T1, int T2, int units_per_tile, int ctas_per_sm) {
 void tuning_candidate_clear() { t_cand_a = t_cand_b = -1; }
 
 static int tuned_upt(cde_ctx* ctx, int T1, int T2) {
-    const int a = shape_index(T1), b = shape_index(T2);
+    const int a = class1(T1), b = class2(T2);
     if (a == t_cand_a && b == t_cand_b) return t_cand_upt;
     return ctx ? ctx->tune_upt[a][b] : 0;
 }
 
 static int tuned_ctas(cde_ctx* ctx, int T1, int T2) {
-    const int a = shape_index(T1), b = shape_index(T2);
+    const int a = class1(T1), b = class2(T2);
     if (a == t_cand_a && b == t_cand_b) return t_cand_ctas;
     return ctx ? ctx->tune_ctas[a][b] : 0;
 }
@@ -453,7 +465,7 @@ static int tuned_ctas(cde_ctx* ctx, int T1, int T2) {
 int loo_units_per_tile(cde_ctx* ctx, int T1, int T2, int64_t n_rows) {
     const int t = tuned_upt(ctx, T1, T2);
     if (t > 0) return t;
-    const int JW = 1024 / (T1 * T2);
+    const int JW = loo_unit_rows(T1, T2);
     int upt = JW >= 8 ? 1 : 8 / JW;
     // Smaller tiles while the grid would give fewer than 64 tiles per resident CTA: the
     // tiles come from an atomic queue, and the last CTAs to finish decide the launch's time.
@@ -485,8 +497,8 @@ struct LooPlan {
 
 static LooPlan loo_plan(cde_ctx* ctx, const Dataset& D, int T1, int T2, int64_t n_rows) {
     LooPlan p{};
-    p.gram = loo_use_gram(D, T1, T2);
-    p.rpu = p.gram ? loo_gram_rows_per_unit(T1, T2) : 1024 / (T1 * T2);
+    p.gram = T1 >= 16 && loo_use_gram(D, T1, T2);
+    p.rpu = p.gram ? loo_gram_rows_per_unit(T1, T2) : loo_unit_rows(T1, T2);
     p.upt = p.gram ? 1 : loo_units_per_tile(ctx, T1, T2, n_rows);
     p.n_units = (int)((n_rows + p.rpu - 1) / p.rpu);
     const int cmax = p.gram ? ctx->sm_count : loo_grid_ctas(ctx, T1, T2);
@@ -501,9 +513,9 @@ static LooPlan loo_plan(cde_ctx* ctx, const Dataset& D, int T1, int T2, int64_t 
 size_t loo_grid_scratch_bytes(cde_ctx* ctx, const Dataset& D, int G1, int G2, int64_t n_rows) {
     size_t mx = 0;
     for (int k0 = 0; k0 < G1; k0 += 32) {
-        const int T1 = loo_pad1(G1 - k0 < 32 ? G1 - k0 : 32);
         for (int l0 = 0; l0 < G2; l0 += 32) {
-            const int T2 = loo_pad2(G2 - l0 < 32 ? G2 - l0 : 32);
+            int T1, T2;
+            loo_shape(D, G1 - k0 < 32 ? G1 - k0 : 32, G2 - l0 < 32 ? G2 - l0 : 32, false, T1, T2);
             const size_t b = loo_plan(ctx, D, T1, T2, n_rows).bytes();
             if (b > mx) mx = b;
         }
@@ -518,10 +530,10 @@ int loo_grid_enqueue(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, c
     if (!d_rows) n_rows = D.N;
     for (int k0 = 0; k0 < G1; k0 += 32) {
         const int g1 = G1 - k0 < 32 ? G1 - k0 : 32;
-        const int T1 = loo_pad1(g1);
         for (int l0 = 0; l0 < G2; l0 += 32) {
             const int g2 = G2 - l0 < 32 ? G2 - l0 : 32;
-            const int T2 = loo_pad2(g2);
+            int T1, T2;
+            loo_shape(D, g1, g2, false, T1, T2);
             LooArgs a{};
             fill_loo_args(a, D, h1 + k0, g1, h2 + l0, g2, T1, T2);
             const LooPlan pl = loo_plan(ctx, D, T1, T2, n_rows);
@@ -592,8 +604,7 @@ int loo_chunked_create(cde_ctx* ctx, const Dataset& D, const double* h1, int G1,
                        LooChunked** out) {
     if (G1 > 32 || G2 > 32) return set_error(CDE_EINVAL, "loo_chunked_create: one grid block (<= 32 x 32) only");
     auto* c = new LooChunked{};
-    c->T1 = loo_pad1(G1);
-    c->T2 = loo_pad2(G2);
+    loo_shape(D, G1, G2, false, c->T1, c->T2);
     c->G1 = G1;
     c->G2 = G2;
     LooArgs& a = c->a;
@@ -640,7 +651,7 @@ int loo_chunked_next(LooChunked* c, void* scratch, double pair_evals, cudaStream
     a.part = static_cast<double*>(scratch);
     a.fb = reinterpret_cast<double*>(static_cast<char*>(scratch) + c->part_bytes);
     a.work = reinterpret_cast<int*>(static_cast<char*>(scratch) + c->part_bytes + c->fb_bytes);
-    const double rows_per_unit = c->gram ? loo_gram_rows_per_unit(c->T1, c->T2) : 1024.0 / (c->T1 * c->T2);
+    const double rows_per_unit = c->gram ? loo_gram_rows_per_unit(c->T1, c->T2) : loo_unit_rows(c->T1, c->T2);
     const double per_unit = rows_per_unit * (double)c->N * c->T1 * c->T2;
     const int G = a.big_g, L = a.big_levels;
     int t0, t1, grid;

@@ -480,18 +480,4 @@ __device__ __forceinline__ void loo_tile_mma(const LooArgs& a, const Coef& cf, i
     }
 }
 
-template <int G1, int G2, int KERN>
-__global__ void __launch_bounds__(256, 2) k_loo_mma(const LooArgs a) {
-    extern __shared__ float4 sm4[];
-    __shared__ int next_tile;
-    const CoefParam cf{a};
-    for (int t0 = blockIdx.x;; t0 += gridDim.x) {
-        if (threadIdx.x == 0) next_tile = a.work ? atomicAdd(a.work, 1) : t0;
-        __syncthreads();
-        const int t = next_tile;
-        if (t >= a.n_tiles) break;
-        loo_tile_mma<G1, G2, KERN>(a, cf, t, reinterpret_cast<float*>(sm4));
-    }
-}
-
 }  // namespace cde

@@ -72,10 +72,11 @@ extern "C" int cde_loo_loglik_noalloc(cde_ctx* ctx, cde_dataset ds, const double
     if (rc != CDE_OK) return rc;
     cudaStream_t st = pick_stream(ctx, stream);
 
-    const int T1 = loo_pad1(G1), T2 = loo_pad2(G2);
+    int T1, T2;
+    loo_shape(*D, G1, G2, true, T1, T2);   // the direct kernel at every d_x
     LooArgs a{};
     fill_loo_args(a, *D, h1, G1, h2, G2, T1, T2);
-    const int JW = 1024 / (T1 * T2);
+    const int JW = loo_unit_rows(T1, T2);
     a.rows = nullptr;
     a.n_rows = D->N;
     a.n_units = (int)((D->N + JW - 1) / JW);
