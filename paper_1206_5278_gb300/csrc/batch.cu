@@ -371,7 +371,8 @@ int autotune_shape(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, con
                    int* best_upt, int* best_ctas, double* best_ms) {
     const int T1 = loo_pad1(G1), T2 = loo_pad2(G2);
     const int a = shape_class(T1), b = shape_class(T2);
-    const int JW = 1024 / (T1 * T2);
+    const int JW = 1024 / (T1 * T2);   // (the packed shapes' units have the 16 x 8 shape's 8 rows)
+    const int64_t n_units = (D.N + JW - 1) / JW;
     std::vector<int> upts;
     for (int u : {1, 2, 4, 8, 16})
         if (u * JW >= 2 && u * JW <= 64) upts.push_back(u);
@@ -391,6 +392,10 @@ int autotune_shape(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, con
     std::vector<Cand> timed;
     for (int u : upts)
             for (int c : {1, 2}) {
+                // larger tiles than the smallest only while they still fill the resident CTAs:
+                // on fewer tiles they can only lose, and the launch is then so short (10-20 us)
+                // that the timings would choose at random
+                if (u != upts[0] && (n_units + u - 1) / u < (int64_t)c * ctx->sm_count) continue;
                 tuning_candidate(T1, T2, u, c);
                 // one untimed launch, then the fastest of three
                 float tmin = 1e30f;
