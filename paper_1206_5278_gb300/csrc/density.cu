@@ -34,6 +34,7 @@
 #include <cstdint>
 
 #include "cde_internal.h"
+#include "dist_tile.cuh"
 #include "tc_util.cuh"
 
 namespace cde {
@@ -64,40 +65,55 @@ __global__ void k_query_pack(const float* __restrict__ xq, int64_t Q, int64_t Qp
 // main kernel).  The data range is split over gridDim.y; split minima are
 // merged with an integer atomicMin on the float bits (exact and order-free:
 // squared distances are non-negative, so their bit patterns order like ints).
-__global__ void __launch_bounds__(256) k_query_shift(const float* __restrict__ xs, int64_t N,
-                                                     int64_t Np, int d, const float* __restrict__ xq,
-                                                     int64_t Q, int64_t Qp, int64_t i_per_split,
-                                                     unsigned int* __restrict__ mq_bits) {
-    extern __shared__ float sm[];  // [d][256]
-    const int64_t q = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int64_t ib = (int64_t)blockIdx.y * i_per_split;
-    const int64_t ie = min(N, ib + i_per_split);
-    float xqr[8];
+// d > 8: the distance tiles of dist_tile.cuh, 128 queries per CTA.
+__global__ void __launch_bounds__(kDtThreads, 2) k_query_shift_tile(const float* __restrict__ xs, int64_t N,
+                                                                     int64_t Np, int d, const float* __restrict__ xq,
+                                                                     int64_t Q, int64_t Qp, int64_t i_per_split,
+                                                                     unsigned int* __restrict__ mq_bits) {
+    extern __shared__ float4 dt4[];
+    float* rows = reinterpret_cast<float*>(dt4);
+    float* pbuf = rows + d * kDtRows;
+    const int nbuf = d * kDtPts;
+    const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 4, pg = tid & 15;
+    const int64_t r0 = (int64_t)blockIdx.x * kDtRows;
+    const int64_t i0 = (int64_t)blockIdx.y * i_per_split, i1 = min(N, i0 + i_per_split);
+    dt_fetch(xs, nullptr, Np, d, i0, pbuf);
+    for (int e = tid; e < d * kDtRows; e += kDtThreads)   // r0 + 127 < Qp (a multiple of 128)
+        rows[e] = xq[(int64_t)(e / kDtRows) * Qp + CDE_CK(r0 + e % kDtRows, Qp, 201)];
+    float best[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) xqr[c] = (q < Qp && c < d) ? xq[(int64_t)c * Qp + q] : 0.f;
-    float best = INFINITY;
-    for (int64_t i0 = ib; i0 < ie; i0 += 256) {
+    for (int r = 0; r < 8; ++r) best[r] = INFINITY;
+    int b = 0;
+    for (int64_t t0 = i0; t0 < i1; t0 += kDtPts, b ^= 1) {
+        float* pts = pbuf + b * nbuf;
         __syncthreads();
-        for (int c = 0; c < d; ++c) sm[c * 256 + threadIdx.x] = xs[(int64_t)c * Np + i0 + threadIdx.x];
+        if (t0 + kDtPts < i1) dt_fetch(xs, nullptr, Np, d, t0 + kDtPts, pbuf + (b ^ 1) * nbuf);
+        else cp_async_commit();
+        cp_async_wait_1();
         __syncthreads();
-        const int n = (int)min((int64_t)256, ie - i0);
-        if (q < Q)
-            for (int tt = 0; tt < n; ++tt) {
-                float dx2 = 0.f;
+        if (t0 + kDtPts > i1) {
+            const int n = (int)(i1 - t0);
+            for (int e = tid; e < nbuf; e += kDtThreads)
+                if (e % kDtPts >= n) pts[e] = INFINITY;
+            __syncthreads();
+        }
+        float2 acc[4][4];
+        dt_distances(rows, pts, d, rg, pg, acc);
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c < d) {
-                        const float u = xqr[c] - sm[c * 256 + tt];
-                        dx2 = fmaf(u, u, dx2);
-                    }
-                for (int c = 8; c < d; ++c) {
-                    const float u = xq[(int64_t)c * Qp + q] - sm[c * 256 + tt];
-                    dx2 = fmaf(u, u, dx2);
-                }
-                best = fminf(best, dx2);
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                best[2 * q] = fminf(best[2 * q], acc[q][e].x);
+                best[2 * q + 1] = fminf(best[2 * q + 1], acc[q][e].y);
             }
     }
-    if (q < Q) atomicMin(mq_bits + q, __float_as_uint(best));
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) best[r] = fminf(best[r], __shfl_xor_sync(0xffffffffu, best[r], o));
+        const int64_t q = r0 + 8 * rg + r;
+        if ((lane & 15) == 0 && q < Q) atomicMin(mq_bits + q, __float_as_uint(best[r]));
+    }
 }
 
 // d <= 8: the same minima with JB queries per thread (two per packed FP32x2
@@ -196,17 +212,13 @@ int query_shift_enqueue(int sm_count, const Dataset& D, const float* xq, int64_t
         CDE_CUDA(cudaGetLastError());
         return CDE_OK;
     }
-    const size_t sm = (size_t)D.d * 256 * sizeof(float);
-    if (sm > 48 * 1024)
-        CDE_CUDA(cudaFuncSetAttribute(k_query_shift, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const int64_t qb = (Q + 255) / 256;
-    const int64_t tiles = (D.N + 255) / 256;
-    int64_t sy = (4LL * sm_count + qb - 1) / qb;
-    if (sy > tiles) sy = tiles;
-    if (sy < 1) sy = 1;
-    const int64_t tps = (tiles + sy - 1) / sy;
-    sy = (tiles + tps - 1) / tps;
-    k_query_shift<<<dim3((unsigned)qb, (unsigned)sy), 256, sm, st>>>(D.xs, D.N, D.Np, D.d, xq, Q, Qp, tps * 256, mqb);
+    const int64_t qb = (Q + kDtRows - 1) / kDtRows;
+    int64_t ns = 1;
+    const int64_t ips = dt_points_per_split(qb, D.N, sm_count, &ns);
+    static std::atomic<uint64_t> attr{0};
+    CDE_CUDA(smem_attr_once(attr, k_query_shift_tile, dt_smem_floats(kMaxD, false) * (int)sizeof(float)));
+    k_query_shift_tile<<<dim3((unsigned)qb, (unsigned)ns), kDtThreads, dt_smem_floats(D.d, false) * sizeof(float), st>>>(
+        D.xs, D.N, D.Np, D.d, xq, Q, Qp, ips, mqb);
     CDE_CUDA(cudaGetLastError());
     return CDE_OK;
 }

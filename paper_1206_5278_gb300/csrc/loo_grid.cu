@@ -35,6 +35,7 @@
 #include <cstdio>
 
 #include "cde_internal.h"
+#include "dist_tile.cuh"
 #include "loo_common.cuh"
 #include "loo_pack.cuh"
 
@@ -116,67 +117,6 @@ int pack_enqueue(Dataset& D, const float* d_x, const float* d_y, cudaStream_t st
 // (it can be no worse than either neighbour), which is what the exact
 // fallback of the grid kernels uses to skip points.
 // --------------------------------------------------------------------------
-
-// (a, b) < (c, d) lexicographically
-__device__ __forceinline__ bool lex_less(float a, float b, float c, float d) {
-    return a < c || (a == c && b < d);
-}
-
-__global__ void __launch_bounds__(256) k_nn_shift(const float* __restrict__ xs,
-                                                  const float* __restrict__ y, int64_t N,
-                                                  int64_t Np, int d, float* __restrict__ mx,
-                                                  float* __restrict__ my, float* __restrict__ qx,
-                                                  float* __restrict__ qy) {
-    extern __shared__ float sm[];  // [d + 1][256]
-    const int64_t j = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const bool vj = j < N;
-    float xj[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) xj[c] = (vj && c < d) ? xs[(int64_t)c * Np + j] : 0.f;
-    const float yj = vj ? y[j] : 0.f;
-    float bx = INFINITY, by = INFINITY, ax = INFINITY, ay = INFINITY;
-    for (int64_t i0 = 0; i0 < N; i0 += 256) {
-        __syncthreads();
-        for (int c = 0; c <= d; ++c) {
-            const float* src = c < d ? xs + (int64_t)c * Np : y;
-            sm[c * 256 + threadIdx.x] = src[i0 + threadIdx.x];  // i0+tid < Np
-        }
-        __syncthreads();
-        const int n = (int)min((int64_t)256, N - i0);
-        for (int t = 0; t < n; ++t) {
-            const int64_t i = i0 + t;
-            float dx2 = 0.f;
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < d) {
-                    float u = xj[c] - sm[c * 256 + t];
-                    dx2 = fmaf(u, u, dx2);
-                }
-            for (int c = 8; c < d; ++c) {
-                float u = xs[(int64_t)c * Np + j * vj] - sm[c * 256 + t];
-                dx2 = fmaf(u, u, dx2);
-            }
-            const float dy = yj - sm[d * 256 + t];
-            const float dy2 = dy * dy;
-            if (i != j) {
-                if (lex_less(dx2, dy2, bx, ax)) {
-                    bx = dx2;
-                    ax = dy2;
-                }
-                if (lex_less(dy2, dx2, by, ay)) {
-                    by = dy2;
-                    ay = dx2;
-                }
-            }
-        }
-    }
-    if (vj) {
-        mx[j] = bx;
-        my[j] = by;
-        qy[j] = ax;
-        qx[j] = ay;
-    }
-}
 
 // d <= 8: four rows per thread, point-major shared tiles (128-bit loads), the
 // data range split over gridDim.y; split minima merge with a 64-bit integer
@@ -271,6 +211,90 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_shift_split(const float* __re
     }
 }
 
+// d > 8: the distance tiles of dist_tile.cuh, with the same keys and merge.  Eight rows
+// per thread hold 16 running keys; points past N are made infinitely far in shared
+// memory, and only the tiles that meet the CTA's own rows test i != j.
+__global__ void __launch_bounds__(kDtThreads, 2) k_nn_shift_tile(const float* __restrict__ xs,
+                                                                  const float* __restrict__ y, int64_t N, int64_t Np,
+                                                                  int d, int64_t i_per_split,
+                                                                  unsigned long long* __restrict__ kx,
+                                                                  unsigned long long* __restrict__ ky) {
+    extern __shared__ float4 dt4[];
+    float* rows = reinterpret_cast<float*>(dt4);
+    float* pbuf = rows + d * kDtRows;
+    const int nbuf = (d + 1) * kDtPts;
+    const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 4, pg = tid & 15;
+    const int64_t r0 = (int64_t)blockIdx.x * kDtRows;
+    const int64_t i0 = (int64_t)blockIdx.y * i_per_split, i1 = min(N, i0 + i_per_split);
+    dt_fetch(xs, y, Np, d, i0, pbuf);
+    for (int e = tid; e < d * kDtRows; e += kDtThreads) {
+        const int c = e / kDtRows, r = e % kDtRows;
+        rows[e] = xs[(int64_t)c * Np + (r0 + r < N ? r0 + r : 0)];
+    }
+    float2 yr[4];
+    unsigned long long mkx[8], mky[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t ja = r0 + 8 * rg + 2 * q;
+        yr[q] = make_float2(y[ja < N ? ja : 0], y[ja + 1 < N ? ja + 1 : 0]);
+        mkx[2 * q] = mkx[2 * q + 1] = mky[2 * q] = mky[2 * q + 1] = nn_key(INFINITY, INFINITY);
+    }
+    int b = 0;
+    for (int64_t t0 = i0; t0 < i1; t0 += kDtPts, b ^= 1) {
+        float* pts = pbuf + b * nbuf;
+        __syncthreads();   // the other buffer's readers are done
+        if (t0 + kDtPts < i1) dt_fetch(xs, y, Np, d, t0 + kDtPts, pbuf + (b ^ 1) * nbuf);
+        else cp_async_commit();
+        cp_async_wait_1();
+        __syncthreads();
+        if (t0 + kDtPts > i1) {   // the split's last, partial tile
+            const int n = (int)(i1 - t0);
+            for (int e = tid; e < nbuf; e += kDtThreads)
+                if (e % kDtPts >= n) pts[e] = INFINITY;
+            __syncthreads();
+        }
+        float2 acc[4][4];
+        dt_distances(rows, pts, d, rg, pg, acc);
+        const float4 y4 = *reinterpret_cast<const float4*>(pts + d * kDtPts + 4 * pg);
+        const float py[4] = {-y4.x, -y4.y, -y4.z, -y4.w};
+        const int off = (int)(t0 - r0) + 4 * pg - 8 * rg;   // point e is row 2q + h iff off + e == 2q + h
+        const bool own = t0 < r0 + kDtRows && t0 + kDtPts > r0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 dy = __fadd2_rn(yr[q], make_float2(py[e], py[e]));
+                const float2 dy2 = __fmul2_rn(dy, dy);
+                float2 dx2 = acc[q][e];
+                float2 dyk = dy2;
+                if (own) {   // the left-out point never counts
+                    if (off + e == 2 * q) dx2.x = dyk.x = INFINITY;
+                    if (off + e == 2 * q + 1) dx2.y = dyk.y = INFINITY;
+                }
+                const unsigned long long x0 = nn_key(dx2.x, dyk.x), x1 = nn_key(dx2.y, dyk.y);
+                const unsigned long long y0 = nn_key(dyk.x, dx2.x), y1 = nn_key(dyk.y, dx2.y);
+                if (x0 < mkx[2 * q]) mkx[2 * q] = x0;
+                if (x1 < mkx[2 * q + 1]) mkx[2 * q + 1] = x1;
+                if (y0 < mky[2 * q]) mky[2 * q] = y0;
+                if (y1 < mky[2 * q + 1]) mky[2 * q + 1] = y1;
+            }
+    }
+    // the 16 threads of a row group are half a warp
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            mkx[r] = min(mkx[r], __shfl_xor_sync(0xffffffffu, mkx[r], o));
+            mky[r] = min(mky[r], __shfl_xor_sync(0xffffffffu, mky[r], o));
+        }
+        const int64_t j = r0 + 8 * rg + r;
+        if ((lane & 15) == 0 && j < N) {
+            atomicMin(kx + j, mkx[r]);
+            atomicMin(ky + j, mky[r]);
+        }
+    }
+}
+
 // unpack the merged (minimum, other distance) keys
 __global__ void k_nn_unpack(const unsigned long long* __restrict__ kx, const unsigned long long* __restrict__ ky,
                             int64_t N, float* __restrict__ mx, float* __restrict__ my, float* __restrict__ qx,
@@ -285,6 +309,11 @@ __global__ void k_nn_unpack(const unsigned long long* __restrict__ kx, const uns
 }
 
 int nn_shift_enqueue(const Dataset& D, cudaStream_t st, int sm_count) {
+    unsigned long long* keys = nullptr;   // [2][N] merge keys, stream-ordered scratch
+    CDE_CUDA(cudaMallocAsync((void**)&keys, (size_t)2 * D.N * sizeof(unsigned long long), st));
+    // d <= 8: 0x7f bytes, the first word 3.4e38; d > 8: 0xff bytes, above infinity (a row
+    // whose every distance overflows keeps an infinite shift)
+    CDE_CUDA(cudaMemsetAsync(keys, D.d <= 8 ? 0x7f : 0xff, (size_t)2 * D.N * sizeof(unsigned long long), st));
     if (D.d <= 8) {
         const int64_t per_cta = (int64_t)kNnThreads * kNnJB;
         const int64_t gx = (D.N + per_cta - 1) / per_cta;
@@ -294,28 +323,24 @@ int nn_shift_enqueue(const Dataset& D, cudaStream_t st, int sm_count) {
         if (ns < 1) ns = 1;
         const int64_t tps = (tiles + ns - 1) / ns;
         ns = (tiles + tps - 1) / tps;
-        unsigned long long* keys = nullptr;   // [2][N] merge keys, stream-ordered scratch
-        CDE_CUDA(cudaMallocAsync((void**)&keys, (size_t)2 * D.N * sizeof(unsigned long long), st));
-        // 0x7f bytes: the first word 3.4e38, above any distance
-        CDE_CUDA(cudaMemsetAsync(keys, 0x7f, (size_t)2 * D.N * sizeof(unsigned long long), st));
         const dim3 grid((unsigned)gx, (unsigned)ns);
         if (D.d <= 4)
             k_nn_shift_split<4><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, keys, keys + D.N);
         else
             k_nn_shift_split<8><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, keys, keys + D.N);
-        CDE_CUDA(cudaGetLastError());
-        k_nn_unpack<<<(unsigned)((D.N + 255) / 256), 256, 0, st>>>(keys, keys + D.N, D.N, D.mx, D.my, D.qx, D.qy);
-        CDE_CUDA(cudaGetLastError());
-        CDE_CUDA(cudaFreeAsync(keys, st));
-        return CDE_OK;
+    } else {
+        const int64_t gx = (D.N + kDtRows - 1) / kDtRows;
+        int64_t ns = 1;
+        const int64_t ips = dt_points_per_split(gx, D.N, sm_count, &ns);
+        static std::atomic<uint64_t> attr{0};
+        CDE_CUDA(smem_attr_once(attr, k_nn_shift_tile, dt_smem_floats(kMaxD, true) * (int)sizeof(float)));
+        k_nn_shift_tile<<<dim3((unsigned)gx, (unsigned)ns), kDtThreads, dt_smem_floats(D.d, true) * sizeof(float), st>>>(
+            D.xs, D.y, D.N, D.Np, D.d, ips, keys, keys + D.N);
     }
-    const int64_t blocks = (D.N + 255) / 256;
-    const size_t smem = (size_t)(D.d + 1) * 256 * sizeof(float);
-    if (smem > 48 * 1024)
-        CDE_CUDA(cudaFuncSetAttribute(k_nn_shift, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-    k_nn_shift<<<(unsigned)blocks, 256, smem, st>>>(D.xs, D.y, D.N, D.Np, D.d, D.mx, D.my, D.qx, D.qy);
     CDE_CUDA(cudaGetLastError());
+    k_nn_unpack<<<(unsigned)((D.N + 255) / 256), 256, 0, st>>>(keys, keys + D.N, D.N, D.mx, D.my, D.qx, D.qy);
+    CDE_CUDA(cudaGetLastError());
+    CDE_CUDA(cudaFreeAsync(keys, st));
     return CDE_OK;
 }
 
