@@ -173,7 +173,228 @@ struct CoefParam {
 constexpr float kFbEx2Fix = 7.39e-8f;
 
 // Exact joint-shift recomputation of the flagged cells of one unit (whole
-// CTA).  For a cell (row j, k, l) let X_i = dx2_i - m_x,j, Y_i = dy2_i - m_y,j and
+// CTA).  For a cell (row j, k, l) let e_i = a1_k (dx2_i - m_x,j) + a2_l (dy2_i - m_y,j).
+// Then At = sum_i 2^{-e_i} = 2^{-e_a} S with S = sum_i 2^{-(e_i - e_a)} for any anchor
+// point a, where e_i - e_a = a1_k (dx2_i - dx2_a) + a2_l (dy2_i - dy2_a) is formed from
+// differences of distances (no cancellation at large e), and log2 At = -e_a + log2 S
+// with e_a in FP64.  One pass over the points: every warp takes chunks of 64
+// consecutive points (two per lane, packed FP32x2 distances, the tile body's formula)
+// and keeps, per flagged cell, its own anchor -- the smallest e it has met -- and the
+// sum relative to it; a point below the anchor rescales the sum and becomes the anchor.
+// All anchors start at the better of the x-nearest and the y-nearest point (their
+// distances are stored with the dataset), so the warps' sums never overflow (terms are
+// at most 1), and the warps are merged in fixed order at the lowest anchor.
+//
+// Candidates.  A term with e_i > e_a + T, T = 32 + ceil(log2 N), adds less than 2^-T of
+// the cell's sum (all of them together less than 2^-32), so only points with
+// X <= max_f (e_af + T)/a1_f and Y <= max_f (e_af + T)/a2_f over the row's cells are
+// looked at; the box follows the warp's anchors down.  A row's candidates of a chunk
+// are compacted into the warp's list (lane = point), then lane = cell: each lane runs
+// its cells over the list.  Every warp's work is a fixed function of the row and the
+// points, so the result does not depend on scheduling.
+//
+// Bound by the distance pass (issue).  Tile kernel with this pass against the two-pass
+// form below, Gaussian, standardised six-component mixture: N = 12,000, d = 12: 4 x 4 0.88
+// against 1.75 ms, 16 x 8 1.72 / 2.61, 16 x 16 2.03 / 2.95, 32 x 16 2.95 / 4.05; N = 20,000,
+// d = 5: 4 x 4 1.20 / 1.42, 16 x 16 3.92 / 4.06, 32 x 16 6.20 / 6.24.
+template <class C, class Coef>
+__device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, float* sm, int nfl) {
+    constexpr int GG = C::GG, G2 = C::G2v, JW = C::JW, NT = C::kThreads, NW = C::kWarps;
+    constexpr int LG2 = G2 == 4 ? 2 : G2 == 8 ? 3 : (G2 == 16 ? 4 : 5);
+    constexpr int JG = JW * GG, CAP = C::FBCAP;
+    static_assert(JW <= 8, "per-row bounds hold 8 rows");
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int d = a.d;
+    const int64_t N = a.N, Np = a.Np;
+    const float* xj_s = sm + C::off_xj(d);
+    const float* yj_s = sm + C::off_yj(d);
+    const float* mx_s = sm + C::off_mx(d);
+    const float* my_s = sm + C::off_my(d);
+    const long long* ji_s = reinterpret_cast<const long long*>(sm + C::off_ji(d));
+    const int* flag_s = reinterpret_cast<const int*>(sm + C::off_flag(d));
+    double* la2 = reinterpret_cast<double*>(sm);
+    float* As = sm + 2 * JG;                       // the round's cells: coefficients
+    float* Bs = sm + 3 * JG;
+    float* Ss = sm + C::off_fbS(d);                // [warp][CAP] sums, then the anchors' dx2, dy2
+    float* Xs = sm + C::off_fbX(d);
+    float* Ys = Xs + NW * CAP;
+    // per warp: a chunk's candidates of one row, and the rows' boxes; then the row ranges
+    float* fbw = sm + C::off_fbw(d);
+    float* lx = fbw + warp * 144;
+    float* ly = lx + 64;
+    float* bx = ly + 64;
+    float* by = bx + 8;
+    int* rs = reinterpret_cast<int*>(fbw + NW * 144);   // cells [rs, re) of the row in the round
+    int* re = rs + 8;
+    float* Sw = Ss + warp * CAP;
+    float* Xw = Xs + warp * CAP;
+    float* Yw = Ys + warp * CAP;
+
+    int lg = 0;
+    while (((int64_t)1 << lg) < N) ++lg;
+    const float T = (float)(32 + lg);
+
+    // the warp's box of a row from its cells' anchors (all lanes return with it stored)
+    const auto box = [&](int r, int f0, int f1) {
+        const float mxr = mx_s[r], myr = my_s[r];
+        float x = 0.f, y = 0.f;
+        for (int f = f0 + lane; f < f1; f += 32) {
+            const float A = As[f], B = Bs[f];
+            // (the factor covers the rounding of e where it is large next to T)
+            const float e = fmaf(fmaf(A, Xw[f] - mxr, B * (Yw[f] - myr)), 1.f + 0x1p-20f, T);
+            x = fmaxf(x, __fdividef(e, A));
+            y = fmaxf(y, __fdividef(e, B));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+            y = fmaxf(y, __shfl_xor_sync(0xffffffffu, y, o));
+        }
+        __syncwarp();
+        if (lane == 0) {
+            bx[r] = mxr + x;
+            by[r] = myr + y;
+        }
+        __syncwarp();
+    };
+
+    for (int base = 0; base < nfl; base += CAP) {
+        const int n = min(CAP, nfl - base);
+        if (tid < JW) rs[tid] = re[tid] = 0;
+        __syncthreads();
+        for (int f = tid; f < n; f += NT) {
+            const int c = flag_s[base + f], r = c / GG, kl = c - r * GG, k = kl >> LG2, l = kl & (G2 - 1);
+            const float A = cf.a1(k), B = cf.a2(l);
+            As[f] = A;
+            Bs[f] = B;
+            if (f == 0 || flag_s[base + f - 1] / GG != r) rs[r] = f;
+            if (f == n - 1 || flag_s[base + f + 1] / GG != r) re[r] = f + 1;
+            // the x-nearest point is (m_x, q_y), the y-nearest (q_x, m_y)
+            const long long j = ji_s[r];
+            const float qx = a.qx[j], qy = a.qy[j];
+            const bool xn = B * (qy - my_s[r]) <= A * (qx - mx_s[r]);
+            const float X0 = xn ? mx_s[r] : qx, Y0 = xn ? qy : my_s[r];
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                Ss[w * CAP + f] = 0.f;
+                Xs[w * CAP + f] = X0;
+                Ys[w * CAP + f] = Y0;
+            }
+        }
+        __syncthreads();
+        const auto boxes = [&]() {
+#pragma unroll 1
+            for (int r = 0; r < JW; ++r)
+                if (rs[r] < re[r]) box(r, rs[r], re[r]);
+        };
+        // One chunk: the candidates of every row with cells
+        const auto chunk = [&](int64_t i0) {
+            const int64_t i = i0 + 2 * lane;   // this lane's points i, i + 1 (inside the padded length)
+            float2 xi[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < d) {
+                    const float2 v = *reinterpret_cast<const float2*>(a.xs + (int64_t)c * Np + CDE_CK(i, Np - 1, 108));
+                    xi[c] = make_float2(-v.x, -v.y);
+                }
+            const float2 yi = *reinterpret_cast<const float2*>(a.y + i);
+#pragma unroll 1
+            for (int r = 0; r < JW; ++r) {
+                const int f0 = rs[r], f1 = re[r];
+                if (f0 == f1) continue;
+                const float* xjr = xj_s + r * d;
+                float2 dx2 = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < d) {
+                        const float2 t = __fadd2_rn(make_float2(xjr[c], xjr[c]), xi[c]);
+                        dx2 = __ffma2_rn(t, t, dx2);
+                    }
+#pragma unroll 4
+                for (int c = 8; c < d; ++c) {
+                    const float2 v = *reinterpret_cast<const float2*>(a.xs + (int64_t)c * Np + i);
+                    const float2 t = __fadd2_rn(make_float2(xjr[c], xjr[c]), make_float2(-v.x, -v.y));
+                    dx2 = __ffma2_rn(t, t, dx2);
+                }
+                const float yr = yj_s[r];
+                const float2 dy = __fadd2_rn(make_float2(yr, yr), make_float2(-yi.x, -yi.y));
+                const float2 dy2 = __fmul2_rn(dy, dy);
+                const int64_t j = ji_s[r];
+                const float RX = bx[r], RY = by[r];
+                const bool in0 = i < N && i != j && dx2.x <= RX && dy2.x <= RY;
+                const bool in1 = i + 1 < N && i + 1 != j && dx2.y <= RX && dy2.y <= RY;
+                const unsigned m0 = __ballot_sync(0xffffffffu, in0), m1 = __ballot_sync(0xffffffffu, in1);
+                if ((m0 | m1) == 0u) continue;
+                const unsigned lt = (1u << lane) - 1u;
+                const int p = __popc(m0 & lt) + __popc(m1 & lt);
+                if (in0) {
+                    lx[p] = dx2.x;
+                    ly[p] = dy2.x;
+                }
+                if (in1) {
+                    lx[p + in0] = dx2.y;
+                    ly[p + in0] = dy2.y;
+                }
+                __syncwarp();
+                const int nc = __popc(m0) + __popc(m1);
+                bool moved = false;
+                for (int f = f0 + lane; f < f1; f += 32) {
+                    const float A = As[f], B = Bs[f];
+                    float X = Xw[f], Y = Yw[f], S = Sw[f];
+                    for (int q = 0; q < nc; ++q) {
+                        const float qx = lx[q], qy = ly[q];
+                        float e = fmaf(A, qx - X, B * (qy - Y));
+                        if (e < 0.f) {   // a lower point: the new anchor
+                            S *= ex2_approx(kFbEx2Fix + e);
+                            X = qx;
+                            Y = qy;
+                            e = 0.f;
+                            moved = true;
+                        }
+                        S += ex2_approx(kFbEx2Fix - e);
+                    }
+                    Xw[f] = X;
+                    Yw[f] = Y;
+                    Sw[f] = S;
+                }
+                __syncwarp();
+                if (__any_sync(0xffffffffu, moved)) box(r, f0, f1);
+            }
+        };
+        boxes();
+#pragma unroll 1
+        for (int64_t i0 = (int64_t)warp * 64; i0 < N; i0 += NW * 64) chunk(i0);
+        __syncthreads();
+        // merge the warps at the lowest anchor, in warp order
+        for (int f = tid; f < n; f += NT) {
+            const int c = flag_s[base + f], r = c / GG;
+            const float A = As[f], B = Bs[f];
+            float X = Xs[f], Y = Ys[f];
+#pragma unroll
+            for (int w = 1; w < NW; ++w) {
+                const float Xo = Xs[w * CAP + f], Yo = Ys[w * CAP + f];
+                if (fmaf(A, Xo - X, B * (Yo - Y)) < 0.f) {
+                    X = Xo;
+                    Y = Yo;
+                }
+            }
+            float tot = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w)
+                tot += Ss[w * CAP + f] *
+                       ex2_approx(kFbEx2Fix - fmaf(A, Xs[w * CAP + f] - X, B * (Ys[w * CAP + f] - Y)));
+            const double e = (double)A * ((double)X - (double)mx_s[r]) + (double)B * ((double)Y - (double)my_s[r]);
+            la2[c] = -e + log2_wide(tot);
+        }
+        __syncthreads();
+    }
+}
+
+// The same recomputation in two passes, for the 32 x 32 shape: there the code of the
+// one-pass form costs the tile body's main loop more than the pass saves (the compiler
+// schedules that loop at its register limit: N = 20,000, d = 5 11.4 against 10.1 ms,
+// d = 2 4.2 / 3.7; only at d = 12, N = 12,000 it would gain, 5.0 / 5.6), as a call or inline.
+// For a cell (row j, k, l) let X_i = dx2_i - m_x,j, Y_i = dy2_i - m_y,j and
 // e_i = a1_k X_i + a2_l Y_i.  Then At = sum_i 2^{-e_i} = 2^{-e_*} S with
 // S = sum_i 2^{-(a1_k (dx2_i - dx2_*) + a2_l (dy2_i - dy2_*))} for the minimiser
 // i* (its term is exactly 1), and log2 At = -e_* + log2 S.  All flagged cells
@@ -199,7 +420,7 @@ constexpr float kFbEx2Fix = 7.39e-8f;
 // order in which warps finish, and it cannot overflow).  Both passes compute
 // dx2 and dy2 with the tile body's FP32 formula.
 template <class C, class Coef>
-__device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, float* sm, int nfl) {
+__device__ __forceinline__ void loo_fallback_two_pass(const LooArgs& a, const Coef& cf, float* sm, int nfl) {
     constexpr int GG = C::GG, G2 = C::G2v, JW = C::JW, NT = C::kThreads, NW = C::kWarps;
     constexpr int LG2 = G2 == 4 ? 2 : G2 == 8 ? 3 : (G2 == 16 ? 4 : 5);
     constexpr int JG = JW * GG;
@@ -450,29 +671,67 @@ __device__ __forceinline__ void loo_unit_epilogue(const LooArgs& a, const Coef& 
     int* nflag_s = reinterpret_cast<int*>(sm + C::off_nflag(d));
         // ---- shifted log numerators; flag cells that lost range ----
         double* la2 = reinterpret_cast<double*>(big);
-#pragma unroll
-        for (int m = 0; m < (CELLS + 255) / 256; ++m) {
-            const int c = tid + 256 * m;
-            if (CELLS % 256 != 0 && c >= CELLS) continue;
+        constexpr int NC = (CELLS + 255) / 256;
+        // cell c of this thread: its log numerator, unless it is to be recomputed.  Cells of
+        // the padded grid (the last bandwidth repeated) are never output: they are not
+        // recomputed either.
+        const auto flagged = [&](int m, int c) {
             const int jl = c / GG;
-            if (!vr_s[jl]) continue;
+            if (!vr_s[jl]) return false;
             const float v = At[m];
-            // cells of the padded grid (the last bandwidth repeated) are never
-            // output: they are not recomputed either
             const int kl = c - jl * GG;
             const bool padded = kl / G2 >= a.G1r || kl % G2 >= a.G2r;
             if (v >= a.thresh || padded) {
                 la2[c] = log2_wide(v);
-            } else {
-                const int q = atomicAdd(nflag_s, 1);
-                flag_s[q] = c;
+                return false;
             }
-        }
-        __syncthreads();
-        if constexpr (KERN == 0) {
-            // (Epanechnikov sums need no shift: their threshold is 0, nothing is flagged)
-            const int nfl = *nflag_s;
-            if (nfl > 0) loo_fallback<C>(a, cf, sm, nfl);
+            return true;
+        };
+        if constexpr (KERN == 0 && C::kOnePass) {
+            // list the flagged cells in cell order: offsets from the (m, warp) counts
+            const int warp = tid >> 5, lane = tid & 31;
+            unsigned fm[NC];
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+                const int c = tid + 256 * m;
+                const bool f = (CELLS % 256 == 0 || c < CELLS) && flagged(m, c);
+                fm[m] = __ballot_sync(0xffffffffu, f);
+                if (lane == 0) nflag_s[8 * m + warp] = __popc(fm[m]);
+            }
+            __syncthreads();
+            const int cnt = lane < 8 * NC ? nflag_s[lane] : 0;
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int nfl = __shfl_sync(0xffffffffu, incl, 31);
+            if (nfl > 0) {
+#pragma unroll
+                for (int m = 0; m < NC; ++m) {
+                    const int b0 = __shfl_sync(0xffffffffu, incl - cnt, 8 * m + warp);
+                    if ((fm[m] >> lane) & 1u) flag_s[b0 + __popc(fm[m] & ((1u << lane) - 1u))] = tid + 256 * m;
+                }
+                __syncthreads();
+                loo_fallback<C>(a, cf, sm, nfl);
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+                const int c = tid + 256 * m;
+                if (CELLS % 256 != 0 && c >= CELLS) continue;
+                if (flagged(m, c)) {
+                    const int q = atomicAdd(nflag_s, 1);
+                    flag_s[q] = c;
+                }
+            }
+            __syncthreads();
+            if constexpr (KERN == 0) {
+                // (Epanechnikov sums need no shift: their threshold is 0, nothing is flagged)
+                const int nfl = *nflag_s;
+                if (nfl > 0) loo_fallback_two_pass<C>(a, cf, sm, nfl);
+            }
         }
         __syncthreads();
 

@@ -23,8 +23,9 @@
 //
 // Bound by instruction issue (61% active, the tensor pipe 9%).  Measured against the
 // 16 x 8 body, tile kernel alone: N = 24,007, d = 12, 4 x 4: 8.3 -> 5.2 ms, of which
-// the exact recomputation of underflowing cells is 3.7 ms on both sides (4.6 -> 1.5 ms
-// without it); N = 2,000, d = 1, 8 x 8: 63 -> 51 us.  Grids with more than 8
+// the exact recomputation of underflowing cells was 3.7 ms on both sides (4.6 -> 1.5 ms
+// without it; with the one-pass recomputation of loo_common.cuh 2.5 ms in all);
+// N = 2,000, d = 1, 8 x 8: 63 -> 51 us (then 38).  Grids with more than 8
 // bandwidths on an axis keep the one-row tiles: at K1 = 16 nothing is shared.
 #pragma once
 
@@ -47,8 +48,9 @@ struct PackCfg {
     static constexpr int WST = (JW / 2) * T1S + JW * T2S;
     static constexpr int COMB = kWarps * JW * GG + kWarps * JW * K1;
     __host__ __device__ static int big(int) {
-        const int s = kWarps * WST;
-        return s > COMB ? s : COMB;
+        const int s = kWarps * WST, f = 28 * JW * GG;   // f: the exact recomputation
+        const int m = s > COMB ? s : COMB;
+        return m > f ? m : f;
     }
     __host__ __device__ static int dpad(int d) { return JW * d; }
     __host__ __device__ static int off_xj(int d) { return big(d); }                   // [JW][d]
@@ -62,8 +64,13 @@ struct PackCfg {
     __host__ __device__ static int off_btl(int d) { return off_rp(d) + 4 * JW; }
     __host__ __device__ static int off_flag(int d) { return off_btl(d) + 2 * JW * K1; }
     __host__ __device__ static int off_nflag(int d) { return off_flag(d) + JW * GG; }
-    static constexpr int FBW = kWarps * 96 + 8 * 8;
-    __host__ __device__ static int off_fbw(int d) { return off_nflag(d) + 4; }
+    // exact recomputation (see MmaCfg): one round holds every cell
+    static constexpr bool kOnePass = true;
+    static constexpr int FBCAP = JW * GG;
+    static constexpr int FBW = kWarps * 144 + 2 * 8;
+    __host__ __device__ static int off_fbw(int d) { return off_nflag(d) + 32; }
+    __host__ __device__ static int off_fbS(int) { return 4 * JW * GG; }
+    __host__ __device__ static int off_fbX(int) { return (4 + kWarps) * JW * GG; }
     static size_t smem_bytes(int d) { return (size_t)(off_fbw(d) + FBW) * sizeof(float); }
     // position of row r in the pair order: its pair (one row of each half of the M
     // tile), then its half
@@ -93,7 +100,6 @@ __device__ __forceinline__ void loo_tile_pack(const LooArgs& a, const Coef& cf, 
     long long* ji_s = reinterpret_cast<long long*>(sm + C::off_ji(d));
     int* vr_s = reinterpret_cast<int*>(sm + C::off_vr(d));
     double* btl_s = reinterpret_cast<double*>(sm + C::off_btl(d));
-    int* nflag_s = reinterpret_cast<int*>(sm + C::off_nflag(d));
     float* t1s = sm + warp * C::WST;
     float* t2s = t1s + NP * C::T1S;
     // this lane's fragment rows and columns: A row g (and g + 8) is bandwidth g % K1 of
@@ -137,7 +143,6 @@ __device__ __forceinline__ void loo_tile_pack(const LooArgs& a, const Coef& cf, 
             rp_s[2 * JW + p] = my;
             reinterpret_cast<int*>(rp_s)[3 * JW + p] = (int)j;
         }
-        if (tid == 0) *nflag_s = 0;
         __syncthreads();
         for (int e = tid; e < JW * d; e += C::kThreads) {
             const int r = e & (JW - 1), c = e / JW;

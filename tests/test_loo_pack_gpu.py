@@ -48,5 +48,22 @@ def test_packed_rows_equal_the_wide_grid(ctx, kernel, N, d, G1, G2):
     tot = got.sum(0)
     fin = np.isfinite(tot)
     assert np.array_equal(np.isfinite(Lc), fin)
-    assert np.all(np.abs(Lc - tot)[fin] <= 1e-12 * np.abs(got).sum(0)[fin])   # FP64 summation order only
+    assert np.all(np.abs(Lc[fin] - tot[fin]) <= 1e-12 * np.abs(got).sum(0)[fin])   # FP64 summation order only
+    cde.cde_destroy_dataset(ctx, ds)
+
+
+@pytest.mark.parametrize("G1,G2,d", [(4, 4, 12), (8, 8, 3), (16, 8, 9), (16, 16, 5), (32, 8, 2), (16, 32, 4), (32, 16, 12)])
+def test_one_pass_recomputation(ctx, G1, G2, d):
+    """Bandwidths so small that most cells of most rows underflow (units with more
+    recomputed cells than one round holds at 16 x 8), on sizes off the chunk grid."""
+    N = 713
+    x, y = synth.gmm_sine(N, d, seed=40 + d)
+    h1, h2 = synth.bandwidth_grid(0.03, 0.3, G1), synth.bandwidth_grid(0.003, 0.05, G2)
+    x64 = (x.astype(np.float64) - x.astype(np.float64).mean(0)) / x.astype(np.float64).std(0, ddof=1)
+    ds = cde.cde_create_dataset(ctx, x, y, standardize=True)
+    rows = np.arange(0, N, 3)
+    got = cde.cde_loo_rows(ctx, ds, h1, h2, rows)
+    ref = oracle.loo_rows(x, y, h1, h2, rows=rows, standardize_x=True)[0]
+    ok, worst = rows_within_bound(got, ref, x64, y, h1, h2, rows)
+    assert ok, worst
     cde.cde_destroy_dataset(ctx, ds)
