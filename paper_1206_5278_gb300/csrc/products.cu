@@ -14,18 +14,23 @@
 // shared memory point-major, the data range split
 // over gridDim.y; split partials are summed in FP64 in split order.
 //
-// k_cond_sample: one CTA per query.  A draw from fhat(.|x_q) is a mixture
+// k_chunk_weights and k_cond_sample: a draw from fhat(.|x_q) is a mixture
 // draw: an index i with probability u_qi / sum u (inverse CDF over the
 // cumulative weights), then y_i + h2 e with e from the y kernel (inverse CDF:
 // Phi^{-1} for the Gaussian, 2 sin(asin(2V - 1)/3) for the Epanechnikov kernel,
-// whose CDF is (2 + 3t - t^3)/4).  The cumulative weights come from a block
-// scan over chunks of 256 points in a fixed order, computed twice (total, then
-// the search) with identical results; the S index targets are sorted so the
-// second pass resolves them chunk by chunk.  The S values are then sorted and
-// the narrowest window of ceil((1 - alpha) S) consecutive values is taken.
-// Random numbers: value k of the SplitMix64 stream of the seed, k = 2 (q S + s)
-// for the index draw of sample s of query q and k + 1 for its kernel offset;
-// 24 random bits give u = (bits + 1/2) 2^-24 in (0, 1).
+// whose CDF is (2 + 3t - t^3)/4).  The cumulative weights are summed in a fixed
+// order: inside a chunk of 256 points by a scan (32-point segments pairwise, then
+// the segments in turn), over the chunks in turn.  k_chunk_weights forms the
+// chunk totals with one query per lane (the points are broadcast, a segment's
+// pairwise sum is a tree in registers: no shuffles and one barrier per chunk);
+// k_cond_sample, one CTA per query, sums them, sorts the S index targets, finds
+// each chunk's targets in the sorted list, and only for chunks with targets
+// repeats the scan, one chunk per warp, to resolve them.  The S values are then
+// sorted and the narrowest window of ceil((1 - alpha) S) consecutive values is
+// taken.  Random numbers: value k of the SplitMix64 stream of the seed,
+// k = 2 (q S + s) for the index draw of sample s of query q and k + 1 for its
+// kernel offset; 24 random bits give u = (bits + 1/2) 2^-24 in (0, 1).
+#include <algorithm>
 #include <cmath>
 
 #include "cde_internal.h"
@@ -203,26 +208,47 @@ __global__ void __launch_bounds__(kCSThreads) k_cond_stats(const StatArgs a) {
     }
 }
 
-// mean = sum u y / sum u (NaN when sum u = 0), fat = norm * sum u w / sum u (0 then)
-__global__ void k_cond_stats_final(const float* __restrict__ part, int n_split, int64_t Q, double norm,
-                                   double* __restrict__ mean, double* __restrict__ fat) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= Q) return;
+// mean = sum u y / sum u (NaN when sum u = 0), fat = norm * sum u w / sum u (0 then).
+// A CTA sums 32 queries' split partials in FP64, eight threads per query over the splits
+// (one thread per query waited for one strided load after the other: 173 us for 1,000
+// queries x 391 splits).
+__global__ void __launch_bounds__(256) k_cond_stats_final(const float* __restrict__ part, int n_split, int64_t Q,
+                                                          double norm, double* __restrict__ mean,
+                                                          double* __restrict__ fat) {
+    __shared__ double red[8][32][3];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t q = (int64_t)blockIdx.x * 32 + lane;
     double s0 = 0, s1 = 0, s2 = 0;
-    for (int s = 0; s < n_split; ++s) {
-        const float* p = part + ((int64_t)s * Q + q) * 3;
-        s0 += p[0];
-        s1 += p[1];
-        s2 += p[2];
+    if (q < Q) {
+#pragma unroll 4
+        for (int s = g; s < n_split; s += 8) {
+            const float* p = part + ((int64_t)s * Q + q) * 3;
+            s0 += p[0];
+            s1 += p[1];
+            s2 += p[2];
+        }
+    }
+    red[g][lane][0] = s0;
+    red[g][lane][1] = s1;
+    red[g][lane][2] = s2;
+    __syncthreads();
+    if (g != 0 || q >= Q) return;
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+        s0 += red[w][lane][0];
+        s1 += red[w][lane][1];
+        s2 += red[w][lane][2];
     }
     if (mean) mean[q] = s1 / s0;
     if (fat) fat[q] = s0 > 0.0 ? norm * s2 / s0 : 0.0;
 }
 
 // --------------------------------------------------------------------------
-// Sampling and the narrowest interval: one CTA (256 threads) per query
+// Sampling and the narrowest interval
 // --------------------------------------------------------------------------
-constexpr int kSmpThreads = 256, kSmpMax = 4096;
+constexpr int kSmpThreads = 256, kSmpWarps = kSmpThreads / 32, kSmpMax = 4096;
+constexpr int kChunk = 256;           // points per chunk of the cumulative weights
+constexpr int kEndsMax = 2048;        // chunk ends kept in shared memory
 
 struct SampleArgs {
     const float* xs;
@@ -230,46 +256,95 @@ struct SampleArgs {
     const float* xq;   // [d][Qp]
     const float* mq;   // [Q] (Gaussian)
     int64_t N, Np, Q, Qp;
+    int64_t q0, nq;    // this launch's queries q0 .. q0 + nq - 1
+    int64_t n_chunks;
     int d, S, SP, m_keep;   // samples, padded power of two, window size ceil((1-alpha) S)
     float a1, h2;
     uint64_t seed;
+    float* ct;         // [n_chunks][nq] chunk totals, then running totals
     float* lo;         // [Q]
     float* hi;         // [Q]
     float* samples;    // [Q][S] sorted, or null
 };
 
+// pairwise sum of n consecutive terms: f(p) the p-th
+template <int n, class F>
+__device__ __forceinline__ float2 tree_sum2(const F& f, int p) {
+    if constexpr (n == 1) return f(p);
+    else return __fadd2_rn(tree_sum2<n / 2>(f, p), tree_sum2<n / 2>(f, p + n / 2));
+}
+
+// Chunk totals: two queries per thread (packed FP32x2), points point-major in shared
+// memory.  Points past N are infinitely far (weight exactly 0).
+constexpr int kCwThreads = 64, kCwQ = 2 * kCwThreads;
+
+template <int KERN, int DREG>
+__global__ void __launch_bounds__(kCwThreads) k_chunk_weights(const SampleArgs a, int64_t chunks_per_cta) {
+    constexpr int TP = DREG > 32 ? kChunk / 2 : kChunk;   // points staged at a time (at most 32 KB)
+    __shared__ __align__(16) float xt[TP][DREG];
+    const int tid = threadIdx.x;
+    const int64_t qa = a.q0 + (int64_t)blockIdx.x * kCwQ + tid, qb = qa + kCwThreads, qe = a.q0 + a.nq;
+    const int64_t qac = qa < qe ? qa : a.q0, qbc = qb < qe ? qb : a.q0;
+    const int d = a.d;
+    float2 xq[DREG];
+#pragma unroll
+    for (int c = 0; c < DREG; ++c)
+        xq[c] = c < d ? make_float2(a.xq[(int64_t)c * a.Qp + qac], a.xq[(int64_t)c * a.Qp + qbc])
+                      : make_float2(0.f, 0.f);
+    const float2 mq = KERN == 0 ? make_float2(a.mq[qac], a.mq[qbc]) : make_float2(0.f, 0.f);
+    const float a1 = a.a1;
+    const int64_t k1 = min(a.n_chunks, ((int64_t)blockIdx.y + 1) * chunks_per_cta);
+    for (int64_t k = (int64_t)blockIdx.y * chunks_per_cta; k < k1; ++k) {
+        const auto weight = [&](int p) {
+            float2 dx2 = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int c = 0; c < DREG; c += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&xt[p][c]);
+                const float x[4] = {-v.x, -v.y, -v.z, -v.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 t = __fadd2_rn(xq[c + e], make_float2(x[e], x[e]));
+                    dx2 = __ffma2_rn(t, t, dx2);
+                }
+            }
+            if constexpr (KERN == 0) {
+                const float2 arg = __fmul2_rn(make_float2(a1, a1), __fadd2_rn(mq, make_float2(-dx2.x, -dx2.y)));
+                return make_float2(ex2p(arg.x), ex2p(arg.y));
+            } else {
+                return make_float2(fma_sat_p(-a1, dx2.x, 1.f), fma_sat_p(-a1, dx2.y, 1.f));
+            }
+        };
+        float2 tot = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int p0 = 0; p0 < kChunk; p0 += TP) {
+            __syncthreads();
+            for (int p = tid; p < TP; p += kCwThreads) {
+                const int64_t i = k * kChunk + p0 + p;
+#pragma unroll
+                for (int c = 0; c < DREG; ++c)
+                    xt[p][c] = c < d ? (i < a.N ? a.xs[(int64_t)c * a.Np + CDE_CK(i, a.Np, 303)] : INFINITY) : 0.f;
+            }
+            __syncthreads();
+            // (the first segment's sum plus an exact 0)
+#pragma unroll 1
+            for (int s = 0; s < TP; s += 32) tot = __fadd2_rn(tree_sum2<32>(weight, s), tot);
+        }
+        if (qa < qe) a.ct[k * a.nq + (qa - a.q0)] = tot.x;
+        if (qb < qe) a.ct[k * a.nq + (qb - a.q0)] = tot.y;
+    }
+}
+
 struct SampleSmem {
     float val[kSmpMax];   // targets, then sample values
     int idx[kSmpMax];     // resolved data index per target
-    float P[kSmpThreads]; // inclusive scan of the chunk's weights
-    float wsum[kSmpThreads / 32];
-    int wpos[kSmpThreads / 32];
+    float ends[kEndsMax]; // running totals after each chunk (a tile of them at a time)
+    float P[kSmpWarps][kChunk]; // inclusive scan of a warp's chunk
     float xq[kMaxD];
-    float total, base;
-    int last, chunk_last, p, p2;
-    float best_w[kSmpThreads / 32];
-    int best_k[kSmpThreads / 32];
+    float total;
+    int last;             // the last chunk with weight
+    float best_w[kSmpWarps];
+    int best_k[kSmpWarps];
 };
-
-// inclusive scan of v over the CTA in a fixed order (warp shuffles, then the
-// warp totals); returns this thread's prefix and leaves the total in P[255]
-__device__ __forceinline__ float block_scan(float v, SampleSmem& S) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float n = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += n;
-    }
-    if (lane == 31) S.wsum[warp] = v;
-    __syncthreads();
-    if (tid == 0)
-        for (int w = 1; w < kSmpThreads / 32; ++w) S.wsum[w] += S.wsum[w - 1];
-    __syncthreads();
-    if (warp > 0) v += S.wsum[warp - 1];
-    S.P[tid] = v;
-    __syncthreads();
-    return v;
-}
 
 __device__ __forceinline__ void bitonic_sort(float* v, int n) {
     for (int k = 2; k <= n; k <<= 1)
@@ -289,40 +364,70 @@ __device__ __forceinline__ void bitonic_sort(float* v, int n) {
         }
 }
 
+// One chunk's weights (point 32 s + lane of the chunk in u[s])
 template <int KERN>
-__device__ __forceinline__ float weight_at(const SampleArgs& a, const SampleSmem& S, int64_t i, float mq) {
-    if (i >= a.N) return 0.f;
-    float dx2 = 0.f;
+__device__ __forceinline__ void chunk_weights(const SampleArgs& a, const SampleSmem& S, int64_t k, float mq,
+                                              float (&u)[kChunk / 32]) {
+    constexpr int NS = kChunk / 32;
+    const int lane = threadIdx.x & 31;
+    const float* x = a.xs + CDE_CK(k * kChunk, a.Np - kChunk + 1, 304) + lane;   // Np is a multiple of 256
+    float dx2[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) dx2[s] = 0.f;
     for (int c = 0; c < a.d; ++c) {
-        const float v = S.xq[c] - a.xs[(int64_t)c * a.Np + i];
-        dx2 = fmaf(v, v, dx2);
+        const float xqc = S.xq[c];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            const float v = xqc - x[(int64_t)c * a.Np + 32 * s];
+            dx2[s] = fmaf(v, v, dx2[s]);
+        }
     }
-    return xweight<KERN>(dx2, a.a1, mq);
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+        u[s] = k * kChunk + 32 * s + lane < a.N ? xweight<KERN>(dx2[s], a.a1, mq) : 0.f;
 }
 
 template <int KERN>
 __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a) {
     extern __shared__ float4 smp4[];
     SampleSmem& S = *reinterpret_cast<SampleSmem*>(smp4);
-    const int tid = threadIdx.x;
-    const int64_t q = blockIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t q = a.q0 + blockIdx.x;
+    const int64_t nch = a.n_chunks;
+    float* ct = a.ct + blockIdx.x;   // stride nq
     for (int c = tid; c < a.d; c += kSmpThreads) S.xq[c] = a.xq[(int64_t)c * a.Qp + q];
     const float mq = KERN == 0 ? a.mq[q] : 0.f;
     if (tid == 0) {
         S.total = 0.f;
         S.last = -1;
     }
-    __syncthreads();
-    const int64_t n_chunks = (a.N + kSmpThreads - 1) / kSmpThreads;
-    // pass 1: the total weight, chunk by chunk in the order of pass 2
-    for (int64_t k = 0; k < n_chunks; ++k) {
-        const int64_t i = k * kSmpThreads + tid;
-        const float u = weight_at<KERN>(a, S, i, mq);
-        block_scan(u, S);
-        if (u > 0.f) atomicMax(&S.last, (int)i);
-        if (tid == 0) S.total = S.total + S.P[kSmpThreads - 1];
+    // running totals over the chunks, in turn (more than kEndsMax chunks: also to global)
+    const bool local = nch <= kEndsMax;
+    for (int64_t k0 = 0; k0 < nch; k0 += kEndsMax) {
+        const int n = (int)min((int64_t)kEndsMax, nch - k0);
         __syncthreads();
+        int last = -1;
+        for (int k = tid; k < n; k += kSmpThreads) {
+            const float v = ct[(k0 + k) * a.nq];
+            S.ends[k] = v;
+            if (v > 0.f) last = (int)(k0 + k);
+        }
+        if (last >= 0) atomicMax(&S.last, last);
+        __syncthreads();
+        if (tid == 0) {
+            float t = S.total;
+#pragma unroll 8
+            for (int k = 0; k < n; ++k) {
+                t = t + S.ends[k];
+                S.ends[k] = t;
+            }
+            S.total = t;
+        }
+        __syncthreads();
+        if (!local)
+            for (int k = tid; k < n; k += kSmpThreads) ct[(k0 + k) * a.nq] = S.ends[k];
     }
+    const auto end_of = [&](int64_t k) { return k < 0 ? 0.f : local ? S.ends[k] : ct[k * a.nq]; };
     const float total = S.total;
     const int last = S.last;
     if (last < 0 || !(total > 0.f)) {  // no weight (Epanechnikov: no x-neighbour)
@@ -339,49 +444,77 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
         S.val[s] = s < a.S ? uniform24(a.seed, 2 * ((uint64_t)q * a.S + s)) * total : INFINITY;
     __syncthreads();
     bitonic_sort(S.val, a.SP);
-    // pass 2: resolve the targets against the cumulative weights
-    if (tid == 0) {
-        S.base = 0.f;
-        S.p = 0;
-    }
-    __syncthreads();
-    for (int64_t k = 0; k < n_chunks; ++k) {
-        const int64_t i = k * kSmpThreads + tid;
-        const float u = weight_at<KERN>(a, S, i, mq);
-        if (tid == 0) S.chunk_last = -1;
-        block_scan(u, S);
-        if (u > 0.f) atomicMax(&S.chunk_last, tid);
-        if (tid == 0) {
-            const float end = S.base + S.P[kSmpThreads - 1];
-            int lo = S.p, hi = a.S;  // first target >= end
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (S.val[mid] < end) lo = mid + 1;
-                else hi = mid;
-            }
-            S.p2 = lo;
+    // Resolve the targets against the cumulative weights: those below the end of chunk k
+    // and not below its beginning are chunk k's.  Warp w takes the chunks 8 m + w, the
+    // target ranges of 32 of them at a time (lane = chunk).
+    const auto first_at = [&](float v) {   // first target >= v
+        int lo = 0, hi = a.S;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (S.val[mid] < v) lo = mid + 1;
+            else hi = mid;
         }
-        __syncthreads();
-        if (S.chunk_last >= 0)
-            for (int s = S.p + tid; s < S.p2; s += kSmpThreads) {
-                const float t = S.val[s] - S.base;
-                int lo = 0, hi = kSmpThreads;  // first prefix above t
+        return lo;
+    };
+    for (int64_t m0 = 0; m0 * kSmpWarps < nch; m0 += 32) {
+        const int64_t kl = (m0 + lane) * kSmpWarps + warp;
+        int p = 0, p2 = 0;
+        if (kl < nch) {
+            p = first_at(end_of(kl - 1));
+            p2 = first_at(end_of(kl));
+        }
+        unsigned live = __ballot_sync(0xffffffffu, p < p2);
+        while (live) {
+            const int src = __ffs(live) - 1;
+            live &= live - 1;
+            const int64_t k = (m0 + src) * kSmpWarps + warp;
+            const int s0 = __shfl_sync(0xffffffffu, p, src), s1 = __shfl_sync(0xffffffffu, p2, src);
+            const float base = end_of(k - 1);
+            float u[kChunk / 32];
+            chunk_weights<KERN>(a, S, k, mq, u);
+            int chunk_last = -1;
+            float before = 0.f;   // the segments before this one
+#pragma unroll
+            for (int g = 0; g < kChunk / 32; ++g) {
+                float v = u[g];
+                const unsigned pos = __ballot_sync(0xffffffffu, v > 0.f);
+                if (pos) chunk_last = 32 * g + 31 - __clz(pos);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float n = __shfl_up_sync(0xffffffffu, v, o);
+                    if (lane >= o) v += n;
+                }
+                const float seg = __shfl_sync(0xffffffffu, v, 31);
+                S.P[warp][32 * g + lane] = g > 0 ? v + before : v;
+                before = g > 0 ? seg + before : seg;
+            }
+            __syncwarp();
+            for (int s = s0 + lane; s < s1; s += 32) {
+                const float t = S.val[s] - base;
+                int lo = 0, hi = kChunk;  // first prefix above t
                 while (lo < hi) {
                     const int mid = (lo + hi) >> 1;
-                    if (S.P[mid] <= t) lo = mid + 1;
+                    if (S.P[warp][mid] <= t) lo = mid + 1;
                     else hi = mid;
                 }
-                if (lo > S.chunk_last) lo = S.chunk_last;  // rounding at the chunk's end
-                S.idx[s] = (int)(k * kSmpThreads + lo);
+                if (lo > chunk_last) lo = chunk_last;  // rounding at the chunk's end
+                S.idx[CDE_CK(s, kSmpMax, 305)] = (int)(k * kChunk + lo);
             }
-        __syncthreads();
-        if (tid == 0) {
-            S.base = S.base + S.P[kSmpThreads - 1];
-            if (S.chunk_last >= 0) S.p = S.p2;
+            __syncwarp();
         }
-        __syncthreads();
     }
-    for (int s = S.p + tid; s < a.S; s += kSmpThreads) S.idx[s] = last;  // targets at the very top
+    const int top = first_at(total);   // targets at the very top: the last point with weight
+    if (top < a.S && warp == 0) {
+        float u[kChunk / 32];
+        chunk_weights<KERN>(a, S, last, mq, u);
+        int at = 0;
+#pragma unroll
+        for (int g = 0; g < kChunk / 32; ++g) {
+            const unsigned pos = __ballot_sync(0xffffffffu, u[g] > 0.f);
+            if (pos) at = 32 * g + 31 - __clz(pos);
+        }
+        for (int s = top + lane; s < a.S; s += 32) S.idx[s] = (int)((int64_t)last * kChunk + at);
+    }
     __syncthreads();
     // sample values, sorted
     for (int s = tid; s < a.SP; s += kSmpThreads) {
@@ -469,6 +602,15 @@ static void launch_stats_d(const StatArgs& a, dim3 grid, cudaStream_t st) {
     else k_cond_stats<KERN, 64, 1><<<grid, kCSThreads, 0, st>>>(a);
 }
 
+template <int KERN>
+static void launch_chunk_weights(const SampleArgs& a, dim3 grid, int64_t cpc, cudaStream_t st) {
+    if (a.d <= 4) k_chunk_weights<KERN, 4><<<grid, kCwThreads, 0, st>>>(a, cpc);
+    else if (a.d <= 8) k_chunk_weights<KERN, 8><<<grid, kCwThreads, 0, st>>>(a, cpc);
+    else if (a.d <= 16) k_chunk_weights<KERN, 16><<<grid, kCwThreads, 0, st>>>(a, cpc);
+    else if (a.d <= 32) k_chunk_weights<KERN, 32><<<grid, kCwThreads, 0, st>>>(a, cpc);
+    else k_chunk_weights<KERN, kMaxD><<<grid, kCwThreads, 0, st>>>(a, cpc);
+}
+
 static int cond_stats_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, const float* d_xq,
                               const float* d_yq, int64_t Q, double* d_mean, double* d_fat, cudaStream_t st) {
     timing_reset(ctx);
@@ -509,7 +651,7 @@ static int cond_stats_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double 
     timing_end(ctx, st);
     CDE_CUDA(cudaGetLastError());
     const double norm = epan ? std::exp(epan_log_norm(1)) / h2 : 1.0 / (2.5066282746310002 * h2);
-    k_cond_stats_final<<<(unsigned)((Q + 255) / 256), 256, 0, st>>>(part, (int)ns, Q, norm, d_mean,
+    k_cond_stats_final<<<(unsigned)((Q + 31) / 32), 256, 0, st>>>(part, (int)ns, Q, norm, d_mean,
                                                                    d_yq ? d_fat : nullptr);
     CDE_CUDA(cudaGetLastError());
     cudaFreeAsync(part, st);
@@ -553,10 +695,28 @@ static int cond_interval_enqueue(cde_ctx* ctx, const Dataset& D, double h1, doub
     static std::atomic<uint64_t> attr0{0}, attr1{0};
     CDE_CUDA(smem_attr_once(attr0, k_cond_sample<0>, (int)sizeof(SampleSmem)));
     CDE_CUDA(smem_attr_once(attr1, k_cond_sample<1>, (int)sizeof(SampleSmem)));
-    // one CTA per query (grid.x allows 2^31 - 1)
-    if (epan) k_cond_sample<1><<<(unsigned)Q, kSmpThreads, sizeof(SampleSmem), st>>>(a);
-    else k_cond_sample<0><<<(unsigned)Q, kSmpThreads, sizeof(SampleSmem), st>>>(a);
-    CDE_CUDA(cudaGetLastError());
+    a.n_chunks = (D.N + kChunk - 1) / kChunk;
+    // queries in batches whose chunk totals fit 64 MB (at least 128)
+    const int64_t qmax = std::max<int64_t>(kCwQ, ((int64_t)16 << 20) / a.n_chunks / kCwQ * kCwQ);
+    const int64_t qbatch = std::min(Q, qmax);
+    CDE_CUDA(cudaMallocAsync((void**)&a.ct, (size_t)(a.n_chunks * qbatch) * sizeof(float), st));
+    for (int64_t q0 = 0; q0 < Q; q0 += qbatch) {
+        a.q0 = q0;
+        a.nq = std::min(qbatch, Q - q0);
+        const int64_t gx = (a.nq + kCwQ - 1) / kCwQ;
+        // about 16 CTAs of 64 threads per SM, each a run of chunks
+        const int64_t gy = std::min(a.n_chunks, std::min<int64_t>(65535, std::max<int64_t>(1, 16LL * ctx->sm_count / gx)));
+        const int64_t cpc = (a.n_chunks + gy - 1) / gy;
+        const dim3 cg((unsigned)gx, (unsigned)((a.n_chunks + cpc - 1) / cpc));
+        if (epan) launch_chunk_weights<1>(a, cg, cpc, st);
+        else launch_chunk_weights<0>(a, cg, cpc, st);
+        CDE_CUDA(cudaGetLastError());
+        // one CTA per query
+        if (epan) k_cond_sample<1><<<(unsigned)a.nq, kSmpThreads, sizeof(SampleSmem), st>>>(a);
+        else k_cond_sample<0><<<(unsigned)a.nq, kSmpThreads, sizeof(SampleSmem), st>>>(a);
+        CDE_CUDA(cudaGetLastError());
+    }
+    cudaFreeAsync(a.ct, st);
     cudaFreeAsync(xq, st);
     cudaFreeAsync(mq, st);
     return CDE_OK;
