@@ -29,9 +29,10 @@
 // derivatives.
 //
 // The i range is split over gridDim.y CTAs; split partials (M, S_A, S_Ax,
-// S_Ay, S_B, S_Bx) are merged per row in FP64 in split order, the per-row
+// S_Ay, S_B, S_Bx) are merged per row in FP64 in a fixed order, the per-row
 // log-ratio and derivatives are formed in FP64, and rows are summed in a
 // fixed order, so the result is bitwise reproducible.
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <type_traits>
@@ -505,50 +506,74 @@ __global__ void __launch_bounds__(kGTThreads, 1) k_grad_tc(const GradArgs g) {
     }
 }
 
-// Per row: merge split partials (FP64, split order), then
+// Per row: merge split partials (FP64, a fixed order), then
 // rowv[j] = {ell_j, d ell_j/d ln h1, d ell_j/d ln h2}.  Gaussian rows whose
-// numerator sum fell below 2^-40 are listed for k_grad_fallback instead.
+// numerator sum fell below `thresh` are listed for k_grad_fallback instead.
+// A CTA has 32 rows, eight threads per row over the splits (the strided loads of 20 splits
+// in one thread took 23 us at N = 2,503), then one thread per row for the FP64 work: one
+// logarithm and two reciprocals.  lnk = ln h2 plus the y kernel's constant.
 __global__ void k_grad_rows(const float* __restrict__ part, int n_split, int64_t N,
-                            const float* __restrict__ my, float a2f, double h1, double h2,
-                            int epan, double lnc1, double* __restrict__ rowv, int* __restrict__ fb_count,
+                            const float* __restrict__ my, float a2f, double h1, double h2, double lnk,
+                            int epan, double thresh, double* __restrict__ rowv, int* __restrict__ fb_count,
                             int* __restrict__ fb_rows) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= N) return;
-    double SA = 0, SAx = 0, SAy = 0, SB = 0, SBx = 0;
-    for (int s = 0; s < n_split; ++s) {
-        const float* p = part + ((int64_t)s * N + j) * 6;
-        SA += p[1];
-        SAx += p[2];
-        SAy += p[3];
-        SB += p[4];
-        SBx += p[5];
+    __shared__ double red[8][32][5];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t j = (int64_t)blockIdx.x * 32 + lane;
+    double v[5] = {0, 0, 0, 0, 0};
+    if (j < N) {
+#pragma unroll 4
+        for (int s = g; s < n_split; s += 8) {
+            const float* p = part + ((int64_t)s * N + j) * 6;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) v[q] += p[q + 1];
+        }
     }
-    const double LN2 = 0.69314718055994530942, LNS2PI = 0.91893853320467274178;
+    if (n_split > 1) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q) red[g][lane][q] = v[q];
+        __syncthreads();
+        if (g == 0)
+            for (int w = 1; w < 8 && w < n_split; ++w)
+#pragma unroll
+                for (int q = 0; q < 5; ++q) v[q] += red[w][lane][q];
+    }
+    if (g != 0 || j >= N) return;
+    const double SA = v[0], SAx = v[1], SAy = v[2], SB = v[3], SBx = v[4];
+    const double LN2 = 0.69314718055994530942;
     double ell, g1, g2;
     if (epan) {
         // slots: sum u w, sum v w, sum u z, sum u, sum v
         const bool live = SA > 0.0;
-        ell = live ? log(SA) - log(SB) - (log(h2) - lnc1) : -INFINITY;
-        g1 = live ? SAx / SA - SBx / SB : 0.0;
-        g2 = live ? SAy / SA - 1.0 : 0.0;
+        const double iA = 1.0 / SA, iB = 1.0 / SB;
+        ell = live ? log(SA * iB) - lnk : -INFINITY;
+        g1 = live ? SAx * iA - SBx * iB : 0.0;
+        g2 = live ? SAy * iA - 1.0 : 0.0;
     } else {
-        if (!(SA >= 0x1p-40)) {
+        if (!(SA >= thresh)) {
             fb_rows[CDE_CK(atomicAdd(fb_count, 1), N, 404)] = (int)j;
             return;
         }
-        ell = log(SA) - log(SB) - LN2 * (double)a2f * (double)my[j] - (LNS2PI + log(h2));
-        g1 = (SAx / SA - SBx / SB) / (h1 * h1);
-        g2 = (SAy / SA) / (h2 * h2) - 1.0;
+        const double iA = 1.0 / SA, iB = 1.0 / SB;
+        ell = log(SA * iB) - LN2 * (double)a2f * (double)my[j] - lnk;
+        g1 = (SAx * iA - SBx * iB) / (h1 * h1);
+        g2 = (SAy * iA) / (h2 * h2) - 1.0;
     }
     rowv[3 * j] = ell;
     rowv[3 * j + 1] = g1;
     rowv[3 * j + 2] = g2;
 }
 
-// Exact recomputation of the listed Gaussian rows (one CTA per row, rows
-// strided over the grid): every i with the online joint shift, thread partials
-// merged with a common shift in a fixed order.
-constexpr int kFbThreads = 256;
+// Exact recomputation of the listed Gaussian rows: every i with the online
+// joint shift.  A work item is four listed rows, which share the points' loads, and
+// one of n_split ranges of the points; n_split follows from the list's length (few
+// rows: enough ranges to fill the GPU, which one CTA per row left waiting for its own
+// L2 loads).  A thread takes two adjacent points at a time, the rows go through the
+// packed FP32x2 pipe in pairs.  Thread partials are merged with a common shift in a fixed order,
+// the item's partial is stored, and the item that finishes its rows last merges them
+// in range order: a row's value depends on N and the list's length only.
+// Measured, N = 100,003, d = 32: 1.69 ms with one row per CTA (every row streamed all
+// points from L2, four loads in flight per thread) -> 0.085 ms.
+constexpr int kFbThreads = 256, kFbRows = 4, kFbCtasPerSm = 4, kFbMaxSplit = 16;
 
 __device__ __forceinline__ void merge_shifted(float& M, float (&S)[5], float Mo, const float (&So)[5]) {
     const float Mm = fminf(M, Mo);
@@ -561,78 +586,173 @@ __device__ __forceinline__ void merge_shifted(float& M, float (&S)[5], float Mo,
     M = Mm;
 }
 
-__global__ void __launch_bounds__(kFbThreads) k_grad_fallback(const GradArgs g, const int* __restrict__ fb_count,
-                                                               const int* __restrict__ fb_rows, double h1,
-                                                               double h2, double* __restrict__ rowv) {
-    __shared__ float xj_s[kMaxD];
-    __shared__ float redM[kFbThreads / 32], redS[kFbThreads / 32][5];
+// partials (M and the five sums) the fallback needs beside the splits' of N rows
+static int64_t grad_fb_entries(int64_t N, int sm_count) { return N + 4 + (int64_t)2 * kFbCtasPerSm * sm_count * kFbRows; }
+
+__global__ void __launch_bounds__(kFbThreads, kFbCtasPerSm) k_grad_fallback(const GradArgs g, const int* __restrict__ fb_count,
+                                                                            const int* __restrict__ fb_rows,
+                                                                            int* __restrict__ fb_done, double h1,
+                                                                            double h2, double* __restrict__ rowv) {
+    constexpr int RB = kFbRows, NW = kFbThreads / 32;
+    __shared__ __align__(16) float xj_s[kMaxD][RB];
+    __shared__ float redM[NW][RB], redS[NW][RB][5];
+    __shared__ int last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = *fb_count;
-    for (int r = blockIdx.x; r < n; r += gridDim.x) {
-        const int j = (int)CDE_CK(fb_rows[r], g.N, 403);
+    if (n == 0) return;
+    const int groups = (n + RB - 1) / RB;
+    const int ns = max(1, min(kFbMaxSplit, (int)(2 * gridDim.x) / groups));
+    const int64_t per = (g.N + (int64_t)ns * 2 * kFbThreads - 1) / ((int64_t)ns * 2 * kFbThreads) * 2 * kFbThreads;
+    for (int64_t item = blockIdx.x; item < (int64_t)groups * ns; item += gridDim.x) {
+        const int grp = (int)(item / ns), sp = (int)(item - (int64_t)grp * ns), r0 = grp * RB;
+        int j[RB];
+        float2 yj[RB / 2];
+        float mx[RB], my[RB], M[RB], S[RB][5];
+#pragma unroll
+        for (int b = 0; b < RB; ++b) {
+            j[b] = (int)CDE_CK(fb_rows[min(r0 + b, n - 1)], g.N, 403);
+            reinterpret_cast<float*>(yj)[b] = g.y[j[b]];
+            mx[b] = g.mx[j[b]];
+            my[b] = g.my[j[b]];
+            M[b] = INFINITY;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) S[b][q] = 0.f;
+        }
         __syncthreads();
-        for (int c = tid; c < g.d; c += kFbThreads) xj_s[c] = g.xs[(int64_t)c * g.Np + j];
+        for (int e = tid; e < g.d * RB; e += kFbThreads)
+            xj_s[e / RB][e % RB] = g.xs[(int64_t)(e / RB) * g.Np + CDE_CK(fb_rows[min(r0 + e % RB, n - 1)], g.N, 403)];
         __syncthreads();
-        const float yj = g.y[j], mx = g.mx[j], my = g.my[j];
-        float M = INFINITY, S[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int64_t i = tid; i < g.N; i += kFbThreads) {
-            float dx2 = 0.f;
+        const int64_t i1 = min(g.N, (sp + 1) * per);
+        for (int64_t i = sp * per + 2 * tid; i < i1; i += 2 * kFbThreads) {   // i + 1 < Np (Np is even)
+            float2 dx2[RB / 2][2];
+#pragma unroll
+            for (int p = 0; p < RB / 2; ++p) dx2[p][0] = dx2[p][1] = make_float2(0.f, 0.f);
+#pragma unroll 8
             for (int c = 0; c < g.d; ++c) {
-                const float q = xj_s[c] - g.xs[(int64_t)c * g.Np + i];
-                dx2 = fmaf(q, q, dx2);
+                const float2 x = *reinterpret_cast<const float2*>(g.xs + (int64_t)c * g.Np + CDE_CK(i, g.Np - 1, 405));
+                const float4 xr = *reinterpret_cast<const float4*>(xj_s[c]);
+                const float2 r[2] = {make_float2(xr.x, xr.y), make_float2(xr.z, xr.w)};
+#pragma unroll
+                for (int p = 0; p < RB / 2; ++p) {
+                    const float2 q0 = __fadd2_rn(r[p], make_float2(-x.x, -x.x));
+                    const float2 q1 = __fadd2_rn(r[p], make_float2(-x.y, -x.y));
+                    dx2[p][0] = __ffma2_rn(q0, q0, dx2[p][0]);
+                    dx2[p][1] = __ffma2_rn(q1, q1, dx2[p][1]);
+                }
             }
-            const float dy = yj - g.y[i];
-            grad_accumulate_joint(i != j, dx2, dy * dy, mx, my, g.a1, g.a2, M, S[0], S[1], S[2], S[3], S[4]);
+            const float2 yi = *reinterpret_cast<const float2*>(g.y + i);
+            const bool v1 = i + 1 < i1;
+#pragma unroll
+            for (int p = 0; p < RB / 2; ++p) {
+                const float2 d0 = __fadd2_rn(yj[p], make_float2(-yi.x, -yi.x)), e0 = __fmul2_rn(d0, d0);
+                const float2 d1 = __fadd2_rn(yj[p], make_float2(-yi.y, -yi.y)), e1 = __fmul2_rn(d1, d1);
+                const int a = 2 * p, b = 2 * p + 1;
+                grad_accumulate_joint(i != j[a], dx2[p][0].x, e0.x, mx[a], my[a], g.a1, g.a2, M[a], S[a][0], S[a][1], S[a][2],
+                                      S[a][3], S[a][4]);
+                grad_accumulate_joint(i != j[b], dx2[p][0].y, e0.y, mx[b], my[b], g.a1, g.a2, M[b], S[b][0], S[b][1], S[b][2],
+                                      S[b][3], S[b][4]);
+                grad_accumulate_joint(v1 && i + 1 != j[a], dx2[p][1].x, e1.x, mx[a], my[a], g.a1, g.a2, M[a], S[a][0],
+                                      S[a][1], S[a][2], S[a][3], S[a][4]);
+                grad_accumulate_joint(v1 && i + 1 != j[b], dx2[p][1].y, e1.y, mx[b], my[b], g.a1, g.a2, M[b], S[b][0],
+                                      S[b][1], S[b][2], S[b][3], S[b][4]);
+            }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float So[5];
+        for (int b = 0; b < RB; ++b) {
 #pragma unroll
-            for (int q = 0; q < 5; ++q) So[q] = __shfl_xor_sync(0xffffffffu, S[q], o);
-            merge_shifted(M, S, __shfl_xor_sync(0xffffffffu, M, o), So);
-        }
-        if (lane == 0) {
-            redM[warp] = M;
-#pragma unroll
-            for (int q = 0; q < 5; ++q) redS[warp][q] = S[q];
-        }
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < kFbThreads / 32; ++w) {
+            for (int o = 16; o > 0; o >>= 1) {
                 float So[5];
 #pragma unroll
-                for (int q = 0; q < 5; ++q) So[q] = redS[w][q];
-                merge_shifted(M, S, redM[w], So);
+                for (int q = 0; q < 5; ++q) So[q] = __shfl_xor_sync(0xffffffffu, S[b][q], o);
+                merge_shifted(M[b], S[b], __shfl_xor_sync(0xffffffffu, M[b], o), So);
             }
+            if (lane == 0) {
+                redM[warp][b] = M[b];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) redS[warp][b][q] = S[b][q];
+            }
+        }
+        __syncthreads();
+        if (tid < RB) {
+            float Mr = redM[0][tid], Sr[5];
+            for (int q = 0; q < 5; ++q) Sr[q] = redS[0][tid][q];
+            for (int w = 1; w < NW; ++w) {
+                float So[5];
+                for (int q = 0; q < 5; ++q) So[q] = redS[w][tid][q];
+                merge_shifted(Mr, Sr, redM[w][tid], So);
+            }
+            float* pp = g.part + ((int64_t)item * RB + tid) * 6;
+            pp[0] = Mr;
+            for (int q = 0; q < 5; ++q) pp[q + 1] = Sr[q];
+            __threadfence();
+        }
+        __syncthreads();
+        if (tid == 0) last = atomicAdd(fb_done + grp, 1) == ns - 1;
+        __syncthreads();
+        if (last && tid < RB && r0 + tid < n) {
+            __threadfence();
+            float Mr = INFINITY, Sr[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int s2 = 0; s2 < ns; ++s2) {
+                const float* pp = g.part + (((int64_t)grp * ns + s2) * RB + tid) * 6;
+                const float Mo = __ldcg(pp);
+                float So[5];
+                for (int q = 0; q < 5; ++q) So[q] = __ldcg(pp + q + 1);
+                merge_shifted(Mr, Sr, Mo, So);
+            }
+            const int64_t jr = fb_rows[r0 + tid];
             const double LN2 = 0.69314718055994530942, LNS2PI = 0.91893853320467274178;
-            const double SA = S[0], SAx = S[1], SAy = S[2], SB = S[3], SBx = S[4];
-            rowv[3 * (int64_t)j] = log(SA) - log(SB) - LN2 * ((double)M + (double)g.a2 * (double)my) -
-                                   (LNS2PI + log(h2));
-            rowv[3 * (int64_t)j + 1] = (SAx / SA - SBx / SB) / (h1 * h1);
-            rowv[3 * (int64_t)j + 2] = (SAy / SA) / (h2 * h2) - 1.0;
+            const double SA = Sr[0], SAx = Sr[1], SAy = Sr[2], SB = Sr[3], SBx = Sr[4];
+            rowv[3 * jr] = log(SA) - log(SB) - LN2 * ((double)Mr + (double)g.a2 * (double)g.my[jr]) - (LNS2PI + log(h2));
+            rowv[3 * jr + 1] = (SAx / SA - SBx / SB) / (h1 * h1);
+            rowv[3 * jr + 2] = (SAy / SA) / (h2 * h2) - 1.0;
         }
     }
 }
 
-// Fixed-order sum of the per-row triples: one CTA of 1024 threads.
-__global__ void k_sum_rows3(const double* __restrict__ rowv, int64_t N, double* __restrict__ out3) {
-    __shared__ double red[3][1024];
-    double s0 = 0, s1 = 0, s2 = 0;
-    for (int64_t j = threadIdx.x; j < N; j += 1024) {
-        s0 += rowv[3 * j];
-        s1 += rowv[3 * j + 1];
-        s2 += rowv[3 * j + 2];
-    }
-    red[0][threadIdx.x] = s0;
-    red[1][threadIdx.x] = s1;
-    red[2][threadIdx.x] = s2;
+// Fixed-order sum of the per-row triples.  CTA b sums its contiguous range of rows into
+// slot b; the CTA that finishes last adds the slots in order (the slots and the order
+// depend on N only, so the result is bitwise reproducible).  (One CTA over all rows took
+// 92 us for 100,000 rows.)
+constexpr int kSumThreads = 256, kSumMax = 128;   // threads per CTA; slots
+
+__device__ __forceinline__ void sum3_block(double (&v)[3], double (*red)[3]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    if (lane == 0)
+        for (int q = 0; q < 3; ++q) red[warp][q] = v[q];
     __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int q = 0; q < 3; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
-        __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < kSumThreads / 32; ++w)
+            for (int q = 0; q < 3; ++q) v[q] += red[w][q];
+}
+
+__global__ void __launch_bounds__(kSumThreads) k_sum_rows3(const double* __restrict__ rowv, int64_t N,
+                                                           int64_t rows_per_cta, double* __restrict__ slots,
+                                                           int* __restrict__ done, double* __restrict__ out3) {
+    __shared__ double red[kSumThreads / 32][3];
+    __shared__ int last;
+    const int64_t j1 = min(N, ((int64_t)blockIdx.x + 1) * rows_per_cta);
+    double v[3] = {0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int64_t j = (int64_t)blockIdx.x * rows_per_cta + threadIdx.x; j < j1; j += kSumThreads)
+        for (int q = 0; q < 3; ++q) v[q] += rowv[3 * j + q];
+    sum3_block(v, red);
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < 3; ++q) slots[3 * blockIdx.x + q] = v[q];
+        __threadfence();
+        last = atomicAdd(done, 1) == (int)gridDim.x - 1;
     }
-    if (threadIdx.x < 3) out3[threadIdx.x] = red[threadIdx.x][0];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x < 3) {
+        double t = 0.0;
+        for (unsigned b = 0; b < gridDim.x; ++b) t += __ldcg(slots + 3 * b + threadIdx.x);
+        out3[threadIdx.x] = t;
+    }
 }
 
 template <int JB, int DREG>
@@ -669,13 +789,15 @@ static int grad_simt_ctas_per_sm() {
 
 // Point splits: the count, among those that leave every CTA at least 8 point
 // tiles, whose CTAs fill the last wave of `slots` resident CTAs best (one CTA
-// per SM for k_grad_tc; the occupancy of k_loo_grad).
+// per SM for k_grad_tc; the occupancy of k_loo_grad).  Where those do not fill
+// the GPU once (small N), shorter splits, down to one tile: N = 2,503, d = 3 ran on 10
+// CTAs (101 us).
 static int64_t grad_splits(int64_t row_ctas, int64_t tiles, int64_t slots) {
-    int64_t best = 1;
+    int64_t best = 1, ctas_before = 0;
     double best_eff = -1.0;
-    for (int64_t ns = 1; ns <= 16; ++ns) {
+    for (int64_t ns = 1; ns <= 64; ++ns) {
         const int64_t per = (tiles + ns - 1) / ns;
-        if (ns > 1 && per < 8) break;
+        if (ns > 1 && (per < 8 || ns > 16) && ctas_before >= slots) break;
         const int64_t n_eff = (tiles + per - 1) / per, ctas = row_ctas * n_eff;
         const int64_t waves = (ctas + slots - 1) / slots;
         const double eff = (double)ctas / (double)(waves * slots);
@@ -683,6 +805,8 @@ static int64_t grad_splits(int64_t row_ctas, int64_t tiles, int64_t slots) {
             best_eff = eff;
             best = ns;
         }
+        ctas_before = ctas;
+        if (per == 1) break;
     }
     return best;
 }
@@ -696,12 +820,15 @@ struct GradChunked {
     GradArgs g;
     bool tc, epan;
     int DREG, DK;
+    int JB;            // rows per thread (SIMT kernel)
     int64_t gx, ns, next_bx;
     int64_t slots;     // resident CTAs of the GPU for this kernel
     double h1, h2;
     double* rowv;
     bool own_rowv;
-    int* fb;
+    double* slots3;    // [kSumMax][3] partial sums of k_sum_rows3
+    int* fb;           // recomputed rows: count, k_sum_rows3's counter, counters per four rows, then the list
+    int64_t fb_list;   // start of the list
 };
 
 int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cudaStream_t st, double* d_rowv_ext,
@@ -724,19 +851,23 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
     c->tc = D.d >= 16;   // tensor-core cross term
     c->DREG = D.d <= 4 ? 4 : D.d <= 8 ? 8 : D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
     c->DK = D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
-    const int JB = c->DREG <= 8 ? 4 : c->DREG <= 32 ? 2 : 1;
-    const int64_t rows_per_cta = c->tc ? (int64_t)kGTRows : (int64_t)kGradThreads * JB;
     const int tile = c->tc ? (c->DK <= 32 ? 256 : 128) : kGradThreads;
-    c->gx = (D.N + rows_per_cta - 1) / rows_per_cta;
     const int64_t tiles = (D.N + tile - 1) / tile;
     int64_t ns;
+    c->JB = 2;
     if (c->tc) {
         c->slots = ctx->sm_count;
     } else {
         const int per_sm = c->DREG == 4 ? grad_simt_ctas_per_sm<4, 4>()
                            : c->DREG == 8 ? grad_simt_ctas_per_sm<4, 8>() : grad_simt_ctas_per_sm<2, 16>();
         c->slots = (int64_t)per_sm * ctx->sm_count;
+        // four rows per thread share a point's loads (d <= 8), unless even one-tile splits
+        // would then leave the GPU part empty
+        const int64_t rows4 = (int64_t)kGradThreads * 4;
+        if (c->DREG <= 8 && (D.N + rows4 - 1) / rows4 * tiles >= c->slots) c->JB = 4;
     }
+    const int64_t rows_per_cta = c->tc ? (int64_t)kGTRows : (int64_t)kGradThreads * c->JB;
+    c->gx = (D.N + rows_per_cta - 1) / rows_per_cta;
     ns = grad_splits(c->gx, tiles, c->slots);
     if (ns > tiles) ns = tiles;
     if (ns < 1) ns = 1;
@@ -751,9 +882,13 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
         rc = cuda_error(e, what);
         return rc;
     };
-    cudaError_t e = cudaMallocAsync((void**)&g.part, (size_t)c->ns * D.N * 6 * sizeof(float), st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&c->fb, (size_t)(D.N + 1) * sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->fb, 0, sizeof(int), st);
+    // (the recomputation reuses the splits' partials, merged by then)
+    const int64_t entries = std::max(c->ns * D.N, c->epan ? 0 : grad_fb_entries(D.N, ctx->sm_count));
+    c->fb_list = 2 + (D.N + kFbRows - 1) / kFbRows;
+    cudaError_t e = cudaMallocAsync((void**)&g.part, (size_t)entries * 6 * sizeof(float), st);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&c->fb, (size_t)(c->fb_list + D.N) * sizeof(int), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->fb, 0, (size_t)c->fb_list * sizeof(int), st);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&c->slots3, (size_t)3 * kSumMax * sizeof(double), st);
     if (e == cudaSuccess && c->own_rowv) e = cudaMallocAsync((void**)&c->rowv, (size_t)D.N * 3 * sizeof(double), st);
     if (e == cudaSuccess && c->tc) {
         uint32_t* xsplit = nullptr;
@@ -784,7 +919,7 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
 // enough row blocks to fill the GPU with their point splits; pair_evals <= 0:
 // all the rest.  *done once every row block has been launched.
 int grad_chunked_next(GradChunked* c, double pair_evals, cudaStream_t st, int* done) {
-    const int64_t rows_per_block = c->tc ? (int64_t)kGTRows : (int64_t)kGradThreads * (c->DREG <= 8 ? 4 : c->DREG <= 32 ? 2 : 1);
+    const int64_t rows_per_block = c->tc ? (int64_t)kGTRows : (int64_t)kGradThreads * c->JB;
     const double per_block = (double)rows_per_block * (double)c->g.N;
     int64_t nb = c->gx - c->next_bx;
     if (pair_evals > 0 && pair_evals < per_block * (double)nb) {
@@ -801,8 +936,10 @@ int grad_chunked_next(GradChunked* c, double pair_evals, cudaStream_t st, int* d
                                      : launch_grad_tc<64>(g, grid, st, c->epan);
         if (rl != CDE_OK) return rl;
     } else {
-        if (c->DREG == 4) launch_grad<4, 4>(g, grid, st, c->epan);
-        else if (c->DREG == 8) launch_grad<4, 8>(g, grid, st, c->epan);
+        if (c->DREG == 4 && c->JB == 4) launch_grad<4, 4>(g, grid, st, c->epan);
+        else if (c->DREG == 4) launch_grad<2, 4>(g, grid, st, c->epan);
+        else if (c->DREG == 8 && c->JB == 4) launch_grad<4, 8>(g, grid, st, c->epan);
+        else if (c->DREG == 8) launch_grad<2, 8>(g, grid, st, c->epan);
         else launch_grad<2, 16>(g, grid, st, c->epan);
     }
     CDE_CUDA(cudaGetLastError());
@@ -815,6 +952,7 @@ void grad_chunked_free(GradChunked* c, cudaStream_t st) {
     if (!c) return;
     if (c->g.part) cudaFreeAsync(c->g.part, st);
     if (c->fb) cudaFreeAsync(c->fb, st);
+    if (c->slots3) cudaFreeAsync(c->slots3, st);
     if (c->g.xsplit) cudaFreeAsync(const_cast<uint32_t*>(c->g.xsplit), st);
     if (c->g.xnorm) cudaFreeAsync(const_cast<float*>(c->g.xnorm), st);
     if (c->own_rowv && c->rowv) cudaFreeAsync(c->rowv, st);
@@ -825,17 +963,25 @@ void grad_chunked_free(GradChunked* c, cudaStream_t st) {
 // rows, and (d_out3) the fixed-order sums; frees the sequence.
 int grad_chunked_finish(cde_ctx* ctx, GradChunked* c, double* d_out3, cudaStream_t st) {
     const GradArgs& g = c->g;
-    k_grad_rows<<<(unsigned)((g.N + 255) / 256), 256, 0, st>>>(g.part, (int)c->ns, g.N, g.my, g.a2, c->h1, c->h2,
-                                                             c->epan ? 1 : 0, epan_log_norm(1), c->rowv, c->fb,
-                                                             c->fb + 1);
+    const double lnk = std::log(c->h2) + (c->epan ? -epan_log_norm(1) : 0.91893853320467274178);
+    // The numerator sum below which a Gaussian row is recomputed with a joint shift: the
+    // exponent arguments of the pairs that carry such a row are over 40, and their FP32
+    // rounding would be over 2^-19 of the sum.  (At 2^(ceil(log2 N) - 91), where factors begin
+    // to flush, the error of an N = 2,503 gradient against 64 bits went from 2.5e-7 to 7e-7.)
+    const double thresh = 0x1p-40;
+    k_grad_rows<<<(unsigned)((g.N + 31) / 32), 256, 0, st>>>(g.part, (int)c->ns, g.N, g.my, g.a2, c->h1, c->h2, lnk,
+                                                             c->epan ? 1 : 0, thresh, c->rowv, c->fb, c->fb + c->fb_list);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && !c->epan) {
         // listed rows only; exits at once when the list is empty
-        k_grad_fallback<<<2 * ctx->sm_count, kFbThreads, 0, st>>>(g, c->fb, c->fb + 1, c->h1, c->h2, c->rowv);
+        k_grad_fallback<<<kFbCtasPerSm * ctx->sm_count, kFbThreads, 0, st>>>(g, c->fb, c->fb + c->fb_list, c->fb + 2, c->h1,
+                                                                             c->h2, c->rowv);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && d_out3) {
-        k_sum_rows3<<<1, 1024, 0, st>>>(c->rowv, g.N, d_out3);
+        const int64_t rpc = std::max<int64_t>((g.N + kSumMax - 1) / kSumMax, kSumThreads);
+        k_sum_rows3<<<(unsigned)((g.N + rpc - 1) / rpc), kSumThreads, 0, st>>>(c->rowv, g.N, rpc, c->slots3, c->fb + 1,
+                                                                              d_out3);
         e = cudaGetLastError();
     }
     grad_chunked_free(c, st);
