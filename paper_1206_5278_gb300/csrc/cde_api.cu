@@ -42,14 +42,12 @@ static int check_grid(const double* h, int G, const char* name) {
     return CDE_OK;
 }
 
-static void free_dataset(Dataset* D) {
-    cudaFree(D->xs);
-    cudaFree(D->y);
-    cudaFree(D->mx);
-    cudaFree(D->my);
-    cudaFree(D->qx);
-    cudaFree(D->qy);
+// (no work that reads the dataset is in flight)
+static void free_dataset(cde_ctx* ctx, Dataset* D) {
+    if (D->mem) cudaFreeAsync(D->mem, ctx->stream);
+    D->mem = nullptr;
     D->xs = D->y = D->mx = D->my = D->qx = D->qy = nullptr;
+    D->stats = nullptr;
 }
 
 __global__ void k_finite_check(const float* a, int64_t n, int* flag) {
@@ -77,6 +75,22 @@ int workspace_reserve(cde_ctx* ctx, size_t dev, size_t host) {
         ctx->ws_host_bytes = host;
     }
     return CDE_OK;
+}
+
+cudaError_t HostCopies::add(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    const size_t off = (used_ + 15) & ~(size_t)15;
+    if (n_ == 4 || off + bytes > kStage || workspace_reserve(ctx_, 0, kStage) != CDE_OK)
+        return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st);
+    const cudaError_t e = cudaMemcpyAsync(static_cast<char*>(ctx_->ws_host) + off, src, bytes, cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) return e;
+    parts_[n_++] = Part{dst, off, bytes};
+    used_ = off + bytes;
+    return cudaSuccess;
+}
+
+void HostCopies::finish() {
+    for (int i = 0; i < n_; ++i) memcpy(parts_[i].dst, static_cast<const char*>(ctx_->ws_host) + parts_[i].off, parts_[i].bytes);
+    n_ = 0;
 }
 }  // namespace cde
 
@@ -123,7 +137,18 @@ int cde_init(cde_ctx** out, int device, size_t budget) {
     e = cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMalloc((void**)&ctx->d_err, 64 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, 64 * sizeof(int));
+    if (e == cudaSuccess) {
+        cudaMemPoolProps pp{};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        pp.location.id = device;
+        e = cudaMemPoolCreate(&ctx->pool, &pp);
+        uint64_t keep = kPoolKeep;
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
     if (e != cudaSuccess) {
+        if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+        if (ctx->d_err) cudaFree(ctx->d_err);
         if (ctx->stream) cudaStreamDestroy(ctx->stream);
         delete ctx;
         return cuda_error(e, "cde_init");
@@ -148,7 +173,7 @@ void cde_shutdown(cde_ctx* ctx) {
     batch_plan_free(ctx);
     {
         std::lock_guard<std::mutex> g(ctx->ds_mu);
-        for (auto& kv : ctx->datasets) free_dataset(kv.second.get());
+        for (auto& kv : ctx->datasets) free_dataset(ctx, kv.second.get());
         ctx->datasets.clear();
     }
     cudaFree(ctx->d_err);
@@ -156,6 +181,8 @@ void cde_shutdown(cde_ctx* ctx) {
     if (ctx->ws_host) cudaFreeHost(ctx->ws_host);
     if (ctx->tev0) cudaEventDestroy(ctx->tev0);
     if (ctx->tev1) cudaEventDestroy(ctx->tev1);
+    cudaStreamSynchronize(ctx->stream);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);   // (frees still pending on callers' streams complete first)
     cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
@@ -187,80 +214,84 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
         return set_error(CDE_ENOMEM, "cde_create_dataset: memory budget exceeded");
     cudaStream_t st = ctx->stream;
     float *dx = nullptr, *dy = nullptr;
-    double* dstats = nullptr;
     int rc = CDE_OK;
     auto fail = [&](int r) {
-        cudaStreamSynchronize(st);
         if (!in_dev) {
-            cudaFree(dx);
-            cudaFree(dy);
+            if (dx) cudaFreeAsync(dx, st);
+            if (dy) cudaFreeAsync(dy, st);
         }
-        cudaFree(dstats);
-        free_dataset(D.get());
+        free_dataset(ctx, D.get());
+        cudaStreamSynchronize(st);
         return r;
     };
-    cudaError_t e = cudaMalloc((void**)&D->xs, (size_t)D->Np * d * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&D->y, (size_t)D->Np * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&D->mx, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&D->my, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&D->qx, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&D->qy, (size_t)N * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&dstats, (size_t)2 * d * sizeof(double) + 64);
-    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: cudaMalloc"));
+    // one allocation: xs, y, mx, my, qx, qy, then the statistics with the word of the finite check
+    const auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t bx = pad((size_t)D->Np * d * 4), by = pad((size_t)D->Np * 4), bn = pad((size_t)N * 4);
+    const size_t stats_bytes = (size_t)2 * d * sizeof(double);
+    cudaError_t e = pool_alloc(ctx, &D->mem, bx + by + 4 * bn + pad(stats_bytes + sizeof(int)), st);
+    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: device memory"));
+    char* m = static_cast<char*>(D->mem);
+    D->xs = reinterpret_cast<float*>(m);
+    D->y = reinterpret_cast<float*>(m += bx);
+    D->mx = reinterpret_cast<float*>(m += by);
+    D->my = reinterpret_cast<float*>(m += bn);
+    D->qx = reinterpret_cast<float*>(m += bn);
+    D->qy = reinterpret_cast<float*>(m += bn);
+    D->stats = reinterpret_cast<double*>(m += bn);
+    int* flag = reinterpret_cast<int*>(m + stats_bytes);
+    // the statistics and the finite check are read back once, at the end (small, page-locked)
+    rc = workspace_reserve(ctx, 0, 2 * kMaxD * sizeof(double) + sizeof(int));
+    if (rc != CDE_OK) return fail(rc);
+    double* stats = static_cast<double*>(ctx->ws_host);
+    for (int c = 0; c < d; ++c) {
+        stats[2 * c] = 0.0;
+        stats[2 * c + 1] = 1.0;
+    }
+    *reinterpret_cast<int*>(stats + 2 * d) = 0;
+    e = cudaMemcpyAsync(D->stats, stats, stats_bytes + sizeof(int), cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: statistics"));
     if (in_dev) {
         dx = const_cast<float*>(x);
         dy = const_cast<float*>(y);
-        int* flag = ctx->d_err + 8;
-        e = cudaMemsetAsync(flag, 0, sizeof(int), st);
-        if (e == cudaSuccess) {
-            k_finite_check<<<256, 256, 0, st>>>(dx, N * d, flag);
-            k_finite_check<<<64, 256, 0, st>>>(dy, N, flag);
-            int h = 0;
-            e = cudaMemcpyAsync(&h, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e == cudaSuccess && h) return fail(set_error(CDE_EINVAL, "cde_create_dataset: non-finite input"));
-        }
+        k_finite_check<<<256, 256, 0, st>>>(dx, N * d, flag);
+        k_finite_check<<<64, 256, 0, st>>>(dy, N, flag);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: finite check"));
     } else {
-        e = cudaMalloc((void**)&dx, (size_t)N * d * 4);
-        if (e == cudaSuccess) e = cudaMalloc((void**)&dy, (size_t)N * 4);
+        e = pool_alloc(ctx, (void**)&dx, (size_t)N * d * 4, st);
+        if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&dy, (size_t)N * 4, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dx, x, (size_t)N * d * 4, cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dy, y, (size_t)N * 4, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: upload"));
     }
-    rc = pack_enqueue(*D, dx, dy, st, dstats);
+    rc = pack_enqueue(*D, dx, dy, st, D->stats);
     if (rc != CDE_OK) return fail(rc);
-    std::vector<double> stats(2 * d, 0.0);
-    if (standardize) {
-        e = cudaMemcpyAsync(stats.data(), dstats, 2 * d * sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: stats"));
+    if (D->kernel == CDE_KERNEL_GAUSS) {
+        rc = nn_shift_enqueue(ctx, *D, st);
+        if (rc != CDE_OK) return fail(rc);
+    } else {
+        e = cudaMemsetAsync(D->mx, 0, 4 * bn, st);   // mx, my, qx, qy
+        if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: shifts"));
+    }
+    e = cudaMemcpyAsync(stats, D->stats, stats_bytes + sizeof(int), cudaMemcpyDeviceToHost, st);
+    cudaError_t e2 = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: kernels"));
+    if (*reinterpret_cast<const int*>(stats + 2 * d))
+        return fail(set_error(CDE_EINVAL, "cde_create_dataset: non-finite input"));
+    if (standardize)
         for (int c = 0; c < d; ++c)
             if (!(stats[2 * c + 1] > 0.0))
                 return fail(set_error(CDE_EINVAL, "cde_create_dataset: zero spread in a dimension"));
-    }
-    if (D->kernel == CDE_KERNEL_GAUSS) {
-        rc = nn_shift_enqueue(*D, st, ctx->sm_count);
-        if (rc != CDE_OK) return fail(rc);
-    } else {
-        e = cudaMemsetAsync(D->mx, 0, (size_t)N * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D->my, 0, (size_t)N * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D->qx, 0, (size_t)N * 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D->qy, 0, (size_t)N * 4, st);
-        if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: shifts"));
-    }
-    e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: kernels"));
     if (!in_dev) {
-        cudaFree(dx);
-        cudaFree(dy);
+        cudaFreeAsync(dx, st);
+        cudaFreeAsync(dy, st);
     }
-    cudaFree(dstats);
     D->mean.resize(d);
     D->sd.resize(d);
     for (int c = 0; c < d; ++c) {
-        D->mean[c] = standardize ? stats[2 * c] : 0.0;
-        D->sd[c] = standardize ? stats[2 * c + 1] : 1.0;
+        D->mean[c] = stats[2 * c];
+        D->sd[c] = stats[2 * c + 1];
     }
     ctx->used += D->bytes;
     {
@@ -287,7 +318,7 @@ int cde_destroy_dataset(cde_ctx* ctx, cde_dataset ds) {
     CDE_CUDA(cudaSetDevice(ctx->device));
     cudaDeviceSynchronize();
     batch_plan_free(ctx);  // a captured batch may reference this dataset
-    free_dataset(D.get());
+    free_dataset(ctx, D.get());
     ctx->used -= D->bytes;
     return CDE_OK;
 }
@@ -425,7 +456,7 @@ int cde_loo_loglik(cde_ctx* ctx, cde_dataset ds, const double* h1, int G1, const
         return CDE_OK;
     }
     double* dbuf = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&dbuf, 2 * n * sizeof(double), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&dbuf, 2 * n * sizeof(double), st));
     rc = loo_grid_enqueue(ctx, *D, h1, G1, h2, G2, nullptr, 0, Lc ? dbuf : nullptr, Le ? dbuf + n : nullptr,
                           nullptr, st);
     cudaError_t e = cudaSuccess;
@@ -458,8 +489,8 @@ int cde_loo_rows(cde_ctx* ctx, cde_dataset ds, const double* h1, int G1, const d
     const size_t n = (size_t)n_rows * G1 * G2;
     int64_t* drows = nullptr;
     double* dell = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&drows, n_rows * sizeof(int64_t), st));
-    CDE_CUDA(cudaMallocAsync((void**)&dell, n * sizeof(double), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&drows, n_rows * sizeof(int64_t), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&dell, n * sizeof(double), st));
     cudaError_t e = cudaMemcpyAsync(drows, rows, n_rows * sizeof(int64_t), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         rc = loo_grid_enqueue(ctx, *D, h1, G1, h2, G2, drows, n_rows, nullptr, nullptr, dell, st);

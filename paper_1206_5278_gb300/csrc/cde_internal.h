@@ -75,6 +75,7 @@ struct Dataset {
     int d = 0;
     int standardized = 0;
     int kernel = 0;        // CDE_KERNEL_GAUSS or CDE_KERNEL_EPAN
+    void* mem = nullptr;   // one allocation of the context's pool holds the arrays below
     float* xs = nullptr;   // [d][Np]
     float* y = nullptr;    // [Np]
     float* mx = nullptr;   // [N] min_{i!=j} |x_j - x_i|^2 (FP32, same formula as the kernels);
@@ -84,7 +85,8 @@ struct Dataset {
     // they bound where the joint minimum of a1 dx^2 + a2 dy^2 can lie):
     float* qx = nullptr;   //     dx^2 to the y-nearest point (the smallest, if several are y-nearest)
     float* qy = nullptr;   //     dy^2 to the x-nearest point (the smallest, if several are x-nearest)
-    std::vector<double> mean, sd;  // per-dimension (identity when not standardised)
+    double* stats = nullptr;       // [d][2] mean, sd per dimension (identity when not standardised)
+    std::vector<double> mean, sd;  // the same on the host
     size_t bytes = 0;
     std::atomic<int> users{0};     // jobs currently reading it (serving)
 };
@@ -104,6 +106,11 @@ struct cde_ctx {
     size_t budget = 0;
     std::atomic<size_t> used{0};
     cudaStream_t stream = nullptr;
+    // stream-ordered pool of every call's scratch and of the datasets.  It keeps up to
+    // kPoolKeep of freed memory across synchronisations (the device's default pool keeps
+    // none, so each call paid to map its scratch again: 300 us of a 370 us density request)
+    // and is destroyed at shutdown.
+    cudaMemPool_t pool = nullptr;
     std::recursive_mutex mu;  // serialises the synchronous API
     std::mutex ds_mu;         // guards the dataset map
     std::map<int64_t, std::shared_ptr<cde::Dataset>> datasets;
@@ -169,6 +176,12 @@ inline void timing_end(cde_ctx* c, cudaStream_t st) {
 
 std::shared_ptr<Dataset> find_dataset(cde_ctx* ctx, cde_dataset ds);
 
+// Device memory of the context's pool, stream-ordered on `st` (freed by cudaFreeAsync)
+constexpr uint64_t kPoolKeep = (uint64_t)256 << 20;
+inline cudaError_t pool_alloc(cde_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
+    return cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+}
+
 // ln c_d of the radial Epanechnikov kernel in d dimensions (loo_grid.cu)
 double epan_log_norm(int d);
 cudaStream_t pick_stream(cde_ctx* ctx, void* s);
@@ -207,8 +220,30 @@ constexpr size_t kWorkspaceMax = (size_t)64 << 20;
 // (synchronous growth; callers hold ctx->mu and no work of theirs is in flight).
 int workspace_reserve(cde_ctx* ctx, size_t dev, size_t host);
 
+// Device -> host copies of a synchronous call (the caller holds ctx->mu): small ones
+// land in the pinned workspace, so that the call waits for its stream once, and are
+// handed over by finish() after the caller's synchronisation; others go straight to the
+// caller's memory.
+class HostCopies {
+  public:
+    explicit HostCopies(cde_ctx* ctx) : ctx_(ctx) {}
+    cudaError_t add(void* dst, const void* src, size_t bytes, cudaStream_t st);
+    void finish();
+
+  private:
+    static constexpr size_t kStage = (size_t)256 << 10;
+    struct Part {
+        void* dst;
+        size_t off, bytes;
+    };
+    cde_ctx* ctx_;
+    Part parts_[4];
+    int n_ = 0;
+    size_t used_ = 0;
+};
+
 // Nearest squared distances per row (cached at dataset creation).
-int nn_shift_enqueue(const Dataset& D, cudaStream_t st, int sm_count);
+int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st);
 
 // Standardise / pack raw row-major x into the SoA layout (device input).
 int pack_enqueue(Dataset& D, const float* d_x_rowmajor, const float* d_y, cudaStream_t st,

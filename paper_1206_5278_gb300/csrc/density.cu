@@ -53,12 +53,11 @@ __device__ __forceinline__ float fma_sat_d(float a, float b, float c) {
 }
 
 __global__ void k_query_pack(const float* __restrict__ xq, int64_t Q, int64_t Qp, int d,
-                             const double* __restrict__ mean, const double* __restrict__ sd,
-                             float* __restrict__ out) {
+                             const double* __restrict__ stats, float* __restrict__ out) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= Qp) return;
     for (int c = 0; c < d; ++c)
-        out[(int64_t)c * Qp + q] = q < Q ? (float)(((double)xq[q * d + c] - mean[c]) / sd[c]) : 0.f;
+        out[(int64_t)c * Qp + q] = q < Q ? (float)(((double)xq[q * d + c] - stats[2 * c]) / stats[2 * c + 1]) : 0.f;
 }
 
 // per-query nearest squared distance to the data (same FP32 formula as the
@@ -628,13 +627,9 @@ int density_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, const 
     if (Q == 0) return CDE_OK;
     const int64_t Qp = (Q + kTcM - 1) / kTcM * kTcM;
     float *xq = nullptr, *mq = nullptr, *part = nullptr, *dpart = nullptr;
-    double* stats = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&xq, (size_t)Qp * D.d * sizeof(float), st));
-    CDE_CUDA(cudaMallocAsync((void**)&mq, (size_t)Q * sizeof(float), st));
-    CDE_CUDA(cudaMallocAsync((void**)&stats, (size_t)2 * D.d * sizeof(double), st));
-    CDE_CUDA(cudaMemcpyAsync(stats, D.mean.data(), D.d * sizeof(double), cudaMemcpyHostToDevice, st));
-    CDE_CUDA(cudaMemcpyAsync(stats + D.d, D.sd.data(), D.d * sizeof(double), cudaMemcpyHostToDevice, st));
-    k_query_pack<<<(unsigned)((Qp + 255) / 256), 256, 0, st>>>(d_xq, Q, Qp, D.d, stats, stats + D.d, xq);
+    CDE_CUDA(pool_alloc(ctx, (void**)&xq, (size_t)Qp * D.d * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&mq, (size_t)Q * sizeof(float), st));
+    k_query_pack<<<(unsigned)((Qp + 255) / 256), 256, 0, st>>>(d_xq, Q, Qp, D.d, D.stats, xq);
     CDE_CUDA(cudaGetLastError());
     const bool epan = D.kernel == CDE_KERNEL_EPAN;
     if (!epan) {
@@ -662,8 +657,8 @@ int density_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, const 
     a.P = (int)std::min<int64_t>(ctx->sm_count, a.U);
     a.MT = (int)(((a.U + a.P - 1) / a.P + a.C - 1) / a.C + 1);
     a.err = ctx->d_err + kErrTensorWait;
-    CDE_CUDA(cudaMallocAsync((void**)&part, (size_t)a.P * a.MT * kTcM * kTcN * sizeof(float), st));
-    CDE_CUDA(cudaMallocAsync((void**)&dpart, (size_t)a.P * a.MT * kTcM * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&part, (size_t)a.P * a.MT * kTcM * kTcN * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&dpart, (size_t)a.P * a.MT * kTcM * sizeof(float), st));
     a.part = part;
     a.dpart = dpart;
     static std::atomic<uint64_t> attr0{0}, attr1{0};
@@ -683,7 +678,6 @@ int density_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, const 
     CDE_CUDA(cudaGetLastError());
     cudaFreeAsync(xq, st);
     cudaFreeAsync(mq, st);
-    cudaFreeAsync(stats, st);
     cudaFreeAsync(part, st);
     cudaFreeAsync(dpart, st);
     return CDE_OK;
@@ -748,29 +742,23 @@ extern "C" int cde_density(cde_ctx* ctx, cde_dataset ds, double h1, double h2, c
             if (!std::isfinite(xq[e])) return set_error(CDE_EINVAL, "cde_density: non-finite query");
         for (int g = 0; g < G; ++g)
             if (!std::isfinite(ygrid[g])) return set_error(CDE_EINVAL, "cde_density: non-finite y grid");
-        CDE_CUDA(cudaMallocAsync((void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
-        CDE_CUDA(cudaMallocAsync((void**)&dyg, (size_t)G * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dyg, (size_t)G * sizeof(float), st));
         CDE_CUDA(cudaMemcpyAsync(dxq, xq, (size_t)Q * D->d * sizeof(float), cudaMemcpyHostToDevice, st));
         CDE_CUDA(cudaMemcpyAsync(dyg, ygrid, (size_t)G * sizeof(float), cudaMemcpyHostToDevice, st));
         dq = dxq;
         dg = dyg;
     }
+    int tw = 0;   // the device-wait word
+    HostCopies out(ctx);
     if (!out_dev) {
-        const int rw = workspace_reserve(ctx, 0, 64);
-        if (rw != CDE_OK) {
-            if (dxq) cudaFreeAsync(dxq, st);
-            if (dyg) cudaFreeAsync(dyg, st);
-            return rw;
-        }
-        CDE_CUDA(cudaMallocAsync((void**)&df, (size_t)Q * G * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&df, (size_t)Q * G * sizeof(float), st));
     }
     int rc = density_enqueue(ctx, *D, h1, h2, dq, Q, dg, G, df, st);
     cudaError_t e = cudaSuccess;
-    int* tw_host = static_cast<int*>(ctx->ws_host);   // pinned; the context lock is held
     if (rc == CDE_OK && !out_dev) {
-        e = cudaMemcpyAsync(f_out, df, (size_t)Q * G * sizeof(float), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && tw_host)
-            e = cudaMemcpyAsync(tw_host, ctx->d_err + kErrTensorWait, sizeof(int), cudaMemcpyDeviceToHost, st);
+        e = out.add(&tw, ctx->d_err + kErrTensorWait, sizeof(int), st);
+        if (e == cudaSuccess) e = out.add(f_out, df, (size_t)Q * G * sizeof(float), st);
     }
     if (dxq) cudaFreeAsync(dxq, st);
     if (dyg) cudaFreeAsync(dyg, st);
@@ -781,7 +769,8 @@ extern "C" int cde_density(cde_ctx* ctx, cde_dataset ds, double h1, double h2, c
     }
     if (rc != CDE_OK) return rc;
     if (e != cudaSuccess) return cuda_error(e, "cde_density: copy");
-    if (!out_dev && tw_host && *tw_host) {
+    out.finish();
+    if (tw) {
         cudaMemsetAsync(ctx->d_err + kErrTensorWait, 0, sizeof(int), st);
         return set_error(CDE_ETIMEOUT, "cde_density: a tensor-core wait ran out on the device");
     }

@@ -885,16 +885,16 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
     // (the recomputation reuses the splits' partials, merged by then)
     const int64_t entries = std::max(c->ns * D.N, c->epan ? 0 : grad_fb_entries(D.N, ctx->sm_count));
     c->fb_list = 2 + (D.N + kFbRows - 1) / kFbRows;
-    cudaError_t e = cudaMallocAsync((void**)&g.part, (size_t)entries * 6 * sizeof(float), st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&c->fb, (size_t)(c->fb_list + D.N) * sizeof(int), st);
+    cudaError_t e = pool_alloc(ctx, (void**)&g.part, (size_t)entries * 6 * sizeof(float), st);
+    if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&c->fb, (size_t)(c->fb_list + D.N) * sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->fb, 0, (size_t)c->fb_list * sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&c->slots3, (size_t)3 * kSumMax * sizeof(double), st);
-    if (e == cudaSuccess && c->own_rowv) e = cudaMallocAsync((void**)&c->rowv, (size_t)D.N * 3 * sizeof(double), st);
+    if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&c->slots3, (size_t)3 * kSumMax * sizeof(double), st);
+    if (e == cudaSuccess && c->own_rowv) e = pool_alloc(ctx, (void**)&c->rowv, (size_t)D.N * 3 * sizeof(double), st);
     if (e == cudaSuccess && c->tc) {
         uint32_t* xsplit = nullptr;
         float* xnorm = nullptr;
-        e = cudaMallocAsync((void**)&xsplit, (size_t)2 * D.Np * c->DK * sizeof(uint32_t), st);
-        if (e == cudaSuccess) e = cudaMallocAsync((void**)&xnorm, (size_t)D.Np * sizeof(float), st);
+        e = pool_alloc(ctx, (void**)&xsplit, (size_t)2 * D.Np * c->DK * sizeof(uint32_t), st);
+        if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&xnorm, (size_t)D.Np * sizeof(float), st);
         g.xsplit = xsplit;
         g.xnorm = xnorm;
         g.err = ctx->d_err + kErrTensorWait;
@@ -1014,13 +1014,16 @@ CDE_CHECK_READER(check_status_grad)
 
 using namespace cde;
 
-// After a synchronous d >= 16 call: a bounded tensor-core wait that ran out on
+// A synchronous call's copies back: the result and, at d >= 16, the device-wait word
+static cudaError_t grad_copy_back(cde_ctx* ctx, const Dataset& D, HostCopies& out, void* dst, const void* src,
+                                  size_t bytes, int* tw, cudaStream_t st) {
+    cudaError_t e = D.d >= 16 ? out.add(tw, ctx->d_err + kErrTensorWait, sizeof(int), st) : cudaSuccess;
+    return e == cudaSuccess ? out.add(dst, src, bytes, st) : e;
+}
+
+// After a synchronous call: a bounded tensor-core wait that ran out on
 // the device (k_grad_tc) becomes CDE_ETIMEOUT, and the report is cleared.
-static int grad_wait_status(cde_ctx* ctx, const Dataset& D, cudaStream_t st, const char* who) {
-    if (D.d < 16) return CDE_OK;
-    int tw = 0;
-    CDE_CUDA(cudaMemcpyAsync(&tw, ctx->d_err + kErrTensorWait, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CDE_CUDA(cudaStreamSynchronize(st));
+static int grad_wait_status(cde_ctx* ctx, int tw, cudaStream_t st, const char* who) {
     if (!tw) return CDE_OK;
     CDE_CUDA(cudaMemsetAsync(ctx->d_err + kErrTensorWait, 0, sizeof(int), st));
     return set_error(CDE_ETIMEOUT, std::string(who) + ": a tensor-core wait ran out on the device");
@@ -1039,16 +1042,19 @@ extern "C" int cde_loo_grad(cde_ctx* ctx, cde_dataset ds, double h1, double h2, 
     cudaStream_t st = pick_stream(ctx, stream);
     if (flags & CDE_OUT_DEVICE) return loo_grad_enqueue(ctx, *D, h1, h2, out3, st, nullptr);
     double* dout = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&dout, 3 * sizeof(double), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&dout, 3 * sizeof(double), st));
     int rc = loo_grad_enqueue(ctx, *D, h1, h2, dout, st, nullptr);
     cudaError_t e = cudaSuccess;
-    if (rc == CDE_OK) e = cudaMemcpyAsync(out3, dout, 3 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    int tw = 0;
+    HostCopies out(ctx);
+    if (rc == CDE_OK) e = grad_copy_back(ctx, *D, out, out3, dout, 3 * sizeof(double), &tw, st);
     cudaFreeAsync(dout, st);
     cudaError_t e2 = cudaStreamSynchronize(st);
     if (rc != CDE_OK) return rc;
     if (e != cudaSuccess) return cuda_error(e, "cde_loo_grad: copy");
     if (e2 != cudaSuccess) return cuda_error(e2, "cde_loo_grad: kernels");
-    return grad_wait_status(ctx, *D, st, "cde_loo_grad");
+    out.finish();
+    return grad_wait_status(ctx, tw, st, "cde_loo_grad");
 }
 
 extern "C" int cde_loo_grad_rows(cde_ctx* ctx, cde_dataset ds, double h1, double h2, double* rows_out,
@@ -1063,15 +1069,17 @@ extern "C" int cde_loo_grad_rows(cde_ctx* ctx, cde_dataset ds, double h1, double
     CDE_CUDA(cudaSetDevice(ctx->device));
     cudaStream_t st = pick_stream(ctx, stream);
     double* rowv = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&rowv, (size_t)D->N * 3 * sizeof(double), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&rowv, (size_t)D->N * 3 * sizeof(double), st));
     int rc = loo_grad_enqueue(ctx, *D, h1, h2, nullptr, st, rowv);
     cudaError_t e = cudaSuccess;
-    if (rc == CDE_OK)
-        e = cudaMemcpyAsync(rows_out, rowv, (size_t)D->N * 3 * sizeof(double), cudaMemcpyDeviceToHost, st);
+    int tw = 0;
+    HostCopies out(ctx);
+    if (rc == CDE_OK) e = grad_copy_back(ctx, *D, out, rows_out, rowv, (size_t)D->N * 3 * sizeof(double), &tw, st);
     cudaFreeAsync(rowv, st);
     cudaError_t e2 = cudaStreamSynchronize(st);
     if (rc != CDE_OK) return rc;
     if (e != cudaSuccess) return cuda_error(e, "cde_loo_grad_rows: copy");
     if (e2 != cudaSuccess) return cuda_error(e2, "cde_loo_grad_rows: kernels");
-    return grad_wait_status(ctx, *D, st, "cde_loo_grad_rows");
+    out.finish();
+    return grad_wait_status(ctx, tw, st, "cde_loo_grad_rows");
 }

@@ -308,9 +308,10 @@ __global__ void k_nn_unpack(const unsigned long long* __restrict__ kx, const uns
     qx[j] = __uint_as_float((unsigned int)b);
 }
 
-int nn_shift_enqueue(const Dataset& D, cudaStream_t st, int sm_count) {
+int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st) {
+    const int sm_count = ctx->sm_count;
     unsigned long long* keys = nullptr;   // [2][N] merge keys, stream-ordered scratch
-    CDE_CUDA(cudaMallocAsync((void**)&keys, (size_t)2 * D.N * sizeof(unsigned long long), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&keys, (size_t)2 * D.N * sizeof(unsigned long long), st));
     // d <= 8: 0x7f bytes, the first word 3.4e38; d > 8: 0xff bytes, above infinity (a row
     // whose every distance overflows keeps an infinite shift)
     CDE_CUDA(cudaMemsetAsync(keys, D.d <= 8 ? 0x7f : 0xff, (size_t)2 * D.N * sizeof(unsigned long long), st));
@@ -579,7 +580,7 @@ int loo_grid_enqueue(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, c
             a.G2r = g2;
             double* part = nullptr;
             const bool own = !(scratch && pl.bytes() <= scratch_bytes);
-            if (own) CDE_CUDA(cudaMallocAsync((void**)&part, pl.bytes(), st));
+            if (own) CDE_CUDA(pool_alloc(ctx, (void**)&part, pl.bytes(), st));
             else part = static_cast<double*>(scratch);
             a.part = part;
             a.fb = reinterpret_cast<double*>(reinterpret_cast<char*>(part) + pl.part_bytes);

@@ -38,8 +38,7 @@
 namespace cde {
 
 __global__ void k_query_pack(const float* __restrict__ xq, int64_t Q, int64_t Qp, int d,
-                             const double* __restrict__ mean, const double* __restrict__ sd,
-                             float* __restrict__ out);
+                             const double* __restrict__ stats, float* __restrict__ out);
 
 __device__ __forceinline__ float ex2p(float x) {
     float r;
@@ -573,19 +572,14 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
 static int prep_queries(cde_ctx* ctx, const Dataset& D, const float* d_xq, int64_t Q, int64_t Qp,
                         float** xq_out, float** mq_out, cudaStream_t st) {
     float *xq = nullptr, *mq = nullptr;
-    double* stats = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&xq, (size_t)Qp * D.d * sizeof(float), st));
-    CDE_CUDA(cudaMallocAsync((void**)&mq, (size_t)Q * sizeof(float), st));
-    CDE_CUDA(cudaMallocAsync((void**)&stats, (size_t)2 * D.d * sizeof(double), st));
-    CDE_CUDA(cudaMemcpyAsync(stats, D.mean.data(), D.d * sizeof(double), cudaMemcpyHostToDevice, st));
-    CDE_CUDA(cudaMemcpyAsync(stats + D.d, D.sd.data(), D.d * sizeof(double), cudaMemcpyHostToDevice, st));
-    k_query_pack<<<(unsigned)((Qp + 255) / 256), 256, 0, st>>>(d_xq, Q, Qp, D.d, stats, stats + D.d, xq);
+    CDE_CUDA(pool_alloc(ctx, (void**)&xq, (size_t)Qp * D.d * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&mq, (size_t)Q * sizeof(float), st));
+    k_query_pack<<<(unsigned)((Qp + 255) / 256), 256, 0, st>>>(d_xq, Q, Qp, D.d, D.stats, xq);
     CDE_CUDA(cudaGetLastError());
     if (D.kernel == CDE_KERNEL_GAUSS) {
         const int rc = query_shift_enqueue(ctx->sm_count, D, xq, Q, Qp, mq, st);
         if (rc != CDE_OK) return rc;
     }
-    CDE_CUDA(cudaFreeAsync(stats, st));
     *xq_out = xq;
     *mq_out = mq;
     return CDE_OK;
@@ -642,7 +636,7 @@ static int cond_stats_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double 
     const int64_t tps = (tiles + ns - 1) / ns;
     ns = (tiles + tps - 1) / tps;
     a.i_per_split = tps * kCSThreads;
-    CDE_CUDA(cudaMallocAsync((void**)&part, (size_t)ns * Q * 3 * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&part, (size_t)ns * Q * 3 * sizeof(float), st));
     a.part = part;
     const dim3 grid((unsigned)gx, (unsigned)ns);
     timing_begin(ctx, st);
@@ -699,7 +693,7 @@ static int cond_interval_enqueue(cde_ctx* ctx, const Dataset& D, double h1, doub
     // queries in batches whose chunk totals fit 64 MB (at least 128)
     const int64_t qmax = std::max<int64_t>(kCwQ, ((int64_t)16 << 20) / a.n_chunks / kCwQ * kCwQ);
     const int64_t qbatch = std::min(Q, qmax);
-    CDE_CUDA(cudaMallocAsync((void**)&a.ct, (size_t)(a.n_chunks * qbatch) * sizeof(float), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&a.ct, (size_t)(a.n_chunks * qbatch) * sizeof(float), st));
     for (int64_t q0 = 0; q0 < Q; q0 += qbatch) {
         a.q0 = q0;
         a.nq = std::min(qbatch, Q - q0);
@@ -759,25 +753,25 @@ extern "C" int cde_cond_stats(cde_ctx* ctx, cde_dataset ds, double h1, double h2
     if (!in_dev) {
         for (int64_t e = 0; e < Q * D->d; ++e)
             if (!std::isfinite(xq[e])) return set_error(CDE_EINVAL, "cde_cond_stats: non-finite query");
-        CDE_CUDA(cudaMallocAsync((void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
         CDE_CUDA(cudaMemcpyAsync(dxq, xq, (size_t)Q * D->d * sizeof(float), cudaMemcpyHostToDevice, st));
         dq = dxq;
         if (yq) {
-            CDE_CUDA(cudaMallocAsync((void**)&dyq, (size_t)Q * sizeof(float), st));
+            CDE_CUDA(pool_alloc(ctx, (void**)&dyq, (size_t)Q * sizeof(float), st));
             CDE_CUDA(cudaMemcpyAsync(dyq, yq, (size_t)Q * sizeof(float), cudaMemcpyHostToDevice, st));
             dy = dyq;
         }
     }
     if (!out_dev) {
-        if (mean_out) CDE_CUDA(cudaMallocAsync((void**)&dmean, (size_t)Q * sizeof(double), st));
-        if (fat_out) CDE_CUDA(cudaMallocAsync((void**)&dfat, (size_t)Q * sizeof(double), st));
+        if (mean_out) CDE_CUDA(pool_alloc(ctx, (void**)&dmean, (size_t)Q * sizeof(double), st));
+        if (fat_out) CDE_CUDA(pool_alloc(ctx, (void**)&dfat, (size_t)Q * sizeof(double), st));
     }
+    HostCopies out(ctx);
     rc = cond_stats_enqueue(ctx, *D, h1, h2, dq, fat_out ? dy : nullptr, Q, dmean, dfat, st);
     cudaError_t e = cudaSuccess;
     if (rc == CDE_OK && !out_dev) {
-        if (mean_out) e = cudaMemcpyAsync(mean_out, dmean, (size_t)Q * sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && fat_out)
-            e = cudaMemcpyAsync(fat_out, dfat, (size_t)Q * sizeof(double), cudaMemcpyDeviceToHost, st);
+        if (mean_out) e = out.add(mean_out, dmean, (size_t)Q * sizeof(double), st);
+        if (e == cudaSuccess && fat_out) e = out.add(fat_out, dfat, (size_t)Q * sizeof(double), st);
     }
     if (dxq) cudaFreeAsync(dxq, st);
     if (dyq) cudaFreeAsync(dyq, st);
@@ -789,6 +783,7 @@ extern "C" int cde_cond_stats(cde_ctx* ctx, cde_dataset ds, double h1, double h2
     }
     if (rc != CDE_OK) return rc;
     if (e != cudaSuccess) return cuda_error(e, "cde_cond_stats");
+    out.finish();
     return CDE_OK;
 }
 
@@ -816,22 +811,22 @@ extern "C" int cde_cond_interval(cde_ctx* ctx, cde_dataset ds, double h1, double
     if (!in_dev) {
         for (int64_t e = 0; e < Q * D->d; ++e)
             if (!std::isfinite(xq[e])) return set_error(CDE_EINVAL, "cde_cond_interval: non-finite query");
-        CDE_CUDA(cudaMallocAsync((void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dxq, (size_t)Q * D->d * sizeof(float), st));
         CDE_CUDA(cudaMemcpyAsync(dxq, xq, (size_t)Q * D->d * sizeof(float), cudaMemcpyHostToDevice, st));
         dq = dxq;
     }
     if (!out_dev) {
-        CDE_CUDA(cudaMallocAsync((void**)&dlo, (size_t)Q * sizeof(float), st));
-        CDE_CUDA(cudaMallocAsync((void**)&dhi, (size_t)Q * sizeof(float), st));
-        if (samples_out) CDE_CUDA(cudaMallocAsync((void**)&dsm, (size_t)Q * S * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dlo, (size_t)Q * sizeof(float), st));
+        CDE_CUDA(pool_alloc(ctx, (void**)&dhi, (size_t)Q * sizeof(float), st));
+        if (samples_out) CDE_CUDA(pool_alloc(ctx, (void**)&dsm, (size_t)Q * S * sizeof(float), st));
     }
+    HostCopies out(ctx);
     rc = cond_interval_enqueue(ctx, *D, h1, h2, dq, Q, S, alpha, seed, dlo, dhi, dsm, st);
     cudaError_t e = cudaSuccess;
     if (rc == CDE_OK && !out_dev) {
-        e = cudaMemcpyAsync(lo_out, dlo, (size_t)Q * sizeof(float), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(hi_out, dhi, (size_t)Q * sizeof(float), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess && samples_out)
-            e = cudaMemcpyAsync(samples_out, dsm, (size_t)Q * S * sizeof(float), cudaMemcpyDeviceToHost, st);
+        e = out.add(lo_out, dlo, (size_t)Q * sizeof(float), st);
+        if (e == cudaSuccess) e = out.add(hi_out, dhi, (size_t)Q * sizeof(float), st);
+        if (e == cudaSuccess && samples_out) e = out.add(samples_out, dsm, (size_t)Q * S * sizeof(float), st);
     }
     if (dxq) cudaFreeAsync(dxq, st);
     if (!out_dev) {
@@ -843,5 +838,6 @@ extern "C" int cde_cond_interval(cde_ctx* ctx, cde_dataset ds, double h1, double
     }
     if (rc != CDE_OK) return rc;
     if (e != cudaSuccess) return cuda_error(e, "cde_cond_interval");
+    out.finish();
     return CDE_OK;
 }

@@ -70,7 +70,7 @@ extern "C" int cde_reference_rule(cde_ctx* ctx, cde_dataset ds, double* h1, doub
     cudaStream_t st = ctx->stream;
     const int d = D->d;
     double* dstats = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&dstats, (size_t)2 * (d + 1) * sizeof(double), st));
+    CDE_CUDA(pool_alloc(ctx, (void**)&dstats, (size_t)2 * (d + 1) * sizeof(double), st));
     // column statistics of the stored (possibly standardised) x and of y
     for (int c = 0; c <= d; ++c) {
         const float* col = c < d ? D->xs + (int64_t)c * D->Np : D->y;
@@ -113,11 +113,12 @@ extern "C" int cde_select_random(cde_ctx* ctx, cde_dataset ds, double h1_max, do
     const int GG = G1 * G2;
     double* dout = nullptr;
     double* hout = nullptr;
-    CDE_CUDA(cudaMallocAsync((void**)&dout, (size_t)2 * GG * sizeof(double), st));
-    if (cudaMallocHost((void**)&hout, (size_t)2 * GG * sizeof(double)) != cudaSuccess) {
+    CDE_CUDA(pool_alloc(ctx, (void**)&dout, (size_t)2 * GG * sizeof(double), st));
+    if (workspace_reserve(ctx, 0, (size_t)2 * GG * sizeof(double)) != CDE_OK) {
         cudaFreeAsync(dout, st);
         return set_error(CDE_ENOMEM, "cde_select_random: pinned buffer");
     }
+    hout = static_cast<double*>(ctx->ws_host);   // (the context lock is held)
     std::vector<double> h1(G1), h2(G2);
     bool have = false;
     double bv = -INFINITY;
@@ -152,7 +153,6 @@ extern "C" int cde_select_random(cde_ctx* ctx, cde_dataset ds, double h1_max, do
     }
     cudaFreeAsync(dout, st);
     cudaStreamSynchronize(st);
-    cudaFreeHost(hout);
     if (rc != CDE_OK) return rc;
     if (!have) {
         best[0] = best[1] = NAN;

@@ -173,9 +173,9 @@ static int advance(Server& S, Job& J) {
         J.h_f = J.h_in + nq + r.G_y;
         memcpy(J.h_in, r.xq, nq * sizeof(float));
         memcpy(J.h_in + nq, r.ygrid, r.G_y * sizeof(float));
-        CDE_CUDA(cudaMallocAsync((void**)&J.d_xq, (nq + r.G_y) * sizeof(float), st));
+        CDE_CUDA(pool_alloc(S.ctx, (void**)&J.d_xq, (nq + r.G_y) * sizeof(float), st));
         J.d_yg = J.d_xq + nq;
-        CDE_CUDA(cudaMallocAsync((void**)&J.d_f, std::max<size_t>(nf, 1) * sizeof(float), st));
+        CDE_CUDA(pool_alloc(S.ctx, (void**)&J.d_f, std::max<size_t>(nf, 1) * sizeof(float), st));
         CDE_CUDA(cudaMemcpyAsync(J.d_xq, J.h_in, (nq + r.G_y) * sizeof(float), cudaMemcpyHostToDevice, st));
         int rc = density_enqueue(S.ctx, D, r.h1, r.h2, J.d_xq, r.Q, J.d_yg, r.G_y, J.d_f, st);
         if (rc != CDE_OK) return rc;
@@ -187,12 +187,12 @@ static int advance(Server& S, Job& J) {
             int prc = slot_pinned(S, J.slot, (g + 4) * sizeof(double), &pb);
             if (prc != CDE_OK) return prc;
             J.h_small = reinterpret_cast<double*>(pb);
-            CDE_CUDA(cudaMallocAsync((void**)&J.d_small, (g + 4) * sizeof(double), st));
+            CDE_CUDA(pool_alloc(S.ctx, (void**)&J.d_small, (g + 4) * sizeof(double), st));
             J.grid_init = true;
             if (r.G1 <= 32 && r.G2 <= 32) {
                 int rc = loo_chunked_create(S.ctx, D, r.h1_grid, r.G1, r.h2_grid, r.G2, &J.gc);
                 if (rc != CDE_OK) return rc;
-                CDE_CUDA(cudaMallocAsync(&J.d_grid, loo_chunked_scratch_bytes(J.gc), st));
+                CDE_CUDA(pool_alloc(S.ctx, &J.d_grid, loo_chunked_scratch_bytes(J.gc), st));
             } else {
                 // wider grids: one enqueue of all its blocks
                 int rc = loo_grid_enqueue(S.ctx, D, r.h1_grid, r.G1, r.h2_grid, r.G2, nullptr, 0, J.d_small,
