@@ -62,29 +62,29 @@ __global__ void __launch_bounds__(256, 2) k_loo_batch(const LooArgs* __restrict_
     }
 }
 
-// one warp per (item, cell); same reduction as the single launch
-__global__ void k_loo_final_batch(const LooArgs* __restrict__ items, const int* __restrict__ item_cell0,
-                                  int n_items, int GG, int G2T, const int64_t* __restrict__ out_off,
-                                  double* __restrict__ out) {
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    // locate the item: cells are numbered item-major
+// one CTA per four cells of an item; same reduction as the single launch
+__global__ void __launch_bounds__(kFinalThreads) k_loo_final_batch(const LooArgs* __restrict__ items,
+                                                                   const int* __restrict__ item_cell0, int n_items,
+                                                                   int GG, int G2T, const int64_t* __restrict__ out_off,
+                                                                   double* __restrict__ out) {
+    const int gc = kFinalCells * blockIdx.x;
+    // locate the item: cells are numbered item-major (a multiple of four each)
     int lo = 0, hi = n_items;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (item_cell0[mid] <= gw) lo = mid;
+        if (item_cell0[mid] <= gc) lo = mid;
         else hi = mid;
     }
-    if (gw >= item_cell0[n_items]) return;
-    const int it = lo, cell = gw - item_cell0[it];
+    const int it = lo;
     const LooArgs& a = items[it];
     double sc, se;
-    loo_final_cell(a.part, a.n_tiles, GG, cell, lane, sc, se);
-    const int k = cell / G2T, l = cell % G2T;
-    if (lane == 0 && k < a.G1r && l < a.G2r) {
+    loo_final_cells(a.part, a.n_tiles, GG, gc - item_cell0[it], sc, se);
+    const int cell = gc - item_cell0[it] + threadIdx.x, k = cell / G2T, l = cell % G2T;
+    if (threadIdx.x < kFinalCells && k < a.G1r && l < a.G2r) {
         const int n = a.G1r * a.G2r;
         double* o = out + out_off[it];
         o[k * a.G2r + l] = sc;
-        o[n + k * a.G2r + l] = se / (double)a.N - log((double)a.N - 1.0);
+        o[n + k * a.G2r + l] = se / (double)a.N - a.logn1;
     }
 }
 
@@ -282,7 +282,7 @@ static int build_plan(cde_ctx* ctx, const std::vector<BatchItem>& items, BatchPl
         if (rc != CDE_OK) break;
         const int GG = T1 * T2;
         const int cells = cell0[s][n];
-        k_loo_final_batch<<<(cells * 32 + 255) / 256, 256, 0, st>>>(
+        k_loo_final_batch<<<cells / kFinalCells, kFinalThreads, 0, st>>>(
             d_items, d_cell0 + (size_t)s * (n + 1), n, GG, T2, d_ooff, d_out);
         e = cudaGetLastError();
         P.kernel_launches += 2;

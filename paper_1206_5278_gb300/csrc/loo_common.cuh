@@ -39,6 +39,7 @@ struct LooArgs {
     int* work;              // batched launch: queue counter
     int kern;               // CDE_KERNEL_GAUSS or CDE_KERNEL_EPAN
     float thresh;           // cells with shifted numerator below this are recomputed
+    double logn1;           // ln(N - 1)
     // per-bandwidth coefficients, padded by repeating the last bandwidth:
     //   Gaussian:     a = log2(e)/(2 h^2), lam1 = d ln(sqrt(2 pi) h1), kap2 = ln(sqrt(2 pi) h2)
     //   Epanechnikov: a = 1/h^2,           lam1 = d ln h1 - ln c_d,     kap2 = ln h2 - ln c_1
@@ -82,21 +83,42 @@ __device__ __forceinline__ double log2_wide(float v) {
     return (double)(e - 1) + (double)log2f(2.0f * m);
 }
 
-// Fixed-order reduction of one grid cell over tile partials (one warp):
-// lane t sums tiles t, t+32, ... in order, then a fixed xor tree.
-__device__ __forceinline__ void loo_final_cell(const double* __restrict__ part, int n_tiles, int GG,
-                                               int cell, int lane, double& sc, double& se) {
+// Fixed-order reduction of four adjacent grid cells over the tile partials (a CTA
+// of 256 threads): thread (cell q = tid % 4, t = tid / 4) sums tiles t, t + 64, ... in
+// order, then a fixed tree over t.  The four cells are one 32-byte sector of every
+// slot.  Returns with the sums in the threads tid < 4.  (One warp per cell, reading a
+// sector per slot and cell: 28 us for the 3,001 slots of a 4 x 4 grid, 11 us for the
+// 250 of an 8 x 8 grid.)
+constexpr int kFinalThreads = 256, kFinalCells = 4;
+
+__device__ __forceinline__ void loo_final_cells(const double* __restrict__ part, int n_tiles, int GG, int cell0,
+                                                double& sc, double& se) {
+    __shared__ double rc[kFinalThreads / 32][kFinalCells], re[kFinalThreads / 32][kFinalCells];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double* p = part + cell0 + (tid & 3);
     sc = 0.0;
     se = 0.0;
-    for (int t = lane; t < n_tiles; t += 32) {
-        sc += part[(int64_t)t * 2 * GG + cell];
-        se += part[(int64_t)t * 2 * GG + GG + cell];
+#pragma unroll 8
+    for (int t = tid >> 2; t < n_tiles; t += kFinalThreads / kFinalCells) {
+        sc += p[(int64_t)t * 2 * GG];
+        se += p[(int64_t)t * 2 * GG + GG];
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o >= kFinalCells; o >>= 1) {
         sc += __shfl_xor_sync(0xffffffffu, sc, o);
         se += __shfl_xor_sync(0xffffffffu, se, o);
     }
+    if (lane < kFinalCells) {
+        rc[warp][lane] = sc;
+        re[warp][lane] = se;
+    }
+    __syncthreads();
+    if (tid < kFinalCells)
+#pragma unroll
+        for (int w = 1; w < kFinalThreads / 32; ++w) {
+            sc += rc[w][tid];
+            se += re[w][tid];
+        }
 }
 
 // Tile partition of a launch's units.  One partial slot per tile; a tile's units
@@ -817,6 +839,9 @@ void loo_shape(const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2);
 inline int loo_unit_rows(int T1, int T2) { return T1 < 16 ? 8 : 1024 / (T1 * T2); }
 
 int launch_loo_tile_kernel(int T1, int T2, const LooArgs& a, int grid, cudaStream_t st);
+// the tile partials of one grid block summed into Lc, Le (row stride ld; either may be null)
+int loo_final_enqueue(const double* part, int n_tiles, int T1, int T2, int g1, int g2, int ld, int64_t N, double* Lc,
+                      double* Le, cudaStream_t st);
 // d_x >= 16: the kernel with the x cross-term on the tensor cores (loo_gram.cu)
 constexpr int kGramMinD = 16;
 int launch_loo_gram(int T1, int T2, const LooArgs& a, int grid, cudaStream_t st);

@@ -346,19 +346,27 @@ int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st) {
 }
 
 // --------------------------------------------------------------------------
-// Final fixed-order reduction of tile partials: one warp per grid cell.
+// Final fixed-order reduction of tile partials: one CTA per four grid cells
+// (GG is a multiple of 16); logn1 = ln(N - 1).
 // --------------------------------------------------------------------------
-__global__ void k_loo_final(const double* __restrict__ part, int n_tiles, int GG, int G2T,
-                            int G1r, int G2r, int ld, double N, double* Lc, double* Le) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= GG) return;
-    const int k = warp / G2T, l = warp % G2T;
+__global__ void __launch_bounds__(kFinalThreads) k_loo_final(const double* __restrict__ part, int n_tiles, int GG,
+                                                             int G2T, int G1r, int G2r, int ld, double N, double logn1,
+                                                             double* Lc, double* Le) {
     double sc, se;
-    loo_final_cell(part, n_tiles, GG, warp, lane, sc, se);
-    if (lane == 0 && k < G1r && l < G2r) {
+    loo_final_cells(part, n_tiles, GG, kFinalCells * blockIdx.x, sc, se);
+    const int cell = kFinalCells * blockIdx.x + threadIdx.x, k = cell / G2T, l = cell % G2T;
+    if (threadIdx.x < kFinalCells && k < G1r && l < G2r) {
         if (Lc) Lc[k * ld + l] = sc;
-        if (Le) Le[k * ld + l] = se / N - log(N - 1.0);
+        if (Le) Le[k * ld + l] = se / N - logn1;
     }
+}
+
+int loo_final_enqueue(const double* part, int n_tiles, int T1, int T2, int g1, int g2, int ld, int64_t N, double* Lc,
+                      double* Le, cudaStream_t st) {
+    k_loo_final<<<T1 * T2 / kFinalCells, kFinalThreads, 0, st>>>(part, n_tiles, T1 * T2, T2, g1, g2, ld, (double)N,
+                                                                std::log((double)N - 1.0), Lc, Le);
+    CDE_CUDA(cudaGetLastError());
+    return CDE_OK;
 }
 
 // --------------------------------------------------------------------------
@@ -413,6 +421,7 @@ void fill_loo_args(LooArgs& a, const Dataset& D, const double* h1, int g1, const
                    int g2, int T1, int T2) {
     a.xs = D.xs; a.y = D.y; a.mx = D.mx; a.my = D.my; a.qx = D.qx; a.qy = D.qy;
     a.N = D.N; a.Np = D.Np; a.d = D.d;
+    a.logn1 = std::log((double)D.N - 1.0);
     a.kern = D.kernel;
     if (D.kernel == CDE_KERNEL_EPAN) {
         // profiles (1 - t/h^2)_+; ln K_h = ln(profile) - (d ln h - ln c_d); no shifts
@@ -586,8 +595,9 @@ int loo_grid_enqueue(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, c
             a.fb = reinterpret_cast<double*>(reinterpret_cast<char*>(part) + pl.part_bytes);
             a.tile_base = 0;
             a.work = reinterpret_cast<int*>(reinterpret_cast<char*>(part) + pl.part_bytes + pl.fb_bytes);
-            CDE_CUDA(cudaMemsetAsync(a.work, 0, sizeof(int), st));
             const int grid = pl.grid;
+            if (pl.n_tiles <= grid) a.work = nullptr;   // a CTA per tile: no queue to reset
+            else CDE_CUDA(cudaMemsetAsync(a.work, 0, sizeof(int), st));
             timing_begin(ctx, st);
             int rc = pl.gram ? launch_loo_gram(T1, T2, a, grid, st) : launch_loo_tile_kernel(T1, T2, a, grid, st);
             timing_end(ctx, st);
@@ -596,12 +606,9 @@ int loo_grid_enqueue(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, c
                 return rc;
             }
             if (d_Lc || d_Le) {
-                const int GG = T1 * T2;
-                k_loo_final<<<(GG * 32 + 255) / 256, 256, 0, st>>>(
-                    part, a.n_tiles, GG, T2, g1, g2, G2, (double)D.N,
-                    d_Lc ? d_Lc + (size_t)k0 * G2 + l0 : nullptr,
-                    d_Le ? d_Le + (size_t)k0 * G2 + l0 : nullptr);
-                CDE_CUDA(cudaGetLastError());
+                rc = loo_final_enqueue(part, a.n_tiles, T1, T2, g1, g2, G2, D.N, d_Lc ? d_Lc + (size_t)k0 * G2 + l0 : nullptr,
+                                       d_Le ? d_Le + (size_t)k0 * G2 + l0 : nullptr, st);
+                if (rc != CDE_OK) return rc;
             }
             if (own) CDE_CUDA(cudaFreeAsync(part, st));
         }
@@ -725,11 +732,8 @@ int loo_chunked_next(LooChunked* c, void* scratch, double pair_evals, cudaStream
 }
 
 int loo_chunked_final(const LooChunked* c, const void* scratch, double* d_Lc, double* d_Le, cudaStream_t st) {
-    const int GG = c->T1 * c->T2;
-    k_loo_final<<<(GG * 32 + 255) / 256, 256, 0, st>>>(static_cast<const double*>(scratch), c->n_tiles, GG, c->T2,
-                                                        c->G1, c->G2, c->G2, (double)c->N, d_Lc, d_Le);
-    CDE_CUDA(cudaGetLastError());
-    return CDE_OK;
+    return loo_final_enqueue(static_cast<const double*>(scratch), c->n_tiles, c->T1, c->T2, c->G1, c->G2, c->G2, c->N,
+                             d_Lc, d_Le, st);
 }
 
 }  // namespace cde

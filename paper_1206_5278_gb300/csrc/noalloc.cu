@@ -15,9 +15,6 @@
 
 namespace cde {
 
-__global__ void k_loo_final(const double* __restrict__ part, int n_tiles, int GG, int G2T, int G1r,
-                            int G2r, int ld, double N, double* Lc, double* Le);
-
 // Scratch: tile partials (2 x G1 x G2 doubles per tile) followed by the tile
 // counter.  16 MiB in total; every GPU that loads the library holds it until exit.
 constexpr size_t kNoAllocScratchBytes = (size_t)16 << 20;
@@ -113,11 +110,7 @@ extern "C" int cde_loo_loglik_noalloc(cde_ctx* ctx, cde_dataset ds, const double
     rc = launch_loo_tile_kernel(T1, T2, a, grid, st);
     timing_end(ctx, st);
     if (rc != CDE_OK) return rc;
-    if (d_L_cond || d_L_eq3) {
-        const int GG = T1 * T2;
-        k_loo_final<<<(GG * 32 + 255) / 256, 256, 0, st>>>(a.part, a.n_tiles, GG, T2, G1, G2, G2,
-                                                          (double)D->N, d_L_cond, d_L_eq3);
-        CDE_CUDA(cudaGetLastError());
-    }
+    if (d_L_cond || d_L_eq3)
+        return loo_final_enqueue(a.part, a.n_tiles, T1, T2, G1, G2, G2, D->N, d_L_cond, d_L_eq3, st);
     return CDE_OK;
 }
