@@ -27,12 +27,14 @@
 // outer-product MMAs on the current block; one CTA barrier per step.
 //
 // The epilogue flags cells below the recompute threshold (as the tile body
-// does) and recomputes them exactly in two passes over the points that reuse
-// the distance blocks: points whose Gram distance, widened by 2^-16 (n_j + n_i)
-// (four times the Gram error bound), can lie in a cell's argmin region or sum
-// box get their distance recomputed directly, and everything after that is the
-// direct fallback's arithmetic (loo_common.cuh), so the recomputed cells are
-// those of the direct path.  Their log-numerators go to a per-CTA FP64 buffer;
+// does) and recomputes them exactly in one more pass over the distance blocks, with
+// the anchors of the direct kernels' one-pass recomputation (loo_common.cuh): a warp
+// owns its rows, so every cell has one anchor and one sum.  Points whose Gram
+// distance, lowered by 2^-16 (n_j + n_i) (four times the Gram error bound), can lie in
+// a cell's box get their distance recomputed directly, and everything after that is
+// direct arithmetic.  (Two passes, the first for every cell's minimiser through the rows'
+// Pareto fronts, took 35 of the 87 ms of a 32 x 32 grid at N = 40,009, d = 32; this one 17.)
+// The log-numerators go to a per-CTA FP64 buffer;
 // the unit's FP64 log-ratios are then summed over its rows in row order into
 // the unit's partial slot, and k_loo_final sums the slots in order: results are
 // bitwise reproducible.
@@ -73,12 +75,12 @@ struct GramCfg {
     __host__ __device__ static int o_pos(int d) { return o_flag(d) + kThreads; }                // [512]
     __host__ __device__ static int o_misc(int d) { return o_pos(d) + kThreads; }                // [64]
     __host__ __device__ static int o_list(int d) { return o_misc(d) + 64; }                     // [FMAX]
-    __host__ __device__ static int o_best(int d) { return o_list(d) + FMAX; }                   // [FMAX] u64
-    __host__ __device__ static int o_acc(int d) { return o_best(d) + 2 * FMAX; }                // [FMAX] u64
+    __host__ __device__ static int o_best(int d) { return o_list(d) + FMAX; }                   // [2][FMAX] a1, a2
+    __host__ __device__ static int o_acc(int d) { return o_best(d) + 2 * FMAX; }                // [FMAX] sums
     __host__ __device__ static int o_dxs(int d) { return o_acc(d) + 2 * FMAX; }                 // [FMAX]
     __host__ __device__ static int o_dys(int d) { return o_dxs(d) + FMAX; }                     // [FMAX]
-    __host__ __device__ static int o_sx(int d) { return o_dys(d) + FMAX; }                      // [FMAX] staircase X
-    __host__ __device__ static int o_sy(int d) { return o_sx(d) + FMAX; }                       // [FMAX] staircase Y
+    __host__ __device__ static int o_sx(int d) { return o_dys(d) + FMAX; }                      // [16][32] staircase buckets per warp
+    __host__ __device__ static int o_sy(int d) { return o_sx(d) + FMAX; }                       
     __host__ __device__ static int o_cf(int d) { return o_sy(d) + FMAX; }   // a1[32], a2[32], lam1[32], kap2[32] (f64)
     __host__ __device__ static int o_rp(int d) { return o_cf(d) + 192; }                        // [8][R]
     static size_t smem_bytes(int d) { return (size_t)(o_rp(d) + 8 * R) * 4; }
@@ -324,34 +326,81 @@ __device__ __forceinline__ int gram_scan(int v, int* pos, int* misc) {
     return total;
 }
 
-// Whether (X, Y) lies in the union of boxes [0, sx[i]] x [0, sy'[i]], given the
-// boxes' X extents sorted ascending (sx) and the suffix maxima of their Y
-// extents (sy): the first box reaching X decides.
-__device__ __forceinline__ bool stair_in(const float* sx, const float* sy, int n, float X, float Y) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int m = (lo + hi) >> 1;
-        if (sx[m] < X) lo = m + 1;
-        else hi = m;
+// The points that can matter to a row's cells, given the cells' boxes
+// [0, rx_f] x [0, ry_f]: lane b holds the largest ry_f over the cells whose rx_f lies in
+// bucket b or above, the buckets dividing [min rx, max rx] evenly in log2.  A point is
+// kept if its Y is at most the entry of its X's bucket: the union of the boxes, rounded
+// up by at most one bucket in X (a search of the exact staircase took about ten dependent
+// shared-memory loads per point).
+struct GramStair {
+    float m;          // this lane's entry
+    float l0, scale;  // bucket of X: (log2 X - l0) scale
+    __device__ __forceinline__ bool in(float X, float Y) const {
+        // (a hundredth of a bucket lower than the cells' buckets: covers the logarithm's rounding)
+        const int b = (int)fminf(fmaxf(fmaf(__log2f(fmaxf(X, 1e-37f)) - l0, scale, -0.01f), 0.f), 31.f);
+        return Y <= __shfl_sync(0xffffffffu, m, b) && X <= hi;
     }
-    return lo < n && Y <= sy[lo];
+    float hi;         // max rx
+};
+
+// The staircase of row rl (this warp's) from its cells' anchors; bk: 32 words of the warp.
+__device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk, const float* As, const float* Bs,
+                                                 const float* dxs, const float* dys, int fb, int fn, float mxv,
+                                                 float myv, float T) {
+    const int lane = threadIdx.x & 31;
+    float lo = INFINITY, hi = 0.f;
+    const auto extents = [&](int f, float& rx, float& ry) {
+        // (the factor covers the rounding of e where it is large next to T)
+        const float e = fmaf(fmaxf(fmaf(As[f], dxs[f] - mxv, Bs[f] * (dys[f] - myv)), 0.f), 1.f + 0x1p-20f, T);
+        rx = __fdividef(e, As[f]);
+        ry = __fdividef(e, Bs[f]);
+    };
+    for (int f = fb + lane; f < fb + fn; f += 32) {
+        float rx, ry;
+        extents(f, rx, ry);
+        lo = fminf(lo, rx);
+        hi = fmaxf(hi, rx);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    st.l0 = __log2f(lo);
+    st.scale = 31.f / fmaxf(__log2f(hi) - st.l0, 1e-3f);
+    st.hi = hi;
+    __syncwarp();
+    bk[lane] = 0u;
+    __syncwarp();
+    for (int f = fb + lane; f < fb + fn; f += 32) {
+        float rx, ry;
+        extents(f, rx, ry);
+        const int b = (int)fminf(fmaxf((__log2f(rx) - st.l0) * st.scale, 0.f), 31.f);
+        atomicMax(bk + b, __float_as_uint(ry));   // ry > 0: bit patterns order like the values
+    }
+    __syncwarp();
+    float m = __uint_as_float(bk[lane]);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {   // suffix maxima
+        const float v = __shfl_down_sync(0xffffffffu, m, o);
+        if (lane + o < 32) m = fmaxf(m, v);
+    }
+    st.m = m;
 }
 
-// One fallback pass over a step's block for this warp's rows with flagged cells
-// of the current round.  Lanes first take the points (the region tests), then
-// the row's cells: each point that passes is broadcast to all lanes, and lane
-// f % 32 updates cell f, which only it owns (no atomics; each cell sees the
-// points in step, chunk and lane order, so the sums are reproducible).
-//   PASS 1: argmin keys (e bits, point) on the block's distances;
-//   PASS 2: the shifted sums over the points inside the row's box, with their
-//           distances recomputed directly.
-template <int G1, int G2, int PASS, int JW>
-__device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_t p0, int buf, float (&fx)[JW],
-                                             float (&fy)[JW], unsigned int (&fp)[JW]) {
+// The recomputation's pass over a step's block, for this warp's rows with flagged cells
+// of the current round.  Lanes first take the points (the staircase test on the block's
+// distance, then on the direct one), then the row's cells: each point that passes is
+// broadcast to all lanes, and lane f % 32 updates cell f, which only it owns (no atomics;
+// each cell sees the points in step, chunk and lane order, so the sums are
+// reproducible).  A point below a cell's anchor rescales the sum and becomes the anchor;
+// the staircase follows the anchors down.
+template <int G1, int G2, int JW>
+__device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_t p0, int buf, float T,
+                                             GramStair (&st)[JW]) {
     using C = GramCfg<G1, G2>;
-    constexpr int R = C::R, PS = C::PS, GG = C::GG;
+    constexpr int R = C::R, PS = C::PS;
     static_assert(JW == C::JW, "rows per warp");
-    constexpr int LG2 = G2 == 8 ? 3 : (G2 == 16 ? 4 : 5);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = a.d, KS = C::ks(d);
     const int64_t Np = a.Np;
@@ -361,94 +410,56 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
     const float* Ys = sm + C::o_y(d) + buf * C::P;
     const float* rc = sm + C::o_rc(d);
     const float *yr_s = rc, *mxr_s = rc + R, *myr_s = rc + 2 * R, *nr_s = rc + 3 * R;
-    const float *qxr_s = rc + 4 * R, *qyr_s = rc + 5 * R;
-    const int* list = reinterpret_cast<const int*>(sm + C::o_list(d));
-    unsigned long long* best = reinterpret_cast<unsigned long long*>(sm + C::o_best(d));
+    const float* As = sm + C::o_best(d);
+    const float* Bs = As + C::FMAX;
     float* sum = sm + C::o_acc(d);
-    const float* dxs = sm + C::o_dxs(d);
-    const float* dys = sm + C::o_dys(d);
-    const float* rp = sm + C::o_rp(d);   // rlo, rhi (per row), rb, rn (ints)
-    const int* rbn = reinterpret_cast<const int*>(rp + 4 * R);
-    const float* sx = sm + C::o_sx(d);
-    const float* sy = sm + C::o_sy(d);
-    // the grid's coefficients in shared memory: 32 entries each, one per bank, so
-    // lanes reading different cells' coefficients never serialise
-    const float* a1s = sm + C::o_cf(d);
-    const float* a2s = a1s + 32;
+    float* dxs = sm + C::o_dxs(d);
+    float* dys = sm + C::o_dys(d);
+    const int* rbn = reinterpret_cast<const int*>(sm + C::o_rp(d) + 4 * R);
+    unsigned int* bk = reinterpret_cast<unsigned int*>(sm + C::o_sx(d)) + 32 * warp;
 #pragma unroll
-    for (int r = 0; r < JW; ++r) {   // unrolled: fx[r], fy[r], fp[r] stay in registers
+    for (int r = 0; r < JW; ++r) {   // unrolled: st[r] stays in registers
         const int rl = warp * JW + r;
         const int fb = rbn[rl], fn = rbn[R + rl];
         if (fn == 0) continue;
         const float mxv = mxr_s[rl], myv = myr_s[rl], yv = yr_s[rl], nr = nr_s[rl];
-        const float Xh = qxr_s[rl] - mxv, Yh = qyr_s[rl] - myv;
-        const float rlo = rp[rl], rhi = rp[R + rl];
-        const float rloY = rlo * Yh;
 #pragma unroll 1
         for (int c = 0; c < C::CPS; ++c) {
             const int pl = 32 * c + lane;
-            const int64_t p = p0 + pl;
             const float t1v = T1[rl * PS + pl];
             const bool live = t1v > -INFINITY;                       // not a masked pair
-            const float Xb = -t1v;                                   // the block's X (Gram, or direct if near)
-            const float Xg = Xb - kGramSlack * (nr + NPs[pl]);      // lowest the exact X can be
+            const float Xg = -t1v - kGramSlack * (nr + NPs[pl]);     // the lowest the exact X can be
             const float dy = yv - Ys[pl];
             const float dy2 = __fmul_rn(dy, dy);
             const float Y = dy2 - myv;
-            if (PASS == 1) {
-                // argmin keys on the block's distances: a key that is not the exact
-                // minimiser is within 2 a1 times the Gram error of it, which is all the
-                // anchor of pass 2 needs (its own distances are then taken directly)
-                const bool in = live && Xg <= Xh && Y <= Yh &&
-                                ((rlo >= 0.f && fmaf(rlo, Y, Xg) <= rloY) || (rhi < INFINITY && fmaf(rhi, Y, Xg) <= Xh));
-                // Every cell's minimiser is on the region's Pareto front (no other point
-                // has both a smaller X and a smaller Y): the warp keeps the row's front,
-                // one entry per lane (free entries hold +inf), and the cells are scored on
-                // it once the pass is done.  A point that finds the front full updates
-                // the cells directly instead.
-                unsigned int m = __ballot_sync(0xffffffffu, in);
-                const float X = fmaxf(Xb, 0.f);
-                while (m) {
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1;
-                    const float Xq = __shfl_sync(0xffffffffu, X, src), Yq = __shfl_sync(0xffffffffu, Y, src);
-                    const unsigned int pq = (unsigned int)(p0 + 32 * c + src);
-                    if (__ballot_sync(0xffffffffu, fx[r] <= Xq && fy[r] <= Yq)) continue;   // dominated
-                    if (Xq <= fx[r] && Yq <= fy[r]) fx[r] = fy[r] = INFINITY;               // entries it dominates
-                    const unsigned int fr = __ballot_sync(0xffffffffu, fx[r] == INFINITY);
-                    if (fr) {
-                        if (lane == __ffs(fr) - 1) {
-                            fx[r] = Xq;
-                            fy[r] = Yq;
-                            fp[r] = pq;
-                        }
-                    } else {
-                        for (int f = fb + lane; f < fb + fn; f += 32) {
-                            const int kl = list[f] - rl * GG, k = kl >> LG2, l = kl & (G2 - 1);
-                            const float e = fmaxf(fmaf(a1s[k], Xq, a2s[l] * Yq), 0.f);
-                            const unsigned long long key = ((unsigned long long)__float_as_uint(e) << 32) | pq;
-                            if (key < best[f]) best[f] = key;
-                        }
+            const bool pre = st[r].in(Xg, Y) && live;
+            if (!__any_sync(0xffffffffu, pre)) continue;
+            float d2 = INFINITY;
+            if (pre) d2 = direct_d2(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
+            const bool in = st[r].in(d2 - mxv, Y) && pre;
+            unsigned int m = __ballot_sync(0xffffffffu, in);
+            if (m == 0u) continue;
+            bool moved = false;
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const float d2q = __shfl_sync(0xffffffffu, d2, src), dy2q = __shfl_sync(0xffffffffu, dy2, src);
+                for (int f = fb + lane; f < fb + fn; f += 32) {
+                    float e = fmaf(As[f], d2q - dxs[f], Bs[f] * (dy2q - dys[f]));
+                    float S = sum[f];
+                    if (e < 0.f) {
+                        S *= ex2_approx(kFbEx2Fix + e);
+                        dxs[f] = d2q;
+                        dys[f] = dy2q;
+                        e = 0.f;
+                        moved = true;
                     }
+                    sum[f] = S + ex2_approx(kFbEx2Fix - e);
                 }
-            } else {
-                (void)fx; (void)fy; (void)fp;
-                // the region's points with their distances recomputed directly (few: each
-                // lane recomputes its own point; the result is then broadcast to the cells)
-                const bool pre = live && stair_in(sx + fb, sy + fb, fn, Xg, Y);
-                float d2 = 0.f;
-                if (pre) d2 = direct_d2(rows_s + rl * KS, a.xs, p, d, Np);
-                const bool in = pre && stair_in(sx + fb, sy + fb, fn, d2 - mxv, Y);
-                unsigned int m = __ballot_sync(0xffffffffu, in);
-                while (m) {
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1;
-                    const float d2q = __shfl_sync(0xffffffffu, d2, src), dy2q = __shfl_sync(0xffffffffu, dy2, src);
-                    for (int f = fb + lane; f < fb + fn; f += 32) {
-                        const int kl = list[f] - rl * GG, k = kl >> LG2, l = kl & (G2 - 1);
-                        sum[f] += ex2_approx(kFbEx2Fix - (a1s[k] * (d2q - dxs[f]) + a2s[l] * (dy2q - dys[f])));
-                    }
-                }
+            }
+            if (__any_sync(0xffffffffu, moved)) {
+                __syncwarp();
+                gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxv, myv, T);
             }
         }
     }
@@ -570,7 +581,7 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
     }
     __syncthreads();
 
-    // ---- cells below the recompute threshold: exact two-pass recomputation ----
+    // ---- cells below the recompute threshold: exact recomputation ----
     double* fbv = a.fb + (size_t)blockIdx.x * C::CELLS;   // this CTA's recomputed log2 At
     unsigned int fw = 0;
     if (KERN == 0) {
@@ -586,12 +597,13 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
     const int total = gram_scan(__popc(fw), pos, misc);
     if (KERN == 0 && total > 0) {
         int* list = reinterpret_cast<int*>(sm + C::o_list(d));
-        unsigned long long* best = reinterpret_cast<unsigned long long*>(sm + C::o_best(d));
+        float* As = sm + C::o_best(d);
+        float* Bs = As + C::FMAX;
         float* sum = sm + C::o_acc(d);
         float* dxs = sm + C::o_dxs(d);
         float* dys = sm + C::o_dys(d);
-        float* rp = sm + C::o_rp(d);
-        int* rbn = reinterpret_cast<int*>(rp + 4 * R);
+        int* rbn = reinterpret_cast<int*>(sm + C::o_rp(d) + 4 * R);
+        unsigned int* bk = reinterpret_cast<unsigned int*>(sm + C::o_sx(d)) + 32 * warp;
         int lg = 0;
         while (((int64_t)1 << lg) < N) ++lg;
         const float T = (float)(32 + lg);
@@ -607,12 +619,21 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
                     ++q;
                 }
             }
+            __syncthreads();
+            // the cells' coefficients and first anchors: the better of the x-nearest point
+            // (m_x, q_y) and the y-nearest (q_x, m_y), direct distances both
             for (int f = tid; f < n; f += NTH) {
-                best[f] = ~0ull;
+                const int rl = list[f] / GG, kl = list[f] - rl * GG;
+                const float A = a1s[kl >> LG2], B = a2s[kl & (G2 - 1)];
+                const float mxv = mxr_s[rl], myv = myr_s[rl], qx = qxr_s[rl], qy = qyr_s[rl];
+                const bool xn = B * (qy - myv) <= A * (qx - mxv);
+                As[f] = A;
+                Bs[f] = B;
+                dxs[f] = xn ? mxv : qx;
+                dys[f] = xn ? qy : myv;
                 sum[f] = 0.f;
             }
-            __syncthreads();
-            // per row: its range of the list, and the argmin region's triangles
+            // per row: its range of the list
             for (int rl = tid; rl < R; rl += NTH) {
                 int lo = 0, hi = n;   // first entry of row rl
                 while (lo < hi) {
@@ -624,114 +645,20 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
                 while (e < n && list[e] / GG == rl) ++e;
                 rbn[rl] = lo;
                 rbn[R + rl] = e - lo;
-                const float Xh = qxr_s[rl] - mxr_s[rl], Yh = qyr_s[rl] - myr_s[rl];
-                float rlo = -1.f, rhi = INFINITY;
-                for (int f = lo; f < e; ++f) {
-                    const int kl = list[f] - rl * GG;
-                    const float rho = a2s[kl & (G2 - 1)] / a1s[kl >> LG2];
-                    if (rho * Yh <= Xh) rlo = fmaxf(rlo, rho);
-                    else rhi = fminf(rhi, rho);
-                }
-                rp[rl] = rlo;
-                rp[R + rl] = rhi;
             }
             __syncthreads();
-            // pass 1: argmin keys (via each row's Pareto front)
-            float fx[JW], fy[JW];
-            unsigned int fp[JW];
+            GramStair st[JW];
 #pragma unroll
             for (int r = 0; r < JW; ++r) {
-                fx[r] = fy[r] = INFINITY;
-                fp[r] = 0u;
+                const int rl = warp * JW + r, fb = rbn[rl], fn = rbn[R + rl];
+                if (fn > 0) gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxr_s[rl], myr_s[rl], T);
             }
             gram_block<G1, G2, KERN, false>(a, sm, 0, 0);
             __syncthreads();
             for (int64_t s = 0; s < n_steps; ++s) {
                 const int b = (int)(s & 1);
                 if (s + 1 < n_steps) gram_block<G1, G2, KERN, false>(a, sm, (s + 1) * P, b ^ 1);
-                gram_fb_scan<G1, G2, 1, JW>(a, sm, s * P, b, fx, fy, fp);
-                __syncthreads();
-            }
-            // score the cells on their row's front (lane = cell)
-#pragma unroll
-            for (int r = 0; r < JW; ++r) {
-                const int rl = warp * JW + r;
-                const int fb = rbn[rl], fn = rbn[R + rl];
-                if (fn == 0) continue;
-                const unsigned int valid = __ballot_sync(0xffffffffu, fx[r] < INFINITY);
-                for (int f0 = fb; f0 < fb + fn; f0 += 32) {
-                    const int f = f0 + lane;
-                    const bool own = f < fb + fn;
-                    const int kl = own ? list[f] - rl * GG : 0, k = kl >> LG2, l = kl & (G2 - 1);
-                    unsigned long long bk = own ? best[f] : ~0ull;
-                    unsigned int vm = valid;
-                    while (vm) {
-                        const int src = __ffs(vm) - 1;
-                        vm &= vm - 1;
-                        const float Xq = __shfl_sync(0xffffffffu, fx[r], src), Yq = __shfl_sync(0xffffffffu, fy[r], src);
-                        const unsigned int pq = __shfl_sync(0xffffffffu, fp[r], src);
-                        const float e = fmaxf(fmaf(a1s[k], Xq, a2s[l] * Yq), 0.f);
-                        const unsigned long long key = ((unsigned long long)__float_as_uint(e) << 32) | pq;
-                        bk = key < bk ? key : bk;
-                    }
-                    if (own) best[f] = bk;
-                }
-            }
-            __syncthreads();
-            // the anchors' direct distances (a cell with no key, which the x- and the
-            // y-nearest points rule out, is anchored at the x-nearest bound: X = 0, Y = Yh)
-            for (int f = tid; f < n; f += NTH) {
-                const int rl = list[f] / GG;
-                const unsigned long long bk = best[f];
-                if (bk == ~0ull) {
-                    dxs[f] = mxr_s[rl];
-                    dys[f] = qyr_s[rl];
-                } else {
-                    const int64_t ps = CDE_CK((int64_t)(unsigned int)bk, N, 124);
-                    dxs[f] = direct_d2(rows_s + rl * KS, a.xs, ps, d, Np);
-                    const float dy = yr_s[rl] - a.y[ps];
-                    dys[f] = __fmul_rn(dy, dy);
-                }
-            }
-            __syncthreads();
-            // the region of pass 2: a cell's terms exceed 2^-T only at X <= (e_* + T)/a1,
-            // Y <= (e_* + T)/a2; a row's region is the union of its cells' boxes, kept
-            // as a staircase: the boxes sorted by X extent (ties by position) with the
-            // largest Y extent at or beyond each (a point is in the union iff its
-            // Y <= that of the first box reaching its X)
-            float* sx = sm + C::o_sx(d);
-            float* sy = sm + C::o_sy(d);
-            for (int f = tid; f < n; f += NTH) {
-                const int rl = list[f] / GG, kl = list[f] - rl * GG, k = kl >> LG2, l = kl & (G2 - 1);
-                const float es = fmaxf(fmaf(a1s[k], dxs[f] - mxr_s[rl], a2s[l] * (dys[f] - myr_s[rl])), 0.f);
-                const float rx = (es + T) / a1s[k], ry = (es + T) / a2s[l];
-                int rank = rbn[rl];
-                for (int g2 = rbn[rl]; g2 < rbn[rl] + rbn[R + rl]; ++g2) {
-                    if (g2 == f) continue;
-                    const int kl2 = list[g2] - rl * GG, k2 = kl2 >> LG2, l2 = kl2 & (G2 - 1);
-                    const float es2 = fmaxf(fmaf(a1s[k2], dxs[g2] - mxr_s[rl], a2s[l2] * (dys[g2] - myr_s[rl])), 0.f);
-                    const float rx2 = (es2 + T) / a1s[k2];
-                    rank += (rx2 < rx || (rx2 == rx && g2 < f));
-                }
-                sx[rank] = rx;
-                sy[rank] = ry;
-            }
-            __syncthreads();
-            for (int rl = tid; rl < R; rl += NTH) {
-                float m = -1.f;
-                for (int f = rbn[rl] + rbn[R + rl] - 1; f >= rbn[rl]; --f) {
-                    m = fmaxf(m, sy[f]);
-                    sy[f] = m;
-                }
-            }
-            __syncthreads();
-            // pass 2: the sums
-            gram_block<G1, G2, KERN, false>(a, sm, 0, 0);
-            __syncthreads();
-            for (int64_t s = 0; s < n_steps; ++s) {
-                const int b = (int)(s & 1);
-                if (s + 1 < n_steps) gram_block<G1, G2, KERN, false>(a, sm, (s + 1) * P, b ^ 1);
-                gram_fb_scan<G1, G2, 2, JW>(a, sm, s * P, b, fx, fy, fp);
+                gram_fb_scan<G1, G2, JW>(a, sm, s * P, b, T, st);
                 __syncthreads();
             }
             for (int f = tid; f < n; f += NTH) {
