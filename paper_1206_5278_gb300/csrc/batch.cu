@@ -169,7 +169,7 @@ static int build_plan(cde_ctx* ctx, const std::vector<BatchItem>& items, BatchPl
     for (int b = 0; b < n; ++b) {
         const BatchItem& it = items[b];
         int T1, T2;
-        loo_shape(*it.D, it.G1, it.G2, true, T1, T2);   // no member takes the d >= 16 kernel here
+        loo_shape(ctx->sm_count, *it.D, it.G1, it.G2, true, T1, T2);   // no member takes the d >= 16 kernel here
         shape[b] = it.D->kernel * 4096 + T1 * 64 + T2;
         LooArgs& a = args[b];
         memset(&a, 0, sizeof(a));

@@ -833,8 +833,9 @@ inline int loo_pad1(int g) { return g <= 16 ? 16 : 32; }
 inline int loo_pad2(int g) { return g <= 8 ? 8 : (g <= 16 ? 16 : 32); }
 // Grids of at most 8 x 8 on the direct kernel (d_x < 16, or `direct`) take the packed
 // body (loo_pack.cuh) with 4 or 8 bandwidths per axis, in the 16 x 8 body's place (and
-// in its tuning class: the units have the same 8 rows).
-void loo_shape(const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2);
+// in its tuning class: the units have the same 8 rows).  The d >= 16 kernel takes the shape
+// whose units fill the GPU best.  A row's terms do not depend on the shape.
+void loo_shape(int sm_count, const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2);
 // rows per unit of a (direct) shape
 inline int loo_unit_rows(int T1, int T2) { return T1 < 16 ? 8 : 1024 / (T1 * T2); }
 

@@ -390,10 +390,33 @@ static int launch_shape(const LooArgs& a, int grid, cudaStream_t st) {
 }
 
 
-void loo_shape(const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2) {
+void loo_shape(int sm_count, const Dataset& D, int g1, int g2, bool direct, int& T1, int& T2) {
     T1 = loo_pad1(g1);
     T2 = loo_pad2(g2);
-    if (g1 <= 8 && g2 <= 8 && (direct || !loo_use_gram(D, T1, T2))) {
+    if (!direct && loo_use_gram(D, T1, T2)) {
+        // The d >= 16 kernel runs one CTA per SM and a narrow shape's unit is many rows (128 at
+        // 16 x 8): where those leave SMs idle or the last wave nearly empty, a wider shape's
+        // smaller units finish sooner although they carry padding.  Waves x rows x the cost of a
+        // row (relative, measured at N = 20,000, d = 32).  8 x 8 grids, tile kernel: N = 3,000,
+        // d = 16 1.35 ms at 16 x 8, 0.73 at 16 x 32; N = 8,000, d = 20 3.47 / 1.99 at 16 x 16;
+        // N = 20,000, d = 32 17.6 / 15.2 at 16 x 16.
+        static const struct { int t1, t2; double cost; } kShapes[] = {{16, 8, 1.0},   {16, 16, 1.15}, {32, 8, 1.23},
+                                                                      {16, 32, 1.49}, {32, 16, 1.53}, {32, 32, 2.03}};
+        double best = INFINITY;
+        int b1 = T1, b2 = T2;
+        for (const auto& s : kShapes) {
+            if (s.t1 < T1 || s.t2 < T2 || !loo_use_gram(D, s.t1, s.t2)) continue;
+            const int64_t rows = loo_gram_rows_per_unit(s.t1, s.t2), units = (D.N + rows - 1) / rows;
+            const double t = (double)((units + sm_count - 1) / sm_count) * (double)rows * s.cost;
+            if (t < best) {
+                best = t;
+                b1 = s.t1;
+                b2 = s.t2;
+            }
+        }
+        T1 = b1;
+        T2 = b2;
+    } else if (g1 <= 8 && g2 <= 8) {
         T1 = g1 <= 4 ? 4 : 8;
         T2 = g2 <= 4 ? 4 : 8;
     }
@@ -550,7 +573,7 @@ size_t loo_grid_scratch_bytes(cde_ctx* ctx, const Dataset& D, int G1, int G2, in
     for (int k0 = 0; k0 < G1; k0 += 32) {
         for (int l0 = 0; l0 < G2; l0 += 32) {
             int T1, T2;
-            loo_shape(D, G1 - k0 < 32 ? G1 - k0 : 32, G2 - l0 < 32 ? G2 - l0 : 32, false, T1, T2);
+            loo_shape(ctx->sm_count, D, G1 - k0 < 32 ? G1 - k0 : 32, G2 - l0 < 32 ? G2 - l0 : 32, false, T1, T2);
             const size_t b = loo_plan(ctx, D, T1, T2, n_rows).bytes();
             if (b > mx) mx = b;
         }
@@ -568,7 +591,7 @@ int loo_grid_enqueue(cde_ctx* ctx, const Dataset& D, const double* h1, int G1, c
         for (int l0 = 0; l0 < G2; l0 += 32) {
             const int g2 = G2 - l0 < 32 ? G2 - l0 : 32;
             int T1, T2;
-            loo_shape(D, g1, g2, false, T1, T2);
+            loo_shape(ctx->sm_count, D, g1, g2, false, T1, T2);
             LooArgs a{};
             fill_loo_args(a, D, h1 + k0, g1, h2 + l0, g2, T1, T2);
             const LooPlan pl = loo_plan(ctx, D, T1, T2, n_rows);
@@ -637,7 +660,7 @@ int loo_chunked_create(cde_ctx* ctx, const Dataset& D, const double* h1, int G1,
                        LooChunked** out) {
     if (G1 > 32 || G2 > 32) return set_error(CDE_EINVAL, "loo_chunked_create: one grid block (<= 32 x 32) only");
     auto* c = new LooChunked{};
-    loo_shape(D, G1, G2, false, c->T1, c->T2);
+    loo_shape(ctx->sm_count, D, G1, G2, false, c->T1, c->T2);
     c->G1 = G1;
     c->G2 = G2;
     LooArgs& a = c->a;

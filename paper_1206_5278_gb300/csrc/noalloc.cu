@@ -70,7 +70,7 @@ extern "C" int cde_loo_loglik_noalloc(cde_ctx* ctx, cde_dataset ds, const double
     cudaStream_t st = pick_stream(ctx, stream);
 
     int T1, T2;
-    loo_shape(*D, G1, G2, true, T1, T2);   // the direct kernel at every d_x
+    loo_shape(ctx->sm_count, *D, G1, G2, true, T1, T2);   // the direct kernel at every d_x
     LooArgs a{};
     fill_loo_args(a, *D, h1, G1, h2, G2, T1, T2);
     const int JW = loo_unit_rows(T1, T2);
