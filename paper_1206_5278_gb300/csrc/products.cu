@@ -23,11 +23,13 @@
 // the segments in turn), over the chunks in turn.  k_chunk_weights forms the
 // chunk totals with one query per lane (the points are broadcast, a segment's
 // pairwise sum is a tree in registers: no shuffles and one barrier per chunk);
-// k_cond_sample, one CTA per query, sums them, sorts the S index targets, finds
-// each chunk's targets in the sorted list, and only for chunks with targets
-// repeats the scan, one chunk per warp, to resolve them.  The S values are then
-// sorted and the narrowest window of ceil((1 - alpha) S) consecutive values is
-// taken.  Random numbers: value k of the SplitMix64 stream of the seed,
+// k_cond_sample, one CTA per query, sums them, sorts the S index targets, finds each
+// target's chunk and 32-point segment in the running totals, and scans only that
+// segment (a warp per target, four at a time).  Where a target lies within rounding of
+// a prefix (2^-19 relative: the float prefixes of neighbouring points need not be
+// ordered there) the whole chunk is scanned and searched, so that every draw is the
+// one the search over the chunk's 256 prefixes finds.  The S values are then sorted
+// and the narrowest window of ceil((1 - alpha) S) consecutive values is taken.  Random numbers: value k of the SplitMix64 stream of the seed,
 // k = 2 (q S + s) for the index draw of sample s of query q and k + 1 for its
 // kernel offset; 24 random bits give u = (bits + 1/2) 2^-24 in (0, 1).
 #include <algorithm>
@@ -208,19 +210,20 @@ __global__ void __launch_bounds__(kCSThreads) k_cond_stats(const StatArgs a) {
 }
 
 // mean = sum u y / sum u (NaN when sum u = 0), fat = norm * sum u w / sum u (0 then).
-// A CTA sums 32 queries' split partials in FP64, eight threads per query over the splits
+// A CTA sums 16 queries' split partials in FP64, sixteen threads per query over the splits
 // (one thread per query waited for one strided load after the other: 173 us for 1,000
 // queries x 391 splits).
 __global__ void __launch_bounds__(256) k_cond_stats_final(const float* __restrict__ part, int n_split, int64_t Q,
                                                           double norm, double* __restrict__ mean,
                                                           double* __restrict__ fat) {
-    __shared__ double red[8][32][3];
-    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t q = (int64_t)blockIdx.x * 32 + lane;
+    constexpr int NG = 16;
+    __shared__ double red[NG][16][3];
+    const int lane = threadIdx.x & 15, g = threadIdx.x >> 4;
+    const int64_t q = (int64_t)blockIdx.x * 16 + lane;
     double s0 = 0, s1 = 0, s2 = 0;
     if (q < Q) {
-#pragma unroll 4
-        for (int s = g; s < n_split; s += 8) {
+#pragma unroll 8
+        for (int s = g; s < n_split; s += NG) {
             const float* p = part + ((int64_t)s * Q + q) * 3;
             s0 += p[0];
             s1 += p[1];
@@ -233,7 +236,7 @@ __global__ void __launch_bounds__(256) k_cond_stats_final(const float* __restric
     __syncthreads();
     if (g != 0 || q >= Q) return;
 #pragma unroll
-    for (int w = 1; w < 8; ++w) {
+    for (int w = 1; w < NG; ++w) {
         s0 += red[w][lane][0];
         s1 += red[w][lane][1];
         s2 += red[w][lane][2];
@@ -247,6 +250,7 @@ __global__ void __launch_bounds__(256) k_cond_stats_final(const float* __restric
 // --------------------------------------------------------------------------
 constexpr int kSmpThreads = 256, kSmpWarps = kSmpThreads / 32, kSmpMax = 4096;
 constexpr int kChunk = 256;           // points per chunk of the cumulative weights
+constexpr int kSegs = kChunk / 32;    // its 32-point segments
 constexpr int kEndsMax = 2048;        // chunk ends kept in shared memory
 
 struct SampleArgs {
@@ -260,7 +264,8 @@ struct SampleArgs {
     int d, S, SP, m_keep;   // samples, padded power of two, window size ceil((1-alpha) S)
     float a1, h2;
     uint64_t seed;
-    float* ct;         // [n_chunks][nq] chunk totals, then running totals
+    float* ct;         // [n_chunks][8][nq] running sums of a chunk after each of its 32-point segments
+    float* ends;       // [n_chunks][nq] running totals after each chunk (more than kEndsMax chunks)
     float* lo;         // [Q]
     float* hi;         // [Q]
     float* samples;    // [Q][S] sorted, or null
@@ -326,10 +331,13 @@ __global__ void __launch_bounds__(kCwThreads) k_chunk_weights(const SampleArgs a
             __syncthreads();
             // (the first segment's sum plus an exact 0)
 #pragma unroll 1
-            for (int s = 0; s < TP; s += 32) tot = __fadd2_rn(tree_sum2<32>(weight, s), tot);
+            for (int s = 0; s < TP; s += 32) {
+                tot = __fadd2_rn(tree_sum2<32>(weight, s), tot);
+                float* ct = a.ct + (k * kSegs + (p0 + s) / 32) * a.nq;
+                if (qa < qe) ct[qa - a.q0] = tot.x;
+                if (qb < qe) ct[qb - a.q0] = tot.y;
+            }
         }
-        if (qa < qe) a.ct[k * a.nq + (qa - a.q0)] = tot.x;
-        if (qb < qe) a.ct[k * a.nq + (qb - a.q0)] = tot.y;
     }
 }
 
@@ -363,6 +371,17 @@ __device__ __forceinline__ void bitonic_sort(float* v, int n) {
         }
 }
 
+// inclusive scan over the warp in the fixed (shuffle) order of the cumulative weights
+__device__ __forceinline__ float warp_scan(float v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float n = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += n;
+    }
+    return v;
+}
+
 // One chunk's weights (point 32 s + lane of the chunk in u[s])
 template <int KERN>
 __device__ __forceinline__ void chunk_weights(const SampleArgs& a, const SampleSmem& S, int64_t k, float mq,
@@ -393,7 +412,8 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t q = a.q0 + blockIdx.x;
     const int64_t nch = a.n_chunks;
-    float* ct = a.ct + blockIdx.x;   // stride nq
+    const float* ct = a.ct + blockIdx.x;   // stride nq
+    float* ge = a.ends + blockIdx.x;
     for (int c = tid; c < a.d; c += kSmpThreads) S.xq[c] = a.xq[(int64_t)c * a.Qp + q];
     const float mq = KERN == 0 ? a.mq[q] : 0.f;
     if (tid == 0) {
@@ -407,7 +427,7 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
         __syncthreads();
         int last = -1;
         for (int k = tid; k < n; k += kSmpThreads) {
-            const float v = ct[(k0 + k) * a.nq];
+            const float v = ct[((k0 + k) * kSegs + kSegs - 1) * a.nq];
             S.ends[k] = v;
             if (v > 0.f) last = (int)(k0 + k);
         }
@@ -424,9 +444,9 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
         }
         __syncthreads();
         if (!local)
-            for (int k = tid; k < n; k += kSmpThreads) ct[(k0 + k) * a.nq] = S.ends[k];
+            for (int k = tid; k < n; k += kSmpThreads) ge[(k0 + k) * a.nq] = S.ends[k];
     }
-    const auto end_of = [&](int64_t k) { return k < 0 ? 0.f : local ? S.ends[k] : ct[k * a.nq]; };
+    const auto end_of = [&](int64_t k) { return k < 0 ? 0.f : local ? S.ends[k] : ge[k * a.nq]; };
     const float total = S.total;
     const int last = S.last;
     if (last < 0 || !(total > 0.f)) {  // no weight (Epanechnikov: no x-neighbour)
@@ -443,66 +463,117 @@ __global__ void __launch_bounds__(kSmpThreads) k_cond_sample(const SampleArgs a)
         S.val[s] = s < a.S ? uniform24(a.seed, 2 * ((uint64_t)q * a.S + s)) * total : INFINITY;
     __syncthreads();
     bitonic_sort(S.val, a.SP);
-    // Resolve the targets against the cumulative weights: those below the end of chunk k
-    // and not below its beginning are chunk k's.  Warp w takes the chunks 8 m + w, the
-    // target ranges of 32 of them at a time (lane = chunk).
-    const auto first_at = [&](float v) {   // first target >= v
-        int lo = 0, hi = a.S;
+    // The index of one target by the whole chunk: its prefixes to shared memory, the first
+    // above t by binary search (the same in every lane)
+    const auto by_chunk = [&](int64_t k, float t) {
+        float u[kSegs];
+        chunk_weights<KERN>(a, S, k, mq, u);
+        int chunk_last = -1;
+        float before = 0.f;   // the segments before this one
+#pragma unroll
+        for (int g = 0; g < kSegs; ++g) {
+            const unsigned pos = __ballot_sync(0xffffffffu, u[g] > 0.f);
+            if (pos) chunk_last = 32 * g + 31 - __clz(pos);
+            const float v = warp_scan(u[g]);
+            const float seg = __shfl_sync(0xffffffffu, v, 31);
+            S.P[warp][32 * g + lane] = g > 0 ? v + before : v;
+            before = g > 0 ? seg + before : seg;
+        }
+        __syncwarp();
+        int lo = 0, hi = kChunk;  // first prefix above t
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (S.val[mid] < v) lo = mid + 1;
+            if (S.P[warp][mid] <= t) lo = mid + 1;
             else hi = mid;
         }
-        return lo;
+        __syncwarp();
+        if (lo > chunk_last) lo = chunk_last;  // rounding at the chunk's end
+        return (int)(k * kChunk + lo);
     };
-    for (int64_t m0 = 0; m0 * kSmpWarps < nch; m0 += 32) {
-        const int64_t kl = (m0 + lane) * kSmpWarps + warp;
-        int p = 0, p2 = 0;
-        if (kl < nch) {
-            p = first_at(end_of(kl - 1));
-            p2 = first_at(end_of(kl));
+    // Resolve the targets, 32 at a time per warp.  Lane = target: the first chunk whose end
+    // lies above it, then the first of its segments whose running sum does; then four targets
+    // at a time, lane = point of the target's segment.
+    constexpr float kNear = 0x1p-19f;   // prefixes closer to a target than this (relative) decide nothing
+    for (int b0 = 32 * warp; b0 < a.S; b0 += kSmpThreads) {
+        const int s = b0 + lane;
+        int64_t k = -1;
+        int g = 0;
+        float t = 0.f, before = 0.f;
+        bool whole = false;
+        if (s < a.S && S.val[s] < total) {
+            const float v = S.val[s];
+            int64_t lo = 0, hi = nch - 1;   // first chunk with its end above v (the last one's is `total`)
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (end_of(mid) > v) hi = mid;
+                else lo = mid + 1;
+            }
+            k = lo;
+            t = v - end_of(k - 1);
+            const float* seg = ct + k * kSegs * a.nq;
+            float c[kSegs];
+#pragma unroll
+            for (int e = 0; e < kSegs; ++e) c[e] = seg[e * a.nq];
+#pragma unroll
+            for (int e = 0; e < kSegs; ++e)
+                if (c[e] <= t) {
+                    g = e + 1;
+                    before = c[e];
+                }
+            whole = g == kSegs || (g > 0 && t - before <= kNear * t);
         }
-        unsigned live = __ballot_sync(0xffffffffu, p < p2);
-        while (live) {
-            const int src = __ffs(live) - 1;
-            live &= live - 1;
-            const int64_t k = (m0 + src) * kSmpWarps + warp;
-            const int s0 = __shfl_sync(0xffffffffu, p, src), s1 = __shfl_sync(0xffffffffu, p2, src);
-            const float base = end_of(k - 1);
-            float u[kChunk / 32];
-            chunk_weights<KERN>(a, S, k, mq, u);
-            int chunk_last = -1;
-            float before = 0.f;   // the segments before this one
+        const unsigned live = __ballot_sync(0xffffffffu, k >= 0);
+        const unsigned full = __ballot_sync(0xffffffffu, whole);
+        for (int j0 = 0; j0 < 32; j0 += 4) {
+            if (((live >> j0) & 15u) == 0u) continue;
+            float u[4], tt[4], bf[4];
+            int64_t kk[4];
+            int gg[4];
 #pragma unroll
-            for (int g = 0; g < kChunk / 32; ++g) {
-                float v = u[g];
-                const unsigned pos = __ballot_sync(0xffffffffu, v > 0.f);
-                if (pos) chunk_last = 32 * g + 31 - __clz(pos);
+            for (int e = 0; e < 4; ++e) {
+                kk[e] = __shfl_sync(0xffffffffu, k, j0 + e);
+                gg[e] = __shfl_sync(0xffffffffu, g, j0 + e) & (kSegs - 1);
+                tt[e] = __shfl_sync(0xffffffffu, t, j0 + e);
+                bf[e] = __shfl_sync(0xffffffffu, before, j0 + e);
+            }
+            float dx2[4] = {0.f, 0.f, 0.f, 0.f};
+            const float* x[4];
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const float n = __shfl_up_sync(0xffffffffu, v, o);
-                    if (lane >= o) v += n;
+            for (int e = 0; e < 4; ++e)   // (dead targets: the first segment)
+                x[e] = a.xs + CDE_CK(max(kk[e], (int64_t)0) * kChunk + 32 * gg[e], a.Np - 31, 306) + lane;
+#pragma unroll 4
+            for (int c = 0; c < a.d; ++c) {
+                const float xqc = S.xq[c];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float v = xqc - x[e][(int64_t)c * a.Np];
+                    dx2[e] = fmaf(v, v, dx2[e]);
                 }
-                const float seg = __shfl_sync(0xffffffffu, v, 31);
-                S.P[warp][32 * g + lane] = g > 0 ? v + before : v;
-                before = g > 0 ? seg + before : seg;
             }
-            __syncwarp();
-            for (int s = s0 + lane; s < s1; s += 32) {
-                const float t = S.val[s] - base;
-                int lo = 0, hi = kChunk;  // first prefix above t
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (S.P[warp][mid] <= t) lo = mid + 1;
-                    else hi = mid;
-                }
-                if (lo > chunk_last) lo = chunk_last;  // rounding at the chunk's end
-                S.idx[CDE_CK(s, kSmpMax, 305)] = (int)(k * kChunk + lo);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                u[e] = max(kk[e], (int64_t)0) * kChunk + 32 * gg[e] + lane < a.N ? xweight<KERN>(dx2[e], a.a1, mq) : 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const unsigned bit = 1u << (j0 + e);
+                if (!(live & bit)) continue;
+                const float v = warp_scan(u[e]);
+                const float P = gg[e] > 0 ? v + bf[e] : v;
+                const unsigned below = __ballot_sync(0xffffffffu, P <= tt[e]);
+                const bool near = __any_sync(0xffffffffu, fabsf(P - tt[e]) <= kNear * tt[e]);
+                int at;
+                if (near || (full & bit) || below == 0xffffffffu) at = by_chunk(kk[e], tt[e]);
+                else at = (int)(kk[e] * kChunk + 32 * gg[e] + __popc(below));
+                if (lane == 0) S.idx[CDE_CK(b0 + j0 + e, kSmpMax, 305)] = at;
             }
-            __syncwarp();
         }
     }
-    const int top = first_at(total);   // targets at the very top: the last point with weight
+    int top = 0;   // first target >= total: from there on the last point with weight
+    for (int hi = a.S; top < hi;) {
+        const int mid = (top + hi) >> 1;
+        if (S.val[mid] < total) top = mid + 1;
+        else hi = mid;
+    }
     if (top < a.S && warp == 0) {
         float u[kChunk / 32];
         chunk_weights<KERN>(a, S, last, mq, u);
@@ -645,7 +716,7 @@ static int cond_stats_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double 
     timing_end(ctx, st);
     CDE_CUDA(cudaGetLastError());
     const double norm = epan ? std::exp(epan_log_norm(1)) / h2 : 1.0 / (2.5066282746310002 * h2);
-    k_cond_stats_final<<<(unsigned)((Q + 31) / 32), 256, 0, st>>>(part, (int)ns, Q, norm, d_mean,
+    k_cond_stats_final<<<(unsigned)((Q + 15) / 16), 256, 0, st>>>(part, (int)ns, Q, norm, d_mean,
                                                                    d_yq ? d_fat : nullptr);
     CDE_CUDA(cudaGetLastError());
     cudaFreeAsync(part, st);
@@ -690,10 +761,12 @@ static int cond_interval_enqueue(cde_ctx* ctx, const Dataset& D, double h1, doub
     CDE_CUDA(smem_attr_once(attr0, k_cond_sample<0>, (int)sizeof(SampleSmem)));
     CDE_CUDA(smem_attr_once(attr1, k_cond_sample<1>, (int)sizeof(SampleSmem)));
     a.n_chunks = (D.N + kChunk - 1) / kChunk;
-    // queries in batches whose chunk totals fit 64 MB (at least 128)
-    const int64_t qmax = std::max<int64_t>(kCwQ, ((int64_t)16 << 20) / a.n_chunks / kCwQ * kCwQ);
+    // queries in batches whose running sums fit 128 MB (at least 128)
+    const int64_t qmax = std::max<int64_t>(kCwQ, ((int64_t)32 << 20) / (a.n_chunks * kSegs) / kCwQ * kCwQ);
     const int64_t qbatch = std::min(Q, qmax);
-    CDE_CUDA(pool_alloc(ctx, (void**)&a.ct, (size_t)(a.n_chunks * qbatch) * sizeof(float), st));
+    const bool more = a.n_chunks > kEndsMax;
+    CDE_CUDA(pool_alloc(ctx, (void**)&a.ct, (size_t)(a.n_chunks * (kSegs + (more ? 1 : 0)) * qbatch) * sizeof(float), st));
+    a.ends = a.ct + a.n_chunks * kSegs * qbatch;
     for (int64_t q0 = 0; q0 < Q; q0 += qbatch) {
         a.q0 = q0;
         a.nq = std::min(qbatch, Q - q0);
