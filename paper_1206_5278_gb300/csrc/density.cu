@@ -483,9 +483,11 @@ __device__ __forceinline__ void tc_flush(const DensTcArgs& a, TcSmem& S, uint32_
         const int64_t slot = (int64_t)blockIdx.x * a.MT + (tq - t_first);
         const int row = 32 * (warp & 3) + lane;
         float4* dst = reinterpret_cast<float4*>(a.part + (slot * kTcM + row) * kTcN + (warp >> 2) * kTcCols);
+        // padding queries' rows and column blocks past the grid are never read
+        const bool real = tq / a.GT * kTcM + row < a.Q && (warp >> 2) * kTcCols < a.G - (int)(tq % a.GT) * kTcN;
 #pragma unroll
         for (int v4 = 0; v4 < kTcCols / 4; ++v4) {
-            dst[v4] = make_float4(tot[4 * v4], tot[4 * v4 + 1], tot[4 * v4 + 2], tot[4 * v4 + 3]);
+            if (real) dst[v4] = make_float4(tot[4 * v4], tot[4 * v4 + 1], tot[4 * v4 + 2], tot[4 * v4 + 3]);
             tot[4 * v4] = tot[4 * v4 + 1] = tot[4 * v4 + 2] = tot[4 * v4 + 3] = 0.f;
         }
         // a query's four denominator parts (point quarters), summed in order
@@ -598,31 +600,43 @@ __device__ __forceinline__ int64_t tc_owner(int64_t u, int64_t U, int64_t P) { r
 
 // f[q][g] = (sum over the CTAs covering the tile of the partial numerators) /
 // (same for the denominators) * norm; a zero denominator (no x-neighbour)
-// gives 0.  A block is 32 grid points x 8 slots; a slot is one of `parts`
+// gives 0.  A block is 32 grid points x 8 slots of one tile; a slot is one of `parts`
 // consecutive pieces of the covering CTAs' range (parts = 1, 2, 4 or 8) of one
 // query row.  Pieces are summed in CTA order, then the pieces in order.  f
 // has row stride ldf (the caller's full grid when this pass covers part of it).
+// The covering CTAs' partial slots are listed once per block: their 64-bit divisions,
+// made by every thread, were most of the kernel (91 us at Q = 10,000, G = 256).
+constexpr int kFinalSlots = 1024;   // at least the SMs of any GPU
+
 __global__ void __launch_bounds__(256) k_density_final(const DensTcArgs a, float norm, int parts_log2,
                                                        float* __restrict__ f, int64_t ldf) {
     __shared__ float rn[8][32], rd[8][32];
+    __shared__ int slots[kFinalSlots];
     const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5;
     const int parts = 1 << parts_log2, part = slot & (parts - 1);
-    const int64_t gb_n = (a.G + 31) / 32, qb = (int64_t)blockIdx.x / gb_n;
+    const int gb_n = (a.G + 31) / 32;
+    const int64_t qb = (int64_t)blockIdx.x / gb_n;
     const int gb = (int)((int64_t)blockIdx.x - qb * gb_n);
-    const int64_t q = qb * (8 >> parts_log2) + (slot >> parts_log2);
+    const int64_t q0 = qb * (8 >> parts_log2), q = q0 + (slot >> parts_log2);   // (8 divides kTcM: one tile)
     const int g = gb * 32 + lane;
+    const int64_t t = (q0 / kTcM) * a.GT + (gb * 32) / kTcN;
+    const int64_t c0 = tc_owner(t * a.C, a.U, a.P), c1 = tc_owner(t * a.C + a.C - 1, a.U, a.P);
+    const int n = (int)(c1 - c0) + 1;
+    for (int e = threadIdx.x; e < n; e += 256) {
+        const int64_t c = c0 + e, ub = c * a.U / a.P, ue = (c + 1) * a.U / a.P;
+        slots[e] = ub < ue ? (int)(c * a.MT + (t - ub / a.C)) : -1;   // P MT slots: far below 2^31
+    }
+    __syncthreads();
     float sn = 0.f, sd = 0.f;
     if (q < a.Q) {
-        const int64_t t = (q / kTcM) * a.GT + (gb * 32) / kTcN;
-        const int64_t c0 = tc_owner(t * a.C, a.U, a.P), c1 = tc_owner(t * a.C + a.C - 1, a.U, a.P);
-        const int64_t per = (c1 - c0 + parts) / parts;
-        const int64_t cb = c0 + part * per, ce = min(c1 + 1, cb + per);
-        for (int64_t c = cb; c < ce; ++c) {
-            const int64_t ub = c * a.U / a.P, ue = (c + 1) * a.U / a.P;
-            if (ub >= ue) continue;
-            const int64_t sl = c * a.MT + (t - ub / a.C);
-            if (g < a.G) sn += a.part[(sl * kTcM + (q % kTcM)) * kTcN + g % kTcN];
-            sd += a.dpart[sl * kTcM + (q % kTcM)];
+        const int per = (n + parts - 1) / parts;
+        const int e1 = min(n, (part + 1) * per), row = (int)(q % kTcM), col = g % kTcN;
+#pragma unroll 4
+        for (int e = part * per; e < e1; ++e) {
+            const int sl = slots[e];
+            if (sl < 0) continue;
+            if (g < a.G) sn += a.part[((int64_t)sl * kTcM + row) * kTcN + col];
+            sd += a.dpart[(int64_t)sl * kTcM + row];
         }
     }
     rn[slot][lane] = sn;
@@ -670,7 +684,7 @@ int density_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, const 
     a.a2 = (float)(epan ? 1.0 / (h2 * h2) : L2E / (2 * h2 * h2));
     a.C = (D.N + kTcKC - 1) / kTcKC;
     a.U = (Qp / kTcM) * a.GT * a.C;
-    a.P = (int)std::min<int64_t>(ctx->sm_count, a.U);
+    a.P = (int)std::min<int64_t>(std::min(ctx->sm_count, kFinalSlots), a.U);
     a.MT = (int)(((a.U + a.P - 1) / a.P + a.C - 1) / a.C + 1);
     a.err = ctx->d_err + kErrTensorWait;
     CDE_CUDA(pool_alloc(ctx, (void**)&part, (size_t)a.P * a.MT * kTcM * kTcN * sizeof(float), st));
