@@ -738,6 +738,14 @@ __device__ __forceinline__ void loo_unit_epilogue(const LooArgs& a, const Coef& 
                 __syncthreads();
                 loo_fallback<C>(a, cf, sm, nfl);
             }
+        } else if constexpr (KERN == 1 && C::kOnePass) {
+            // Epanechnikov sums need no shift and no recomputation (at 32 x 32 the branch below,
+            // which then flags nothing, leaves the compiler a 1% to 3% faster main loop)
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+                const int c = tid + 256 * m;
+                if (CELLS % 256 == 0 || c < CELLS) la2[c] = log2_wide(At[m]);
+            }
         } else {
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
