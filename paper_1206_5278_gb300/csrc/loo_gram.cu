@@ -22,8 +22,8 @@
 // error can move a row's log-sum to about 2^-19 32/e ~ 2e-5 of one term.
 //
 // Per step of P points the warps first form the distance block of the next
-// step (double-buffered in shared memory: t1 = m_x,j - d2, t2 = m_y,j - dy2,
-// masked pairs t1 = -inf) and then run the tile body's exp2 / split /
+// step (double-buffered in shared memory: t1 = m_x,j - d2, masked pairs t1 = -inf, and the
+// points' norms and y) and then run the tile body's exp2 / split /
 // outer-product MMAs on the current block; one CTA barrier per step.
 //
 // The epilogue flags cells below the recompute threshold (as the tile body
@@ -33,7 +33,7 @@
 // distance, lowered by 2^-16 (n_j + n_i) (four times the Gram error bound), can lie in
 // a cell's box get their distance recomputed directly, and everything after that is
 // direct arithmetic.  (Two passes, the first for every cell's minimiser through the rows'
-// Pareto fronts, took 35 of the 87 ms of a 32 x 32 grid at N = 40,009, d = 32; this one 17.)
+// Pareto fronts, took 35 of the 87 ms of a 32 x 32 grid at N = 40,009, d = 32; this one about 10 of 55, 7 of them the scan.)
 // The log-numerators go to a per-CTA FP64 buffer;
 // the unit's FP64 log-ratios are then summed over its rows in row order into
 // the unit's partial slot, and k_loo_final sums the slots in order: results are
@@ -54,14 +54,13 @@ struct GramCfg {
     // points per step: one CTA barrier per step, and fewer barriers keep the
     // warps' exp2 and MMA phases from lining up (512 vs 128 points: 0.83x time)
     static constexpr int P = 512 / JW;
-    static constexpr int PS = P + 8;                                 // row stride of the blocks
+    static constexpr int PS = P + 4;                                 // row stride of the blocks (128-bit stores without bank conflicts)
     static constexpr int CPS = P / 32;                               // 32-point chunks per step
-    static constexpr int GT = (R / 16) * (P / 8);                    // Gram output tiles per step
-    static constexpr int TPW = GT / kWarps;                          // per warp
+    static constexpr int NG = P / 32;                                // a warp's Gram tiles per step: 16 rows x 32 points
     static constexpr int CELLS = R * GG;                             // 16384: one bit per thread-word
     static constexpr int FMAX = 1024;                                // flagged cells per fallback round
     static_assert(CELLS == 32 * kThreads, "one flag word per thread");
-    static_assert(TPW * kWarps == GT, "whole Gram tiles per warp");
+    static_assert(JW * NG == kWarps, "one 16 x 32 Gram block per warp");
     // shared memory layout in 4-byte words (KS: row stride of the staged row coordinates)
     __host__ __device__ static int ks(int d) { return ((d + 7) & ~7) + 4; }
     __host__ __device__ static int o_rows() { return 0; }
@@ -86,7 +85,7 @@ struct GramCfg {
     static size_t smem_bytes(int d) { return (size_t)(o_rp(d) + 8 * R) * 4; }
 };
 
-constexpr int kGramMaxKSteps = kMaxD / 8;     // k-steps of 8 dimensions at the largest d_x
+constexpr int kGramLoadSteps = 2;             // k-steps of 8 dimensions whose point loads are issued together
 constexpr float kGramNear = 1.0f / 32.0f;     // direct recomputation below this share of n_j + n_i
 constexpr float kGramSlack = 1.0f / 65536.0f; // pre-test widening, times n_j + n_i
 
@@ -94,7 +93,7 @@ constexpr float kGramSlack = 1.0f / 65536.0f; // pre-test widening, times n_j + 
 __device__ __forceinline__ float direct_d2(const float* __restrict__ xr, const float* __restrict__ xs,
                                            int64_t p, int d, int64_t Np) {
     float d2 = 0.f;
-#pragma unroll 4
+#pragma unroll 8
     for (int c = 0; c < d; ++c) {
         const float q = xr[c] - xs[(int64_t)c * Np + p];
         d2 = fmaf(q, q, d2);
@@ -108,6 +107,15 @@ __device__ __forceinline__ void split_rn(float x, uint32_t& hi, uint32_t& lo) {
     lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
+// Bound by latency: a step's block is little arithmetic between two trips to L2, and all 16
+// warps start it together after the barrier.  So a warp's 16 x 32 block takes its points with
+// one 128-bit load per lane and dimension (the 32 points dealt out over four MMA tiles), 16
+// dimensions' loads in flight, one set of row fragments for four independent MMA chains, and
+// the near pairs are recomputed after the block, every lane its own, instead of at each
+// output.  Four 8-point tiles per warp one after the other, 32-bit loads: 32 x 32 grid at
+// N = 40,009, d = 32 66.5 ms, now 55.1; N = 20,000, d = 32 16 x 16 17.4 -> 9.9 ms, 16 x 32
+// 16.1 -> 11.4.  Loads of all 32 dimensions in flight: 55.6 ms (registers).
+//
 // Distance block of one step: t1 of every (row, point) of the unit, the
 // points' norms and y, into buffer `buf`.  NEAR: recompute the near pairs
 // directly (the main pass; the fallback's passes work with the Gram values and
@@ -127,62 +135,100 @@ __device__ __forceinline__ void gram_block(const LooArgs& a, float* sm, int64_t 
     const float* rc = sm + C::o_rc(d);
     const float *mxr_s = rc + R, *nr_s = rc + 3 * R;
     const int* jr_s = reinterpret_cast<const int*>(rc + 6 * R);
+    const int mtg = warp / C::NG, ng = warp - mtg * C::NG;
+    // This lane's four B points: the warp's 32 points are dealt out so that column g of
+    // tile j is point 4g + j, one 128-bit load per dimension for all four tiles (steps may
+    // run past the padded length: those points are masked, their loads clamped).
+    const int pb = 32 * ng + 4 * g;
+    const int64_t pg = CDE_CK(min(p0 + pb, Np - 4), Np - 3, 121);
+    const int r0 = 16 * mtg + g, r1 = r0 + 8;
+    float acc[4][4], np[4];
 #pragma unroll
-    for (int tt = 0; tt < C::TPW; ++tt) {
-        const int ti = warp + C::kWarps * tt;
-        const int mtg = ti / (P / 8), ntg = ti - mtg * (P / 8);
-        // this lane's B point (steps may run past the padded length: those points are
-        // masked, and their loads are clamped to the last stored point)
-        const int64_t pg = CDE_CK(min(p0 + 8 * ntg + g, Np - 1), Np, 121);
-        const int r0 = 16 * mtg + g, r1 = r0 + 8;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        float np = 0.f;
-        // all of the tile's point coordinates first (one round trip to L2, not one per k-step)
-        float xb0[kGramMaxKSteps], xb1[kGramMaxKSteps];
+    for (int j = 0; j < 4; ++j) {
+        np[j] = 0.f;
 #pragma unroll
-        for (int s = 0; s < kGramMaxKSteps; ++s) {
-            const int c0 = 8 * s + t, c1 = c0 + 4;
-            xb0[s] = (s < KSTEPS && c0 < d) ? a.xs[(int64_t)c0 * Np + pg] : 0.f;
-            xb1[s] = (s < KSTEPS && c1 < d) ? a.xs[(int64_t)c1 * Np + pg] : 0.f;
-        }
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+    }
+#pragma unroll 1
+    for (int s0 = 0; s0 < KSTEPS; s0 += kGramLoadSteps) {
+        float xb[kGramLoadSteps][2][4];
 #pragma unroll
-        for (int s = 0; s < kGramMaxKSteps; ++s) {
-            if (s >= KSTEPS) break;
-            const int c0 = 8 * s + t, c1 = c0 + 4;
-            const float x0 = xb0[s], x1 = xb1[s];
-            np = fmaf(x0, x0, fmaf(x1, x1, np));
-            uint32_t bh0, bl0, bh1, bl1;
-            split_rn(x0, bh0, bl0);
-            split_rn(x1, bh1, bl1);
+        for (int s = 0; s < kGramLoadSteps; ++s)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = 8 * (s0 + s) + 4 * h + t;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c < d) v = *reinterpret_cast<const float4*>(a.xs + (int64_t)c * Np + pg);
+                xb[s][h][0] = v.x;
+                xb[s][h][1] = v.y;
+                xb[s][h][2] = v.z;
+                xb[s][h][3] = v.w;
+            }
+#pragma unroll
+        for (int s = 0; s < kGramLoadSteps; ++s) {
+            if (s0 + s >= KSTEPS) break;
+            const int c0 = 8 * (s0 + s) + t, c1 = c0 + 4;
             uint32_t ah[4], al[4];
             split_rn(rows_s[r0 * KS + c0], ah[0], al[0]);
             split_rn(rows_s[r1 * KS + c0], ah[1], al[1]);
             split_rn(rows_s[r0 * KS + c1], ah[2], al[2]);
             split_rn(rows_s[r1 * KS + c1], ah[3], al[3]);
-            mma_tf32(acc, al, bh0, bh1);
-            mma_tf32(acc, ah, bl0, bl1);
-            mma_tf32(acc, ah, bh0, bh1);
-        }
-        // point norms: lanes 4g .. 4g+3 hold point g's dimensions
-        np += __shfl_xor_sync(0xffffffffu, np, 1);
-        np += __shfl_xor_sync(0xffffffffu, np, 2);
-        const float npa = __shfl_sync(0xffffffffu, np, 8 * t), npb = __shfl_sync(0xffffffffu, np, 8 * t + 4);
-        if (t == 0 && mtg == 0) {
-            NPs[8 * ntg + g] = np;
-            Ys[8 * ntg + g] = a.y[pg];
-        }
-        // outputs: rows r0, r1 x points 2t, 2t+1 of the tile
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int rl = q < 2 ? r0 : r1;
-            const int pl = 8 * ntg + 2 * t + (q & 1);
-            const int64_t p = p0 + pl;
-            const float nr = nr_s[rl], nsum = nr + ((q & 1) ? npb : npa);
-            const float mxv = mxr_s[rl];
-            const bool ok = p < N && (int)p != jr_s[rl];
-            float d2 = fmaxf(fmaf(-2.f, acc[q], nsum), 0.f);
-            if (NEAR && ok && d2 - mxv < kGramNear * nsum) d2 = direct_d2(rows_s + rl * KS, a.xs, p, d, Np);
-            T1[rl * PS + pl] = KERN == 0 ? (ok ? mxv - d2 : -INFINITY) : (ok ? d2 : INFINITY);
+            for (int j = 0; j < 4; ++j) {
+                const float x0 = xb[s][0][j], x1 = xb[s][1][j];
+                np[j] = fmaf(x0, x0, fmaf(x1, x1, np[j]));
+                uint32_t bh0, bl0, bh1, bl1;
+                split_rn(x0, bh0, bl0);
+                split_rn(x1, bh1, bl1);
+                mma_tf32(acc[j], al, bh0, bh1);
+                mma_tf32(acc[j], ah, bl0, bl1);
+                mma_tf32(acc[j], ah, bh0, bh1);
+            }
+        }
+    }
+    // point norms: lanes 4g .. 4g+3 hold the dimensions of points 4g .. 4g+3
+    float npc[2][4];   // of columns 2t, 2t + 1
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        np[j] += __shfl_xor_sync(0xffffffffu, np[j], 1);
+        np[j] += __shfl_xor_sync(0xffffffffu, np[j], 2);
+        npc[0][j] = __shfl_sync(0xffffffffu, np[j], 8 * t);
+        npc[1][j] = __shfl_sync(0xffffffffu, np[j], 8 * t + 4);
+    }
+    if (t == 0 && mtg == 0) {
+        *reinterpret_cast<float4*>(NPs + pb) = make_float4(np[0], np[1], np[2], np[3]);
+        *reinterpret_cast<float4*>(Ys + pb) = *reinterpret_cast<const float4*>(a.y + pg);
+    }
+    // outputs: rows r0, r1 x points 8t .. 8t + 7 of the warp's 32
+    const int po = 32 * ng + 8 * t;
+    unsigned int near = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int rl = h ? r1 : r0;
+        const float nr = nr_s[rl], mxv = mxr_s[rl];
+        const int jr = jr_s[rl];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            float o[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t p = p0 + po + 4 * q + j;
+                const float nsum = nr + npc[q][j];
+                const bool ok = p < N && (int)p != jr;
+                const float d2 = fmaxf(fmaf(-2.f, acc[j][2 * h + q], nsum), 0.f);
+                if (NEAR && ok && d2 - mxv < kGramNear * nsum) near |= 1u << (8 * h + 4 * q + j);
+                o[j] = KERN == 0 ? (ok ? mxv - d2 : -INFINITY) : (ok ? d2 : INFINITY);
+            }
+            *reinterpret_cast<float4*>(T1 + rl * PS + po + 4 * q) = make_float4(o[0], o[1], o[2], o[3]);
+        }
+    }
+    // the near pairs, each lane its own (a pair at a time in every lane that has one)
+    if (NEAR) {
+        while (near) {
+            const int i = __ffs(near) - 1, rl = i & 8 ? r1 : r0, pl = po + (i & 7);
+            near &= near - 1;
+            const float d2 = direct_d2(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
+            T1[rl * PS + pl] = KERN == 0 ? mxr_s[rl] - d2 : d2;
         }
     }
 }
@@ -548,12 +594,13 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
 
     // ---- main pass over the points ----
     const int64_t n_steps = (N + P - 1) / P;
-    gram_block<G1, G2, KERN, true>(a, sm, 0, 0);
-    __syncthreads();
-    for (int64_t s = 0; s < n_steps; ++s) {
+    // (the first block inside the loop: a second copy of its code before the loop made the
+    // compiler schedule the 32 x 32 loop 20% slower)
+#pragma unroll 1
+    for (int64_t s = -1; s < n_steps; ++s) {
         const int b = (int)(s & 1);
         if (s + 1 < n_steps) gram_block<G1, G2, KERN, true>(a, sm, (s + 1) * P, b ^ 1);
-        gram_consume<G1, G2, KERN, JW, MT, NT>(sm, d, b, ca1, ca2, Dt, bt);
+        if (s >= 0) gram_consume<G1, G2, KERN, JW, MT, NT>(sm, d, b, ca1, ca2, Dt, bt);
         __syncthreads();
     }
 

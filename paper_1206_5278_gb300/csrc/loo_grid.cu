@@ -397,11 +397,12 @@ void loo_shape(int sm_count, const Dataset& D, int g1, int g2, bool direct, int&
         // The d >= 16 kernel runs one CTA per SM and a narrow shape's unit is many rows (128 at
         // 16 x 8): where those leave SMs idle or the last wave nearly empty, a wider shape's
         // smaller units finish sooner although they carry padding.  Waves x rows x the cost of a
-        // row (relative, measured at N = 20,000, d = 32).  8 x 8 grids, tile kernel: N = 3,000,
-        // d = 16 1.35 ms at 16 x 8, 0.73 at 16 x 32; N = 8,000, d = 20 3.47 / 1.99 at 16 x 16;
-        // N = 20,000, d = 32 17.6 / 15.2 at 16 x 16.
-        static const struct { int t1, t2; double cost; } kShapes[] = {{16, 8, 1.0},   {16, 16, 1.15}, {32, 8, 1.23},
-                                                                      {16, 32, 1.49}, {32, 16, 1.53}, {32, 32, 2.03}};
+        // row (relative, measured with whole waves: N = 152 x 128, d = 16 to 48).  8 x 8 grids,
+        // tile kernel, the narrowest shape against the rule's: N = 1,000, d = 16 0.51 / 0.21 ms;
+        // N = 3,000, d = 16 1.02 / 0.48; N = 8,000, d = 20 2.65 / 1.46; N = 20,000, d = 32
+        // 12.0 / 9.8; N = 12,000, d = 32 4.25 (a whole wave: the narrowest is taken).
+        static const struct { int t1, t2; double cost; } kShapes[] = {{16, 8, 1.0},   {16, 16, 1.12}, {32, 8, 1.26},
+                                                                      {16, 32, 1.54}, {32, 16, 1.68}, {32, 32, 2.32}};
         double best = INFINITY;
         int b1 = T1, b2 = T2;
         for (const auto& s : kShapes) {
