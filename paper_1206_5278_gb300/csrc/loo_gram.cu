@@ -33,7 +33,7 @@
 // distance, lowered by 2^-16 (n_j + n_i) (four times the Gram error bound), can lie in
 // a cell's box get their distance recomputed directly, and everything after that is
 // direct arithmetic.  (Two passes, the first for every cell's minimiser through the rows'
-// Pareto fronts, took 35 of the 87 ms of a 32 x 32 grid at N = 40,009, d = 32; this one about 10 of 55, 7 of them the scan.)
+// Pareto fronts, took 35 of the 87 ms of a 32 x 32 grid at N = 40,009, d = 32; this one about 8 of 51.)
 // The log-numerators go to a per-CTA FP64 buffer;
 // the unit's FP64 log-ratios are then summed over its rows in row order into
 // the unit's partial slot, and k_loo_final sums the slots in order: results are
@@ -89,11 +89,12 @@ constexpr int kGramLoadSteps = 2;             // k-steps of 8 dimensions whose p
 constexpr float kGramNear = 1.0f / 32.0f;     // direct recomputation below this share of n_j + n_i
 constexpr float kGramSlack = 1.0f / 65536.0f; // pre-test widening, times n_j + n_i
 
-// direct FP32 squared distance, the tile body's order (dimension 0 first, fmaf)
+// direct FP32 squared distance, the tile body's order (dimension 0 first, fmaf); U loads in flight
+template <int U>
 __device__ __forceinline__ float direct_d2(const float* __restrict__ xr, const float* __restrict__ xs,
                                            int64_t p, int d, int64_t Np) {
     float d2 = 0.f;
-#pragma unroll 8
+#pragma unroll U
     for (int c = 0; c < d; ++c) {
         const float q = xr[c] - xs[(int64_t)c * Np + p];
         d2 = fmaf(q, q, d2);
@@ -227,7 +228,7 @@ __device__ __forceinline__ void gram_block(const LooArgs& a, float* sm, int64_t 
         while (near) {
             const int i = __ffs(near) - 1, rl = i & 8 ? r1 : r0, pl = po + (i & 7);
             near &= near - 1;
-            const float d2 = direct_d2(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
+            const float d2 = direct_d2<8>(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
             T1[rl * PS + pl] = KERN == 0 ? mxr_s[rl] - d2 : d2;
         }
     }
@@ -436,11 +437,11 @@ __device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk
 
 // The recomputation's pass over a step's block, for this warp's rows with flagged cells
 // of the current round.  Lanes first take the points (the staircase test on the block's
-// distance, then on the direct one), then the row's cells: each point that passes is
-// broadcast to all lanes, and lane f % 32 updates cell f, which only it owns (no atomics;
-// each cell sees the points in step, chunk and lane order, so the sums are
-// reproducible).  A point below a cell's anchor rescales the sum and becomes the anchor;
-// the staircase follows the anchors down.
+// distance, then, for up to 32 of them at a time, on the direct one), then the row's cells:
+// each point that passes is broadcast to all lanes, and lane f % 32 updates cell f, which
+// only it owns (no atomics; each cell sees the points in step, chunk and lane order, so the
+// sums are reproducible).  A point below a cell's anchor rescales the sum and becomes the
+// anchor; the staircase follows the anchors down.
 template <int G1, int G2, int JW>
 __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_t p0, int buf, float T,
                                              GramStair (&st)[JW]) {
@@ -463,28 +464,25 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
     float* dys = sm + C::o_dys(d);
     const int* rbn = reinterpret_cast<const int*>(sm + C::o_rp(d) + 4 * R);
     unsigned int* bk = reinterpret_cast<unsigned int*>(sm + C::o_sx(d)) + 32 * warp;
+    int* hits = reinterpret_cast<int*>(sm + C::o_sy(d)) + 64 * warp;   // up to 31 waiting and a chunk's 32
 #pragma unroll
     for (int r = 0; r < JW; ++r) {   // unrolled: st[r] stays in registers
         const int rl = warp * JW + r;
         const int fb = rbn[rl], fn = rbn[R + rl];
         if (fn == 0) continue;
         const float mxv = mxr_s[rl], myv = myr_s[rl], yv = yr_s[rl], nr = nr_s[rl];
-#pragma unroll 1
-        for (int c = 0; c < C::CPS; ++c) {
-            const int pl = 32 * c + lane;
-            const float t1v = T1[rl * PS + pl];
-            const bool live = t1v > -INFINITY;                       // not a masked pair
-            const float Xg = -t1v - kGramSlack * (nr + NPs[pl]);     // the lowest the exact X can be
+        // the points that pass, in order, collected over the step's chunks: their direct
+        // distances wait for L2 once per 32 of them (once per chunk with such a point: 32 x 32
+        // at N = 40,009, d = 32 55.2 ms, now 51.3)
+        int n = 0;
+        const auto batch = [&](int cnt) {
+            const int pl = lane < cnt ? hits[lane] : 0;
+            float d2 = INFINITY;
+            if (lane < cnt) d2 = direct_d2<16>(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
             const float dy = yv - Ys[pl];
             const float dy2 = __fmul_rn(dy, dy);
-            const float Y = dy2 - myv;
-            const bool pre = st[r].in(Xg, Y) && live;
-            if (!__any_sync(0xffffffffu, pre)) continue;
-            float d2 = INFINITY;
-            if (pre) d2 = direct_d2(rows_s + rl * KS, a.xs, p0 + pl, d, Np);
-            const bool in = st[r].in(d2 - mxv, Y) && pre;
+            const bool in = st[r].in(d2 - mxv, dy2 - myv) && lane < cnt;
             unsigned int m = __ballot_sync(0xffffffffu, in);
-            if (m == 0u) continue;
             bool moved = false;
             while (m) {
                 const int src = __ffs(m) - 1;
@@ -507,6 +505,41 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
                 __syncwarp();
                 gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxv, myv, T);
             }
+        };
+constexpr int W = C::CPS < 4 ? C::CPS : 4;   // chunks tested together (2: 52.8 ms, 4: 51.3)
+#pragma unroll 1
+        for (int c = 0; c < C::CPS; c += W) {
+            unsigned int m[W];
+#pragma unroll
+            for (int h = 0; h < W; ++h) {
+                const int pl = 32 * (c + h) + lane;
+                const float t1v = T1[rl * PS + pl];
+                const bool live = t1v > -INFINITY;                       // not a masked pair
+                const float Xg = -t1v - kGramSlack * (nr + NPs[pl]);     // the lowest the exact X can be
+                const float dy = yv - Ys[pl];
+                const bool pre = st[r].in(Xg, __fmul_rn(dy, dy) - myv) && live;
+                m[h] = __ballot_sync(0xffffffffu, pre);
+            }
+#pragma unroll
+            for (int h = 0; h < W; ++h) {
+                if (m[h] == 0u) continue;
+                if (m[h] >> lane & 1u) hits[n + __popc(m[h] & ((1u << lane) - 1u))] = 32 * (c + h) + lane;
+                n += __popc(m[h]);
+                __syncwarp();
+                if (n >= 32) {
+                    batch(32);
+                    n -= 32;
+                    __syncwarp();
+                    const int mv = lane < n ? hits[32 + lane] : 0;
+                    __syncwarp();
+                    if (lane < n) hits[lane] = mv;
+                    __syncwarp();
+                }
+            }
+        }
+        if (n > 0) {
+            batch(n);
+            __syncwarp();
         }
     }
 }
