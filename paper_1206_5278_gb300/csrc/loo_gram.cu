@@ -506,7 +506,7 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
                 gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxv, myv, T);
             }
         };
-constexpr int W = C::CPS < 4 ? C::CPS : 4;   // chunks tested together (2: 52.8 ms, 4: 51.3)
+        constexpr int W = C::CPS < 4 ? C::CPS : 4;   // chunks tested together (2: 52.8 ms, 4: 51.3)
 #pragma unroll 1
         for (int c = 0; c < C::CPS; c += W) {
             unsigned int m[W];
