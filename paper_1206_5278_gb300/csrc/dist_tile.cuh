@@ -10,7 +10,7 @@
 // accumulated dimension 0 first, one fused multiply-add per dimension on the
 // rounded difference: bitwise every other pair kernel's value.
 //
-// Measured, dataset shifts: N = 24,007, d = 12: 5.5 -> 0.85 ms; N = 100,003, d = 32:
+// Measured, dataset shifts: N = 24,007, d = 12: 5.5 -> 0.71 ms; N = 100,003, d = 32:
 // 129 -> 23 ms (before: one row per thread, coordinates past the eighth re-read from
 // global memory for every pair, one CTA per 256 rows).  At N = 50,000 a dimension costs
 // 0.0167 clocks per pair and SM (0.0156: the FMA pipe), the two running keys 0.18 (the
