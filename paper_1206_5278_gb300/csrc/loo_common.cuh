@@ -194,6 +194,36 @@ struct CoefParam {
 // the tile body's factors do
 constexpr float kFbEx2Fix = 7.39e-8f;
 
+// An anchor of the one-pass recomputation moves once a term would exceed 2^kFbMove of its
+// scale: the terms within 20 of the minimum see a handful of moves.  (Anchors that follow
+// every lower point were off by 7.0e-5 where N = 100,000 rows lie in descending order of e.)
+constexpr float kFbMove = 4.f;
+
+// 2^e (e <= 0, or the rounding of a 0) as (1 + p) m, applied to about an ulp (ex2.approx alone is off by two, the
+// same way at every move): m = 2^n, n = round(e), p the Taylor series of exp((e - n) ln 2) - 1
+struct Exp2Scale {
+    float p, m;
+    __device__ __forceinline__ explicit Exp2Scale(float e) {
+        const float n = rintf(fmaxf(e, -126.f));
+        const float z = fmaxf(e - n, -0.5f) * 0.693147181f;
+        p = fmaf(z, 1.f / 5040.f, 1.f / 720.f);
+        p = fmaf(z, p, 1.f / 120.f);
+        p = fmaf(z, p, 1.f / 24.f);
+        p = fmaf(z, p, 1.f / 6.f);
+        p = fmaf(z, p, 0.5f);
+        p = fmaf(z * z, p, z);
+        m = __int_as_float(((int)n + 127) << 23);
+    }
+    __device__ __forceinline__ float operator()(float v) const { return fmaf(v, p, v) * m; }
+};
+
+// s + v into the unevaluated sum s + c (Knuth's two-sum)
+__device__ __forceinline__ void add_two(float& s, float& c, float v) {
+    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+    s = t;
+}
+
 // Exact joint-shift recomputation of the flagged cells of one unit (whole
 // CTA).  For a cell (row j, k, l) let e_i = a1_k (dx2_i - m_x,j) + a2_l (dy2_i - m_y,j).
 // Then At = sum_i 2^{-e_i} = 2^{-e_a} S with S = sum_i 2^{-(e_i - e_a)} for any anchor
@@ -201,11 +231,17 @@ constexpr float kFbEx2Fix = 7.39e-8f;
 // differences of distances (no cancellation at large e), and log2 At = -e_a + log2 S
 // with e_a in FP64.  One pass over the points: every warp takes chunks of 64
 // consecutive points (two per lane, packed FP32x2 distances, the tile body's formula)
-// and keeps, per flagged cell, its own anchor -- the smallest e it has met -- and the
-// sum relative to it; a point below the anchor rescales the sum and becomes the anchor.
-// All anchors start at the better of the x-nearest and the y-nearest point (their
-// distances are stored with the dataset), so the warps' sums never overflow (terms are
-// at most 1), and the warps are merged in fixed order at the lowest anchor.
+// and keeps, per flagged cell, its own anchor -- a point within 2^kFbMove of the smallest e
+// it has met -- and the sum relative to it; a point further below rescales the sum and
+// becomes the anchor.  All anchors start at the better of the x-nearest and the y-nearest
+// point (their distances are stored with the dataset), so the warps' sums never overflow
+// (terms are at most 2^kFbMove), and the warps are merged in fixed order at the lowest anchor.
+//
+// Precision.  A chunk's terms are summed in four floats (at most 16 terms each), which are
+// added to the cell's sum with a compensated add: the error of 18 FP32 additions, whatever N
+// is (the two-pass form: of 32; one running float: 3.1e-5 on 20,000 tied points).  The
+// compensation and the low parts' 4 bytes per cell and warp cost 3.71 -> 3.74 ms of a new
+// dataset with a 4 x 4 grid at N = 24,007, d = 12.
 //
 // Candidates.  A term with e_i > e_a + T, T = 32 + ceil(log2 N), adds less than 2^-T of
 // the cell's sum (all of them together less than 2^-32), so only points with
@@ -237,7 +273,8 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
     double* la2 = reinterpret_cast<double*>(sm);
     float* As = sm + 2 * JG;                       // the round's cells: coefficients
     float* Bs = sm + 3 * JG;
-    float* Ss = sm + C::off_fbS(d);                // [warp][CAP] sums, then the anchors' dx2, dy2
+    float* Ss = sm + C::off_fbS(d);                // [warp][CAP] sums and their low parts; the anchors' dx2, dy2
+    float* Cs = sm + C::off_fbC(d);
     float* Xs = sm + C::off_fbX(d);
     float* Ys = Xs + NW * CAP;
     // per warp: a chunk's candidates of one row, and the rows' boxes; then the row ranges
@@ -249,6 +286,7 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
     int* rs = reinterpret_cast<int*>(fbw + NW * 144);   // cells [rs, re) of the row in the round
     int* re = rs + 8;
     float* Sw = Ss + warp * CAP;
+    float* Cw = Cs + warp * CAP;
     float* Xw = Xs + warp * CAP;
     float* Yw = Ys + warp * CAP;
 
@@ -298,7 +336,7 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
             const float X0 = xn ? mx_s[r] : qx, Y0 = xn ? qy : my_s[r];
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
-                Ss[w * CAP + f] = 0.f;
+                Ss[w * CAP + f] = Cs[w * CAP + f] = 0.f;
                 Xs[w * CAP + f] = X0;
                 Ys[w * CAP + f] = Y0;
             }
@@ -357,27 +395,47 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
                     lx[p + in0] = dx2.y;
                     ly[p + in0] = dy2.y;
                 }
-                __syncwarp();
                 const int nc = __popc(m0) + __popc(m1);
+                if (lane < (-nc & 3)) lx[nc + lane] = ly[nc + lane] = INFINITY;   // up to a multiple of four
+                __syncwarp();
                 bool moved = false;
                 for (int f = f0 + lane; f < f1; f += 32) {
                     const float A = As[f], B = Bs[f];
-                    float X = Xw[f], Y = Yw[f], S = Sw[f];
-                    for (int q = 0; q < nc; ++q) {
-                        const float qx = lx[q], qy = ly[q];
-                        float e = fmaf(A, qx - X, B * (qy - Y));
-                        if (e < 0.f) {   // a lower point: the new anchor
-                            S *= ex2_approx(kFbEx2Fix + e);
-                            X = qx;
-                            Y = qy;
-                            e = 0.f;
+                    float X = Xw[f], Y = Yw[f], S = Sw[f], Sc = Cw[f];
+                    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll 1
+                    for (int q = 0; q < nc; q += 4) {
+                        const float4 qx = *reinterpret_cast<const float4*>(lx + q);
+                        const float4 qy = *reinterpret_cast<const float4*>(ly + q);
+                        const auto ex = [&](float x, float y) { return fmaf(A, x - X, B * (y - Y)); };
+                        float e0 = ex(qx.x, qy.x), e1 = ex(qx.y, qy.y), e2 = ex(qx.z, qy.z), e3 = ex(qx.w, qy.w);
+                        const float lo = fminf(fminf(e0, e1), fminf(e2, e3));
+                        if (lo < -kFbMove) {   // a lower point: the new anchor
+                            const Exp2Scale by(lo);
+                            S = by(S);
+                            Sc = by(Sc);
+                            s0 = by(s0);
+                            s1 = by(s1);
+                            s2 = by(s2);
+                            s3 = by(s3);
+                            X = lo == e0 ? qx.x : lo == e1 ? qx.y : lo == e2 ? qx.z : qx.w;
+                            Y = lo == e0 ? qy.x : lo == e1 ? qy.y : lo == e2 ? qy.z : qy.w;
+                            e0 = ex(qx.x, qy.x);
+                            e1 = ex(qx.y, qy.y);
+                            e2 = ex(qx.z, qy.z);
+                            e3 = ex(qx.w, qy.w);
                             moved = true;
                         }
-                        S += ex2_approx(kFbEx2Fix - e);
+                        s0 += ex2_approx(kFbEx2Fix - e0);
+                        s1 += ex2_approx(kFbEx2Fix - e1);
+                        s2 += ex2_approx(kFbEx2Fix - e2);
+                        s3 += ex2_approx(kFbEx2Fix - e3);
                     }
+                    add_two(S, Sc, (s0 + s1) + (s2 + s3));
                     Xw[f] = X;
                     Yw[f] = Y;
                     Sw[f] = S;
+                    Cw[f] = Sc;
                 }
                 __syncwarp();
                 if (__any_sync(0xffffffffu, moved)) box(r, f0, f1);
@@ -400,11 +458,12 @@ __device__ __forceinline__ void loo_fallback(const LooArgs& a, const Coef& cf, f
                     Y = Yo;
                 }
             }
-            float tot = 0.f;
+            float tot = 0.f, low = 0.f;
 #pragma unroll
             for (int w = 0; w < NW; ++w)
-                tot += Ss[w * CAP + f] *
-                       ex2_approx(kFbEx2Fix - fmaf(A, Xs[w * CAP + f] - X, B * (Ys[w * CAP + f] - Y)));
+                add_two(tot, low, Exp2Scale(-fmaf(A, Xs[w * CAP + f] - X, B * (Ys[w * CAP + f] - Y)))(
+                                      Ss[w * CAP + f] + Cs[w * CAP + f]));
+            tot += low;
             const double e = (double)A * ((double)X - (double)mx_s[r]) + (double)B * ((double)Y - (double)my_s[r]);
             la2[c] = -e + log2_wide(tot);
         }

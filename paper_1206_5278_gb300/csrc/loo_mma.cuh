@@ -94,19 +94,23 @@ struct MmaCfg {
     __host__ __device__ static int off_nflag(int d) { return off_flag(d) + 1024; }
     // exact recomputation: per warp a list of 64 candidate points and the rows' boxes,
     // then per row (at most 8) its cell range; per round of FBCAP cells the warps' sums
-    // (behind the coefficients in the combine buffer) and anchors (over the running totals)
+    // (behind the coefficients in the combine buffer), their low parts (behind the running
+    // totals) and anchors (over the running totals)
     static constexpr bool kOnePass = GG < 1024;   // see loo_fallback_two_pass
     static constexpr int FBCAP = 512;
     static constexpr int FBW = kWarps * 144 + 2 * 8;
     __host__ __device__ static int off_fbw(int d) { return off_nflag(d) + 32; }
     __host__ __device__ static int off_fbS(int) { return 4 * JW * GG; }
     __host__ __device__ static int off_fbX(int d) { return off_dts(d); }
+    __host__ __device__ static int off_fbC(int d) { return off_dts(d) + kWarps * 1024; }
     static_assert(4 * JW * GG + kWarps * FBCAP <= COMB, "the sums fit behind the coefficients");
     static_assert(2 * kWarps * FBCAP <= kWarps * 1024, "the anchors fit over the running totals");
     // per warp the FP32 running totals of its 1024 cells in MMA fragment order
     // (lane-contiguous float4 per (row, M tile, N tile): conflict-free)
     __host__ __device__ static int off_dts(int d) { return (off_fbw(d) + FBW + 3) & ~3; }
-    static size_t smem_bytes(int d) { return (size_t)(off_dts(d) + kWarps * 1024) * sizeof(float); }
+    static size_t smem_bytes(int d) {
+        return (size_t)(off_fbC(d) + (kOnePass ? kWarps * FBCAP : 0)) * sizeof(float);
+    }
 };
 
 __device__ __forceinline__ uint32_t tf32_rna(float v) {

@@ -48,7 +48,7 @@ struct PackCfg {
     static constexpr int WST = (JW / 2) * T1S + JW * T2S;
     static constexpr int COMB = kWarps * JW * GG + kWarps * JW * K1;
     __host__ __device__ static int big(int) {
-        const int s = kWarps * WST, f = 28 * JW * GG;   // f: the exact recomputation
+        const int s = kWarps * WST, f = 36 * JW * GG;   // f: the exact recomputation
         const int m = s > COMB ? s : COMB;
         return m > f ? m : f;
     }
@@ -71,6 +71,7 @@ struct PackCfg {
     __host__ __device__ static int off_fbw(int d) { return off_nflag(d) + 32; }
     __host__ __device__ static int off_fbS(int) { return 4 * JW * GG; }
     __host__ __device__ static int off_fbX(int) { return (4 + kWarps) * JW * GG; }
+    __host__ __device__ static int off_fbC(int) { return (4 + 3 * kWarps) * JW * GG; }
     static size_t smem_bytes(int d) { return (size_t)(off_fbw(d) + FBW) * sizeof(float); }
     // position of row r in the pair order: its pair (one row of each half of the M
     // tile), then its half
