@@ -440,8 +440,8 @@ __device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk
 // distance, then, for up to 32 of them at a time, on the direct one), then the row's cells:
 // each point that passes is broadcast to all lanes, and lane f % 32 updates cell f, which
 // only it owns (no atomics; each cell sees the points in step, chunk and lane order, so the
-// sums are reproducible).  A point below a cell's anchor rescales the sum and becomes the
-// anchor; the staircase follows the anchors down.
+// sums are reproducible).  A point more than kFbMove below a cell's anchor rescales the sum and
+// becomes the anchor; the staircase follows the anchors down.
 template <int G1, int G2, int JW>
 __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_t p0, int buf, float T,
                                              GramStair (&st)[JW]) {
@@ -491,7 +491,7 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
                 for (int f = fb + lane; f < fb + fn; f += 32) {
                     float e = fmaf(As[f], d2q - dxs[f], Bs[f] * (dy2q - dys[f]));
                     float S = sum[f];
-                    if (e < 0.f) {
+                    if (e < -kFbMove) {
                         S *= ex2_approx(kFbEx2Fix + e);
                         dxs[f] = d2q;
                         dys[f] = dy2q;
