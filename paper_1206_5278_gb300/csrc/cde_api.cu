@@ -169,7 +169,9 @@ void cde_shutdown(cde_ctx* ctx) {
     if (!ctx) return;
     cde_server_stop_internal(ctx);
     cudaSetDevice(ctx->device);
-    cudaStreamSynchronize(ctx->stream);
+    // calls with device outputs may still be running on their callers' streams: the datasets
+    // they read are given back in the order of the context's stream, which does not wait for those
+    cudaDeviceSynchronize();
     batch_plan_free(ctx);
     {
         std::lock_guard<std::mutex> g(ctx->ds_mu);
