@@ -53,7 +53,7 @@ static void free_dataset(cde_ctx* ctx, Dataset* D) {
 __global__ void k_finite_check(const float* a, int64_t n, int* flag) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        if (!isfinite(a[i])) atomicOr(flag, 1);
+        if (!isfinite(a[i])) atomicOr(flag, kBadFinite);
 }
 
 }  // namespace cde
@@ -226,7 +226,7 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
         cudaStreamSynchronize(st);
         return r;
     };
-    // one allocation: xs, y, mx, my, qx, qy, then the statistics with the word of the finite check
+    // one allocation: xs, y, mx, my, qx, qy, then the statistics with the word that refuses
     const auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t bx = pad((size_t)D->Np * d * 4), by = pad((size_t)D->Np * 4), bn = pad((size_t)N * 4);
     const size_t stats_bytes = (size_t)2 * d * sizeof(double);
@@ -241,7 +241,7 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
     D->qy = reinterpret_cast<float*>(m += bn);
     D->stats = reinterpret_cast<double*>(m += bn);
     int* flag = reinterpret_cast<int*>(m + stats_bytes);
-    // the statistics and the finite check are read back once, at the end (small, page-locked)
+    // the statistics and that word are read back once, at the end (small, page-locked)
     rc = workspace_reserve(ctx, 0, 2 * kMaxD * sizeof(double) + sizeof(int));
     if (rc != CDE_OK) return fail(rc);
     double* stats = static_cast<double*>(ctx->ws_host);
@@ -266,10 +266,10 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
         if (e == cudaSuccess) e = cudaMemcpyAsync(dy, y, (size_t)N * 4, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: upload"));
     }
-    rc = pack_enqueue(*D, dx, dy, st, D->stats);
+    rc = pack_enqueue(*D, dx, dy, st, D->stats, flag);
     if (rc != CDE_OK) return fail(rc);
     if (D->kernel == CDE_KERNEL_GAUSS) {
-        rc = nn_shift_enqueue(ctx, *D, st);
+        rc = nn_shift_enqueue(ctx, *D, st, flag);
         if (rc != CDE_OK) return fail(rc);
     } else {
         e = cudaMemsetAsync(D->mx, 0, 4 * bn, st);   // mx, my, qx, qy
@@ -279,12 +279,9 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
     cudaError_t e2 = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = e2;
     if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: kernels"));
-    if (*reinterpret_cast<const int*>(stats + 2 * d))
-        return fail(set_error(CDE_EINVAL, "cde_create_dataset: non-finite input"));
-    if (standardize)
-        for (int c = 0; c < d; ++c)
-            if (!(stats[2 * c + 1] > 0.0))
-                return fail(set_error(CDE_EINVAL, "cde_create_dataset: zero spread in a dimension"));
+    const int bad = *reinterpret_cast<const int*>(stats + 2 * d);
+    if (bad & kBadFinite) return fail(set_error(CDE_EINVAL, "cde_create_dataset: non-finite input"));
+    if (bad & kBadSpread) return fail(set_error(CDE_EINVAL, "cde_create_dataset: zero spread in a dimension"));
     if (!in_dev) {
         cudaFreeAsync(dx, st);
         cudaFreeAsync(dy, st);

@@ -242,12 +242,16 @@ class HostCopies {
     size_t used_ = 0;
 };
 
+// Device word of a dataset in the making: why it will be refused (bits; 0: it will not).
+// The O(N^2 d) kernels return at once when it is set.
+constexpr int kBadFinite = 1, kBadSpread = 2;
+
 // Nearest squared distances per row (cached at dataset creation).
-int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st);
+int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st, const int* d_bad);
 
 // Standardise / pack raw row-major x into the SoA layout (device input).
 int pack_enqueue(Dataset& D, const float* d_x_rowmajor, const float* d_y, cudaStream_t st,
-                 double* d_stats);
+                 double* d_stats, int* d_bad);
 
 // ---- gradient (loo_grad.cu) ----
 // d_rowv (optional, N x 3 doubles) receives per-row {ell_j, d ell_j/d ln h1, d ell_j/d ln h2}.

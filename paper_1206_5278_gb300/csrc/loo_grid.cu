@@ -44,7 +44,7 @@ namespace cde {
 // --------------------------------------------------------------------------
 // Dataset packing: optional FP64 standardisation, row-major -> SoA.
 // --------------------------------------------------------------------------
-__global__ void k_col_stats(const float* __restrict__ x, int64_t N, int d, double* stats) {
+__global__ void k_col_stats(const float* __restrict__ x, int64_t N, int d, double* stats, int* bad) {
     // one CTA per column: mean, then sum of squared deviations (fixed-order tree)
     __shared__ double red[1024];
     const int c = blockIdx.x;
@@ -71,7 +71,9 @@ __global__ void k_col_stats(const float* __restrict__ x, int64_t N, int d, doubl
     }
     if (threadIdx.x == 0) {
         stats[2 * c] = mean;
-        stats[2 * c + 1] = sqrt(red[0] / (double)(N - 1));
+        const double sd = sqrt(red[0] / (double)(N - 1));
+        stats[2 * c + 1] = sd;
+        if (bad && !(sd > 0.0)) atomicOr(bad, kBadSpread);
     }
 }
 
@@ -93,9 +95,9 @@ __global__ void k_pack(const float* __restrict__ x, const float* __restrict__ y,
     ys[i] = i < N ? y[i] : 0.f;
 }
 
-int pack_enqueue(Dataset& D, const float* d_x, const float* d_y, cudaStream_t st, double* d_stats) {
+int pack_enqueue(Dataset& D, const float* d_x, const float* d_y, cudaStream_t st, double* d_stats, int* d_bad) {
     if (D.standardized) {
-        k_col_stats<<<D.d, 1024, 0, st>>>(d_x, D.N, D.d, d_stats);
+        k_col_stats<<<D.d, 1024, 0, st>>>(d_x, D.N, D.d, d_stats, d_bad);
         CDE_CUDA(cudaGetLastError());
     }
     const int64_t blocks = (D.Np + 255) / 256;
@@ -116,6 +118,8 @@ int pack_enqueue(Dataset& D, const float* d_x, const float* d_y, cudaStream_t st
 // a1 (dx^2 - m_x) + a2 (dy^2 - m_y) (a1, a2 > 0) has dx^2 <= qx and dy^2 <= qy
 // (it can be no worse than either neighbour), which is what the exact
 // fallback of the grid kernels uses to skip points.
+// Nothing is done for a dataset that will be refused (*bad): the word is on the device, and
+// the host reads it once, after these kernels.
 // --------------------------------------------------------------------------
 
 // d <= 8: four rows per thread, point-major shared tiles (128-bit loads), the
@@ -135,10 +139,12 @@ template <int DREG>
 __global__ void __launch_bounds__(kNnThreads) k_nn_shift_split(const float* __restrict__ xs,
                                                                const float* __restrict__ y, int64_t N,
                                                                int64_t Np, int d, int64_t i_per_split,
+                                                               const int* __restrict__ bad,
                                                                unsigned long long* __restrict__ kx,
                                                                unsigned long long* __restrict__ ky) {
     __shared__ __align__(16) float xt[kNnThreads][DREG];
     __shared__ float yt[kNnThreads];
+    if (*bad) return;
     const int tid = threadIdx.x;
     const int64_t jbase = (int64_t)blockIdx.x * kNnThreads * kNnJB + tid;
     const int64_t i0 = (int64_t)blockIdx.y * i_per_split;
@@ -217,9 +223,11 @@ __global__ void __launch_bounds__(kNnThreads) k_nn_shift_split(const float* __re
 __global__ void __launch_bounds__(kDtThreads, 2) k_nn_shift_tile(const float* __restrict__ xs,
                                                                   const float* __restrict__ y, int64_t N, int64_t Np,
                                                                   int d, int64_t i_per_split,
+                                                                  const int* __restrict__ bad,
                                                                   unsigned long long* __restrict__ kx,
                                                                   unsigned long long* __restrict__ ky) {
     extern __shared__ float4 dt4[];
+    if (*bad) return;
     float* rows = reinterpret_cast<float*>(dt4);
     float* pbuf = rows + d * kDtRows;
     const int nbuf = (d + 1) * kDtPts;
@@ -308,7 +316,7 @@ __global__ void k_nn_unpack(const unsigned long long* __restrict__ kx, const uns
     qx[j] = __uint_as_float((unsigned int)b);
 }
 
-int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st) {
+int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st, const int* d_bad) {
     const int sm_count = ctx->sm_count;
     unsigned long long* keys = nullptr;   // [2][N] merge keys, stream-ordered scratch
     CDE_CUDA(pool_alloc(ctx, (void**)&keys, (size_t)2 * D.N * sizeof(unsigned long long), st));
@@ -326,9 +334,11 @@ int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st) {
         ns = (tiles + tps - 1) / tps;
         const dim3 grid((unsigned)gx, (unsigned)ns);
         if (D.d <= 4)
-            k_nn_shift_split<4><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, keys, keys + D.N);
+            k_nn_shift_split<4><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, d_bad, keys,
+                                                             keys + D.N);
         else
-            k_nn_shift_split<8><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, keys, keys + D.N);
+            k_nn_shift_split<8><<<grid, kNnThreads, 0, st>>>(D.xs, D.y, D.N, D.Np, D.d, tps * kNnThreads, d_bad, keys,
+                                                             keys + D.N);
     } else {
         const int64_t gx = (D.N + kDtRows - 1) / kDtRows;
         int64_t ns = 1;
@@ -336,7 +346,7 @@ int nn_shift_enqueue(cde_ctx* ctx, const Dataset& D, cudaStream_t st) {
         static std::atomic<uint64_t> attr{0};
         CDE_CUDA(smem_attr_once(attr, k_nn_shift_tile, dt_smem_floats(kMaxD, true) * (int)sizeof(float)));
         k_nn_shift_tile<<<dim3((unsigned)gx, (unsigned)ns), kDtThreads, dt_smem_floats(D.d, true) * sizeof(float), st>>>(
-            D.xs, D.y, D.N, D.Np, D.d, ips, keys, keys + D.N);
+            D.xs, D.y, D.N, D.Np, D.d, ips, d_bad, keys, keys + D.N);
     }
     CDE_CUDA(cudaGetLastError());
     k_nn_unpack<<<(unsigned)((D.N + 255) / 256), 256, 0, st>>>(keys, keys + D.N, D.N, D.mx, D.my, D.qx, D.qy);

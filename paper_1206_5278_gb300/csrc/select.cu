@@ -23,7 +23,7 @@
 
 namespace cde {
 
-__global__ void k_col_stats(const float* __restrict__ x, int64_t N, int d, double* stats);
+__global__ void k_col_stats(const float* __restrict__ x, int64_t N, int d, double* stats, int* bad);
 
 // SplitMix64 (Steele, Lea & Flood, 2014) as a counter-based stream: the k-th
 // value of the stream with seed s is mix(s + (k + 1) * gamma).
@@ -74,7 +74,7 @@ extern "C" int cde_reference_rule(cde_ctx* ctx, cde_dataset ds, double* h1, doub
     // column statistics of the stored (possibly standardised) x and of y
     for (int c = 0; c <= d; ++c) {
         const float* col = c < d ? D->xs + (int64_t)c * D->Np : D->y;
-        k_col_stats<<<1, 1024, 0, st>>>(col, D->N, 1, dstats + 2 * c);
+        k_col_stats<<<1, 1024, 0, st>>>(col, D->N, 1, dstats + 2 * c, nullptr);
     }
     cudaError_t e = cudaGetLastError();
     std::vector<double> stats(2 * (d + 1));
