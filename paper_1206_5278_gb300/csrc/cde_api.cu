@@ -42,9 +42,18 @@ static int check_grid(const double* h, int G, const char* name) {
     return CDE_OK;
 }
 
+static cudaError_t pool_keep(cde_ctx* ctx) {
+    uint64_t keep = kPoolKeep + ctx->resident;
+    return cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
 // (no work that reads the dataset is in flight)
 static void free_dataset(cde_ctx* ctx, Dataset* D) {
-    if (D->mem) cudaFreeAsync(D->mem, ctx->stream);
+    if (D->mem) {
+        cudaFreeAsync(D->mem, ctx->stream);
+        ctx->resident -= D->mem_bytes;
+        pool_keep(ctx);
+    }
     D->mem = nullptr;
     D->xs = D->y = D->mx = D->my = D->qx = D->qy = nullptr;
     D->stats = nullptr;
@@ -143,8 +152,7 @@ int cde_init(cde_ctx** out, int device, size_t budget) {
         pp.location.type = cudaMemLocationTypeDevice;
         pp.location.id = device;
         e = cudaMemPoolCreate(&ctx->pool, &pp);
-        uint64_t keep = kPoolKeep;
-        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) e = pool_keep(ctx);
     }
     if (e != cudaSuccess) {
         if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
@@ -230,8 +238,12 @@ int cde_create_dataset(cde_ctx* ctx, const float* x, const float* y, int64_t N, 
     const auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t bx = pad((size_t)D->Np * d * 4), by = pad((size_t)D->Np * 4), bn = pad((size_t)N * 4);
     const size_t stats_bytes = (size_t)2 * d * sizeof(double);
-    cudaError_t e = pool_alloc(ctx, &D->mem, bx + by + 4 * bn + pad(stats_bytes + sizeof(int)), st);
+    const size_t mem_bytes = bx + by + 4 * bn + pad(stats_bytes + sizeof(int));
+    cudaError_t e = pool_alloc(ctx, &D->mem, mem_bytes, st);
     if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: device memory"));
+    ctx->resident += D->mem_bytes = mem_bytes;
+    e = pool_keep(ctx);
+    if (e != cudaSuccess) return fail(cuda_error(e, "cde_create_dataset: pool"));
     char* m = static_cast<char*>(D->mem);
     D->xs = reinterpret_cast<float*>(m);
     D->y = reinterpret_cast<float*>(m += bx);

@@ -76,6 +76,7 @@ struct Dataset {
     int standardized = 0;
     int kernel = 0;        // CDE_KERNEL_GAUSS or CDE_KERNEL_EPAN
     void* mem = nullptr;   // one allocation of the context's pool holds the arrays below
+    size_t mem_bytes = 0;
     float* xs = nullptr;   // [d][Np]
     float* y = nullptr;    // [Np]
     float* mx = nullptr;   // [N] min_{i!=j} |x_j - x_i|^2 (FP32, same formula as the kernels);
@@ -109,8 +110,10 @@ struct cde_ctx {
     // stream-ordered pool of every call's scratch and of the datasets.  It keeps up to
     // kPoolKeep of freed memory across synchronisations (the device's default pool keeps
     // none, so each call paid to map its scratch again: 300 us of a 370 us density request)
-    // and is destroyed at shutdown.
+    // and is destroyed at shutdown.  A pool's release threshold counts the memory in use too:
+    // it is kPoolKeep and the datasets' bytes, set as those come and go.
     cudaMemPool_t pool = nullptr;
+    size_t resident = 0;      // bytes of the datasets' allocations (guarded by mu)
     std::recursive_mutex mu;  // serialises the synchronous API
     std::mutex ds_mu;         // guards the dataset map
     std::map<int64_t, std::shared_ptr<cde::Dataset>> datasets;
