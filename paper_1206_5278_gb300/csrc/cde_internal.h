@@ -268,6 +268,7 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
 int grad_chunked_next(GradChunked* c, double pair_evals, cudaStream_t st, int* done);
 int grad_chunked_finish(cde_ctx* ctx, GradChunked* c, double* d_out3, cudaStream_t st);
 void grad_chunked_free(GradChunked* c, cudaStream_t st);
+size_t grad_scratch_bytes(const cde_ctx* ctx, const Dataset& D);   // what create allocates
 int loo_grad_enqueue(cde_ctx* ctx, const Dataset& D, double h1, double h2, double* d_out3,
                      cudaStream_t st, double* d_rowv);
 

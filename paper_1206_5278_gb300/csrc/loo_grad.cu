@@ -811,29 +811,81 @@ static int64_t grad_splits(int64_t row_ctas, int64_t tiles, int64_t slots) {
     return best;
 }
 
+// The launches and scratch of a gradient evaluation: of the dataset only
+struct GradPlan {
+    bool tc, epan;
+    int DREG, DK;
+    int JB;            // rows per thread (SIMT kernel)
+    int64_t gx, ns, i_per_split;
+    int64_t slots;     // resident CTAs of the GPU for this kernel
+    int64_t entries;   // partials of six floats: the splits', or the recomputation's
+    int64_t fb_list;   // start of the list of recomputed rows, behind their counters
+};
+
 // A gradient evaluation as a sequence of launches over ranges of row blocks.
 // Every (row block, point split) writes its own partial and the per-row
 // merge and the sums run once at the end, so the result does not depend on
 // how the row blocks are split over launches (the request loop runs
 // gradient steps this way, so queued density jobs run in between).
-struct GradChunked {
+struct GradChunked : GradPlan {
     GradArgs g;
-    bool tc, epan;
-    int DREG, DK;
-    int JB;            // rows per thread (SIMT kernel)
-    int64_t gx, ns, next_bx;
-    int64_t slots;     // resident CTAs of the GPU for this kernel
+    int64_t next_bx;
     double h1, h2;
     double* rowv;
     bool own_rowv;
     double* slots3;    // [kSumMax][3] partial sums of k_sum_rows3
     int* fb;           // recomputed rows: count, k_sum_rows3's counter, counters per four rows, then the list
-    int64_t fb_list;   // start of the list
 };
+
+static GradPlan grad_plan(const cde_ctx* ctx, const Dataset& D) {
+    GradPlan p{};
+    p.epan = D.kernel == CDE_KERNEL_EPAN;
+    p.tc = D.d >= 16;   // tensor-core cross term
+    p.DREG = D.d <= 4 ? 4 : D.d <= 8 ? 8 : D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
+    p.DK = D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
+    const int tile = p.tc ? (p.DK <= 32 ? 256 : 128) : kGradThreads;
+    const int64_t tiles = (D.N + tile - 1) / tile;
+    int64_t ns;
+    p.JB = 2;
+    if (p.tc) {
+        p.slots = ctx->sm_count;
+    } else {
+        const int per_sm = p.DREG == 4 ? grad_simt_ctas_per_sm<4, 4>()
+                           : p.DREG == 8 ? grad_simt_ctas_per_sm<4, 8>() : grad_simt_ctas_per_sm<2, 16>();
+        p.slots = (int64_t)per_sm * ctx->sm_count;
+        // four rows per thread share a point's loads (d <= 8), unless even one-tile splits
+        // would then leave the GPU part empty
+        const int64_t rows4 = (int64_t)kGradThreads * 4;
+        if (p.DREG <= 8 && (D.N + rows4 - 1) / rows4 * tiles >= p.slots) p.JB = 4;
+    }
+    const int64_t rows_per_cta = p.tc ? (int64_t)kGTRows : (int64_t)kGradThreads * p.JB;
+    p.gx = (D.N + rows_per_cta - 1) / rows_per_cta;
+    ns = grad_splits(p.gx, tiles, p.slots);
+    if (ns > tiles) ns = tiles;
+    if (ns < 1) ns = 1;
+    const int64_t tiles_per = (tiles + ns - 1) / ns;
+    p.i_per_split = tiles_per * tile;
+    p.ns = (tiles + tiles_per - 1) / tiles_per;
+    // (the recomputation reuses the splits' partials, merged by then)
+    p.entries = std::max(p.ns * D.N, p.epan ? 0 : grad_fb_entries(D.N, ctx->sm_count));
+    p.fb_list = 2 + (D.N + kFbRows - 1) / kFbRows;
+    return p;
+}
+
+// bytes of grad_chunked_create's allocations (with the rows' values)
+size_t grad_scratch_bytes(const cde_ctx* ctx, const Dataset& D) {
+    const GradPlan p = grad_plan(ctx, D);
+    const auto pad = [](size_t b) { return (b + 511) & ~(size_t)511; };   // the pool's granularity
+    size_t b = pad((size_t)p.entries * 6 * sizeof(float)) + pad((size_t)(p.fb_list + D.N) * sizeof(int)) +
+               pad((size_t)3 * kSumMax * sizeof(double)) + pad((size_t)D.N * 3 * sizeof(double));
+    if (p.tc) b += pad((size_t)2 * D.Np * p.DK * sizeof(uint32_t)) + pad((size_t)D.Np * sizeof(float));
+    return b;
+}
 
 int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cudaStream_t st, double* d_rowv_ext,
                         GradChunked** out) {
     auto* c = new GradChunked{};
+    static_cast<GradPlan&>(*c) = grad_plan(ctx, D);
     GradArgs& g = c->g;
     g.xs = D.xs;
     g.y = D.y;
@@ -843,37 +895,11 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
     g.Np = D.Np;
     g.d = D.d;
     const double L2E = 1.4426950408889634074;
-    c->epan = D.kernel == CDE_KERNEL_EPAN;
     c->h1 = h1;
     c->h2 = h2;
     g.a1 = (float)(c->epan ? 1.0 / (h1 * h1) : L2E / (2 * h1 * h1));
     g.a2 = (float)(c->epan ? 1.0 / (h2 * h2) : L2E / (2 * h2 * h2));
-    c->tc = D.d >= 16;   // tensor-core cross term
-    c->DREG = D.d <= 4 ? 4 : D.d <= 8 ? 8 : D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
-    c->DK = D.d <= 16 ? 16 : D.d <= 32 ? 32 : 64;
-    const int tile = c->tc ? (c->DK <= 32 ? 256 : 128) : kGradThreads;
-    const int64_t tiles = (D.N + tile - 1) / tile;
-    int64_t ns;
-    c->JB = 2;
-    if (c->tc) {
-        c->slots = ctx->sm_count;
-    } else {
-        const int per_sm = c->DREG == 4 ? grad_simt_ctas_per_sm<4, 4>()
-                           : c->DREG == 8 ? grad_simt_ctas_per_sm<4, 8>() : grad_simt_ctas_per_sm<2, 16>();
-        c->slots = (int64_t)per_sm * ctx->sm_count;
-        // four rows per thread share a point's loads (d <= 8), unless even one-tile splits
-        // would then leave the GPU part empty
-        const int64_t rows4 = (int64_t)kGradThreads * 4;
-        if (c->DREG <= 8 && (D.N + rows4 - 1) / rows4 * tiles >= c->slots) c->JB = 4;
-    }
-    const int64_t rows_per_cta = c->tc ? (int64_t)kGTRows : (int64_t)kGradThreads * c->JB;
-    c->gx = (D.N + rows_per_cta - 1) / rows_per_cta;
-    ns = grad_splits(c->gx, tiles, c->slots);
-    if (ns > tiles) ns = tiles;
-    if (ns < 1) ns = 1;
-    const int64_t tiles_per = (tiles + ns - 1) / ns;
-    g.i_per_split = tiles_per * tile;
-    c->ns = (tiles + tiles_per - 1) / tiles_per;
+    g.i_per_split = c->i_per_split;
     c->next_bx = 0;
     c->rowv = d_rowv_ext;
     c->own_rowv = d_rowv_ext == nullptr;
@@ -882,10 +908,7 @@ int grad_chunked_create(cde_ctx* ctx, const Dataset& D, double h1, double h2, cu
         rc = cuda_error(e, what);
         return rc;
     };
-    // (the recomputation reuses the splits' partials, merged by then)
-    const int64_t entries = std::max(c->ns * D.N, c->epan ? 0 : grad_fb_entries(D.N, ctx->sm_count));
-    c->fb_list = 2 + (D.N + kFbRows - 1) / kFbRows;
-    cudaError_t e = pool_alloc(ctx, (void**)&g.part, (size_t)entries * 6 * sizeof(float), st);
+    cudaError_t e = pool_alloc(ctx, (void**)&g.part, (size_t)c->entries * 6 * sizeof(float), st);
     if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&c->fb, (size_t)(c->fb_list + D.N) * sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->fb, 0, (size_t)c->fb_list * sizeof(int), st);
     if (e == cudaSuccess) e = pool_alloc(ctx, (void**)&c->slots3, (size_t)3 * kSumMax * sizeof(double), st);

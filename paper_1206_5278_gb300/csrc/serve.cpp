@@ -106,16 +106,18 @@ static double pct(std::vector<double> v, double p) {
     return v[lo] + (v[hi] - v[lo]) * (pos - lo);
 }
 
-static size_t job_mem(const Job& J, int sm_count) {
+static size_t job_mem(const Job& J, const cde_ctx* ctx) {
     const cde_request& r = J.req;
     if (r.kind == CDE_REQ_DENSITY) {
         const int64_t qt = (r.Q + 31) / 32;
-        const int64_t ns = std::max<int64_t>(1, (4LL * sm_count + qt - 1) / std::max<int64_t>(qt, 1));
+        const int64_t ns = std::max<int64_t>(1, (4LL * ctx->sm_count + qt - 1) / std::max<int64_t>(qt, 1));
         return (size_t)r.Q * J.D->d * 8 + (size_t)r.G_y * 4 + (size_t)r.Q * r.G_y * 4 * (2 + ns) +
                (size_t)r.Q * 16 + 4096;
     }
     const size_t tiles = (size_t)(J.D->N / 8 + 2);
-    return tiles * 2 * 1024 * 8 + (size_t)J.D->N * (6 * 4 * 16 + 24) + 65536;
+    // the grid's partials; a gradient step: 16 point splits, or its plan's where those are more
+    const size_t grad = std::max((size_t)J.D->N * (6 * 4 * 16 + 24), grad_scratch_bytes(ctx, *J.D));
+    return tiles * 2 * 1024 * 8 + grad + 65536;
 }
 
 // A job's stream: density jobs run on their slot's high-priority stream, so the
@@ -513,7 +515,8 @@ int cde_submit(cde_ctx* ctx, const cde_request* req, int64_t* ticket) {
     } else {
         return set_error(CDE_EINVAL, "cde_submit: unknown request kind");
     }
-    J->mem = job_mem(*J, ctx->sm_count);
+    CDE_CUDA(cudaSetDevice(ctx->device));
+    J->mem = job_mem(*J, ctx);
     std::lock_guard<std::mutex> g(S->mu);
     if (S->stop) return set_error(CDE_EINVAL, "cde_submit: server stopping");
     if ((int)S->queue.size() >= S->cfg.queue_capacity) return set_error(CDE_EBUSY, "cde_submit: queue full");
