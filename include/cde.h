@@ -87,7 +87,8 @@ void cde_shutdown(cde_ctx *ctx);
 /*
  * Make a dataset resident on the device.
  *   x: N x d_x row-major float32; y: N float32 (host, or device with
- *   CDE_IN_DEVICE in `flags`).  standardize != 0 centres each x dimension and
+ *   CDE_IN_DEVICE in `flags`; device arrays must be complete: the call reads
+ *   them on the context's own stream).  standardize != 0 centres each x dimension and
  *   divides it by its sample standard deviation (ddof = 1), in FP64 (Sec. 4);
  *   y is never scaled.  Requires N >= 2, d_x >= 1, finite values, and a
  *   non-zero spread in every dimension when standardising.

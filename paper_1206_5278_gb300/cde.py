@@ -220,7 +220,7 @@ def cde_shutdown(ctx) -> None:
 def cde_create_dataset(ctx, x, y, standardize: bool = False, kernel: str = "gauss") -> int:
     """x: (N, d_x) float32, y: (N,) float32 -- numpy (host) or CUDA tensors.
     kernel: "gauss" or "epan" (radial Epanechnikov, Sec. 4) for every call on
-    the dataset."""
+    the dataset.  CUDA tensors: waits for torch's current stream first."""
     if kernel not in KERNELS:
         raise ValueError("kernel must be one of %s" % sorted(KERNELS))
     dev = _is_cuda(x)
@@ -230,6 +230,10 @@ def cde_create_dataset(ctx, x, y, standardize: bool = False, kernel: str = "gaus
         xs = x.contiguous() if x.dim() == 2 else x.reshape(-1, 1).contiguous()
         ys = y.contiguous()
         N, d = int(xs.shape[0]), int(xs.shape[1])
+        # the library reads them on its own stream: what makes them (and the copies above) is
+        # on torch's current one
+        import torch
+        torch.cuda.current_stream(x.device).synchronize()
     else:
         xs = _f32(x)
         if xs.ndim == 1:
