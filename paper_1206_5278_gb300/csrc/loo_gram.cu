@@ -61,7 +61,9 @@ struct GramCfg {
     static constexpr int FMAX = 1024;                                // flagged cells per fallback round
     static_assert(CELLS == 32 * kThreads, "one flag word per thread");
     static_assert(JW * NG == kWarps, "one 16 x 32 Gram block per warp");
-    // shared memory layout in 4-byte words (KS: row stride of the staged row coordinates)
+    // shared memory layout in 4-byte words (KS: row stride of the staged row coordinates).  Half
+    // of o_sx and six of o_rp's eight rows are spare: their 5 KB keep the 16 x 8 shape on the
+    // direct kernel at d = 49 to 56, where the two have not been measured against each other.
     __host__ __device__ static int ks(int d) { return ((d + 7) & ~7) + 4; }
     __host__ __device__ static int o_rows() { return 0; }
     __host__ __device__ static int o_blk(int d) { return (R * ks(d) + 3) & ~3; }                // [2][R][PS] t1
@@ -79,9 +81,9 @@ struct GramCfg {
     __host__ __device__ static int o_dxs(int d) { return o_acc(d) + 2 * FMAX; }                 // [FMAX]
     __host__ __device__ static int o_dys(int d) { return o_dxs(d) + FMAX; }                     // [FMAX]
     __host__ __device__ static int o_sx(int d) { return o_dys(d) + FMAX; }                      // [16][32] staircase buckets per warp
-    __host__ __device__ static int o_sy(int d) { return o_sx(d) + FMAX; }                       
+    __host__ __device__ static int o_sy(int d) { return o_sx(d) + FMAX; }                       // [16][64] points that pass, per warp
     __host__ __device__ static int o_cf(int d) { return o_sy(d) + FMAX; }   // a1[32], a2[32], lam1[32], kap2[32] (f64)
-    __host__ __device__ static int o_rp(int d) { return o_cf(d) + 192; }                        // [8][R]
+    __host__ __device__ static int o_rp(int d) { return o_cf(d) + 192; }                        // [8][R]: rows 4, 5 the rows' ranges of the list
     static size_t smem_bytes(int d) { return (size_t)(o_rp(d) + 8 * R) * 4; }
 };
 

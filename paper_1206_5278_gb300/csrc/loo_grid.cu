@@ -21,12 +21,13 @@
 // A cell whose shifted numerator At falls below 2^(ceil(log2 N) - 91) (the
 // x-nearest and the y-nearest neighbours differ and both factors are small;
 // below it the terms that lost precision to the FP32 range could matter) is
-// recomputed exactly with a joint shift anchored at
-// argmin_i [a1 (dx2-m_x) + a2 (dy2-m_y)].
+// recomputed exactly with a joint shift anchored near
+// min_i [a1 (dx2-m_x) + a2 (dy2-m_y)].
 //
 // Work decomposition: a CTA of 8 warps owns a "unit" of JW = 1024/(G1 G2)
-// rows (G1 padded to 16 or 32, G2 to 8, 16 or 32); the 8 warps split the i
-// range in interleaved chunks of 32 points and their FP32 partial sums are
+// rows (G1 padded to 16 or 32, G2 to 8, 16 or 32; grids of at most 8 x 8: 8 rows,
+// both padded to 4 or 8, loo_pack.cuh); the 8 warps split the i range in
+// interleaved chunks of 64 points and their FP32 partial sums are
 // combined in fixed warp order.  Units are grouped
 // into tiles; each tile's FP64 partial scores go to their own slot and a final
 // kernel sums the slots in tile order, so results are bitwise reproducible and

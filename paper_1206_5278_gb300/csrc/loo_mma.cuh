@@ -1,8 +1,7 @@
 // Tensor-core tile body of the leave-one-out grid kernel.
 //
-// Same sums as the FP32 tile body in loo_common.cuh (At_j(k,l) = sum_i
-// u_i(k) w_i(l), Bt_j(k) = sum_i u_i(k)), with the outer-product accumulation
-// issued as m16n8k8 TF32 tensor-core MMAs whose operands never touch shared
+// The sums At_j(k,l) = sum_i u_i(k) w_i(l), Bt_j(k) = sum_i u_i(k), with the
+// outer-product accumulation issued as m16n8k8 TF32 tensor-core MMAs whose operands never touch shared
 // memory: for row j the GEMM is D[k][l] += sum_i U[k][i] W[i][l] (M = k,
 // N = l, K = i), and every lane produces exactly the fragment elements it
 // owns -- A: (k = 16 mt + g [+8], i = t [+4]), B: (i = t [+4], l = 8 nt + g),
@@ -38,7 +37,7 @@
 // grid: mean per-row error of L_cond -1.8e-7 before, ~0 after.  Each lane takes
 // the points (2t, 2t+1) of a k-step so the TF32 and BF16 fragment layouts hold
 // the same points.  The tensor core's FP32 accumulation is kept short: each
-// chunk of 64 points (128 at 32 x 32: 16 or 32 MMAs per accumulator) starts
+// chunk of 64 points (16 MMAs per accumulator) starts
 // from zero and is then added to an FP32 running total with a rounded add; the
 // running totals live in shared memory.
 #pragma once
