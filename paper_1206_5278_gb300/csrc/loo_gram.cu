@@ -76,11 +76,10 @@ struct GramCfg {
     __host__ __device__ static int o_pos(int d) { return o_flag(d) + kThreads; }                // [512]
     __host__ __device__ static int o_misc(int d) { return o_pos(d) + kThreads; }                // [64]
     __host__ __device__ static int o_list(int d) { return o_misc(d) + 64; }                     // [FMAX]
-    __host__ __device__ static int o_best(int d) { return o_list(d) + FMAX; }                   // [2][FMAX] a1, a2
-    __host__ __device__ static int o_acc(int d) { return o_best(d) + 2 * FMAX; }                // [2][FMAX] sums and their low parts
-    __host__ __device__ static int o_dxs(int d) { return o_acc(d) + 2 * FMAX; }                 // [FMAX]
-    __host__ __device__ static int o_dys(int d) { return o_dxs(d) + FMAX; }                     // [FMAX]
-    __host__ __device__ static int o_sx(int d) { return o_dys(d) + FMAX; }                      // [16][32] staircase buckets per warp
+    __host__ __device__ static int o_best(int d) { return o_list(d) + FMAX; }                   // [FMAX][2] a1, a2
+    __host__ __device__ static int o_acc(int d) { return o_best(d) + 2 * FMAX; }                // [FMAX][2] sums and their low parts
+    __host__ __device__ static int o_dxy(int d) { return o_acc(d) + 2 * FMAX; }                 // [FMAX][2] the anchors' dx2, dy2
+    __host__ __device__ static int o_sx(int d) { return o_dxy(d) + 2 * FMAX; }                      // [16][32] staircase buckets per warp
     __host__ __device__ static int o_sy(int d) { return o_sx(d) + FMAX; }                       // [16][64] points that pass, per warp
     __host__ __device__ static int o_cf(int d) { return o_sy(d) + FMAX; }   // a1[32], a2[32], lam1[32], kap2[32] (f64)
     __host__ __device__ static int o_rp(int d) { return o_cf(d) + 192; }                        // [8][R]: rows 4, 5 the rows' ranges of the list
@@ -393,16 +392,17 @@ struct GramStair {
 };
 
 // The staircase of row rl (this warp's) from its cells' anchors; bk: 32 words of the warp.
-__device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk, const float* As, const float* Bs,
-                                                 const float* dxs, const float* dys, int fb, int fn, float mxv,
+__device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk, const float2* AB,
+                                                 const float2* dxy, int fb, int fn, float mxv,
                                                  float myv, float T) {
     const int lane = threadIdx.x & 31;
     float lo = INFINITY, hi = 0.f;
     const auto extents = [&](int f, float& rx, float& ry) {
         // (the factor covers the rounding of e where it is large next to T)
-        const float e = fmaf(fmaxf(fmaf(As[f], dxs[f] - mxv, Bs[f] * (dys[f] - myv)), 0.f), 1.f + 0x1p-20f, T);
-        rx = __fdividef(e, As[f]);
-        ry = __fdividef(e, Bs[f]);
+        const float2 c = AB[f], q = dxy[f];
+        const float e = fmaf(fmaxf(fmaf(c.x, q.x - mxv, c.y * (q.y - myv)), 0.f), 1.f + 0x1p-20f, T);
+        rx = __fdividef(e, c.x);
+        ry = __fdividef(e, c.y);
     };
     for (int f = fb + lane; f < fb + fn; f += 32) {
         float rx, ry;
@@ -442,9 +442,13 @@ __device__ __forceinline__ void gram_stair_build(GramStair& st, unsigned int* bk
 // distance, then, for up to 32 of them at a time, on the direct one), then the row's cells:
 // each point that passes is broadcast to all lanes, and lane f % 32 updates cell f, which
 // only it owns (no atomics; each cell sees the points in step, chunk and lane order, so the
-// sums are reproducible).  The sums are two floats, added to with compensation: one warp takes
-// all points of a row, and one float is off by 2.7e-4 on 20,000 tied points (51.3 -> 51.6 ms at
-// N = 40,009, d = 32).  A point more than kFbMove below a cell's anchor rescales the sum and
+// sums are reproducible).  The sums are two floats, added to with compensation (exact where the
+// sum is the larger; its first terms are few): one warp takes all points of a row, and one float
+// is off by 2.7e-4 on 20,000 tied points.  Two points at a time for one visit of the cell in
+// shared memory, each pair of its numbers in one 64-bit word; against single points and one
+// float: 32 x 32 at N = 40,009, d = 32 51.3 -> 51.6 ms, at N = 1,066, d = 22 0.374 -> 0.355,
+// 16 x 32 at N = 9,448 2.31 -> 2.27, 8 x 32 at N = 1,652, d = 19 0.345 -> 0.333 (single points
+// and two floats: 51.7, 0.393, 2.33, 0.357).  A point more than kFbMove below a cell's anchor rescales the sum and
 // becomes the anchor; the staircase follows the anchors down.
 template <int G1, int G2, int JW>
 __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_t p0, int buf, float T,
@@ -461,11 +465,9 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
     const float* Ys = sm + C::o_y(d) + buf * C::P;
     const float* rc = sm + C::o_rc(d);
     const float *yr_s = rc, *mxr_s = rc + R, *myr_s = rc + 2 * R, *nr_s = rc + 3 * R;
-    const float* As = sm + C::o_best(d);
-    const float* Bs = As + C::FMAX;
-    float* sum = sm + C::o_acc(d);
-    float* dxs = sm + C::o_dxs(d);
-    float* dys = sm + C::o_dys(d);
+    const float2* AB = reinterpret_cast<const float2*>(sm + C::o_best(d));
+    float2* sum = reinterpret_cast<float2*>(sm + C::o_acc(d));
+    float2* dxy = reinterpret_cast<float2*>(sm + C::o_dxy(d));
     const int* rbn = reinterpret_cast<const int*>(sm + C::o_rp(d) + 4 * R);
     unsigned int* bk = reinterpret_cast<unsigned int*>(sm + C::o_sx(d)) + 32 * warp;
     int* hits = reinterpret_cast<int*>(sm + C::o_sy(d)) + 64 * warp;   // up to 31 waiting and a chunk's 32
@@ -488,30 +490,41 @@ __device__ __forceinline__ void gram_fb_scan(const LooArgs& a, float* sm, int64_
             const bool in = st[r].in(d2 - mxv, dy2 - myv) && lane < cnt;
             unsigned int m = __ballot_sync(0xffffffffu, in);
             bool moved = false;
-            while (m) {
-                const int src = __ffs(m) - 1;
+            while (m) {   // two at a time (the last one's partner is infinitely far)
+                const int sa = __ffs(m) - 1;
                 m &= m - 1;
-                const float d2q = __shfl_sync(0xffffffffu, d2, src), dy2q = __shfl_sync(0xffffffffu, dy2, src);
+                const int sb = m ? __ffs(m) - 1 : 32;
+                m &= m - 1;
+                const float da = __shfl_sync(0xffffffffu, d2, sa), ya = __shfl_sync(0xffffffffu, dy2, sa);
+                const float dbs = __shfl_sync(0xffffffffu, d2, sb & 31), ybs = __shfl_sync(0xffffffffu, dy2, sb & 31);
+                const float db = sb < 32 ? dbs : INFINITY, yb = sb < 32 ? ybs : INFINITY;
                 for (int f = fb + lane; f < fb + fn; f += 32) {
-                    float e = fmaf(As[f], d2q - dxs[f], Bs[f] * (dy2q - dys[f]));
-                    float S = sum[f], Sc = sum[C::FMAX + f];
-                    if (e < -kFbMove) {
-                        const float by = ex2_approx(kFbEx2Fix + e);
+                    const float2 c = AB[f], q = dxy[f];
+                    const auto ex = [&](float x, float y, float X, float Y) { return fmaf(c.x, x - X, c.y * (y - Y)); };
+                    float ea = ex(da, ya, q.x, q.y), eb = ex(db, yb, q.x, q.y);
+                    const float2 sv = sum[f];
+                    float S = sv.x, Sc = sv.y;
+                    const float lo = fminf(ea, eb);
+                    if (lo < -kFbMove) {   // a lower point: the new anchor
+                        const float by = ex2_approx(kFbEx2Fix + lo);
                         S *= by;
                         Sc *= by;
-                        dxs[f] = d2q;
-                        dys[f] = dy2q;
-                        e = 0.f;
+                        const bool first = lo == ea;
+                        const float Xn = first ? da : db, Yn = first ? ya : yb;
+                        ea = ex(da, ya, Xn, Yn);
+                        eb = ex(db, yb, Xn, Yn);
+                        dxy[f] = make_float2(Xn, Yn);
                         moved = true;
                     }
-                    add_two(S, Sc, ex2_approx(kFbEx2Fix - e));
-                    sum[f] = S;
-                    sum[C::FMAX + f] = Sc;
+                    const float v = ex2_approx(kFbEx2Fix - ea) + ex2_approx(kFbEx2Fix - eb), t = __fadd_rn(S, v);
+                    Sc += __fsub_rn(v, __fsub_rn(t, S));
+                    S = t;
+                    sum[f] = make_float2(S, Sc);
                 }
             }
             if (__any_sync(0xffffffffu, moved)) {
                 __syncwarp();
-                gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxv, myv, T);
+                gram_stair_build(st[r], bk, AB, dxy, fb, fn, mxv, myv, T);
             }
         };
         constexpr int W = C::CPS < 4 ? C::CPS : 4;   // chunks tested together (2: 52.8 ms, 4: 51.3)
@@ -685,11 +698,9 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
     const int total = gram_scan(__popc(fw), pos, misc);
     if (KERN == 0 && total > 0) {
         int* list = reinterpret_cast<int*>(sm + C::o_list(d));
-        float* As = sm + C::o_best(d);
-        float* Bs = As + C::FMAX;
-        float* sum = sm + C::o_acc(d);
-        float* dxs = sm + C::o_dxs(d);
-        float* dys = sm + C::o_dys(d);
+        float2* AB = reinterpret_cast<float2*>(sm + C::o_best(d));
+        float2* sum = reinterpret_cast<float2*>(sm + C::o_acc(d));
+        float2* dxy = reinterpret_cast<float2*>(sm + C::o_dxy(d));
         int* rbn = reinterpret_cast<int*>(sm + C::o_rp(d) + 4 * R);
         unsigned int* bk = reinterpret_cast<unsigned int*>(sm + C::o_sx(d)) + 32 * warp;
         int lg = 0;
@@ -715,11 +726,9 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
                 const float A = a1s[kl >> LG2], B = a2s[kl & (G2 - 1)];
                 const float mxv = mxr_s[rl], myv = myr_s[rl], qx = qxr_s[rl], qy = qyr_s[rl];
                 const bool xn = B * (qy - myv) <= A * (qx - mxv);
-                As[f] = A;
-                Bs[f] = B;
-                dxs[f] = xn ? mxv : qx;
-                dys[f] = xn ? qy : myv;
-                sum[f] = sum[C::FMAX + f] = 0.f;
+                AB[f] = make_float2(A, B);
+                dxy[f] = make_float2(xn ? mxv : qx, xn ? qy : myv);
+                sum[f] = make_float2(0.f, 0.f);
             }
             // per row: its range of the list
             for (int rl = tid; rl < R; rl += NTH) {
@@ -739,7 +748,7 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
 #pragma unroll
             for (int r = 0; r < JW; ++r) {
                 const int rl = warp * JW + r, fb = rbn[rl], fn = rbn[R + rl];
-                if (fn > 0) gram_stair_build(st[r], bk, As, Bs, dxs, dys, fb, fn, mxr_s[rl], myr_s[rl], T);
+                if (fn > 0) gram_stair_build(st[r], bk, AB, dxy, fb, fn, mxr_s[rl], myr_s[rl], T);
             }
             gram_block<G1, G2, KERN, false>(a, sm, 0, 0);
             __syncthreads();
@@ -751,9 +760,9 @@ __device__ __forceinline__ void gram_unit(const LooArgs& a, const Coef& cf, int 
             }
             for (int f = tid; f < n; f += NTH) {
                 const int cell = list[f], rl = cell / GG, kl = cell - rl * GG, k = kl >> LG2, l = kl & (G2 - 1);
-                const float tot = sum[f] + sum[C::FMAX + f];
-                const double es = (double)a1s[k] * ((double)dxs[f] - (double)mxr_s[rl]) +
-                                  (double)a2s[l] * ((double)dys[f] - (double)myr_s[rl]);
+                const float tot = sum[f].x + sum[f].y;
+                const double es = (double)a1s[k] * ((double)dxy[f].x - (double)mxr_s[rl]) +
+                                  (double)a2s[l] * ((double)dxy[f].y - (double)myr_s[rl]);
                 fbv[cell] = -es + log2_wide(tot);
             }
             __syncthreads();
